@@ -228,13 +228,13 @@ def _network_inputs(case, seed):
         f = torch.nn.functional.interpolate(f, size=(H, W), mode="bicubic", align_corners=False)[0, 0]
         x = torch.empty(3, H, W, dtype=torch.float32, device=DEV)
         x[0], x[1:] = f, torch.rand(2, 1, 1, generator=g, device=DEV)
-        y = (torch.arange(H, device=DEV) + 1.0)[:, None] / (H + 1)
-        z = (torch.arange(W, device=DEV) + 1.0)[None, :] / (W + 1)
+        y = (torch.arange(H, device=DEV, dtype=torch.float64) + 1.0)[:, None] / (H + 1)
+        z = (torch.arange(W, device=DEV, dtype=torch.float64) + 1.0)[None, :] / (W + 1)
         modes = [torch.sin((1 + j // 4) * math.pi * y) * torch.sin((1 + j % 4) * math.pi * z) for j in range(q)]
-        Q = torch.stack(modes).reshape(q, -1).double() + 1e-3 * _randn(g, q, H * W)
-        Q = torch.linalg.qr(Q.T.contiguous())[0]
+        modes = torch.stack(modes).reshape(q, -1) * (2.0 / math.sqrt((H + 1) * (W + 1)))   # orthonormal
+        R = np.linalg.qr(np.random.RandomState((int(seed) + len(xs)) % 2**31).randn(q, q))[0]
         xs.append(x)
-        qs.append(Q.T.float().contiguous())
+        qs.append((torch.from_numpy(R).to(DEV) @ modes).float().contiguous())
     return xs, qs
 
 
