@@ -154,6 +154,25 @@ int dalloc(T** p, size_t count) {
   return RKS_OK;
 }
 
+// A status word in pinned host memory for calls that synchronise before they
+// return: kernels set it over the bus only when something failed, so a call
+// needs neither an allocation nor a copy back for it.  One word per host
+// thread (a thread has one such call in flight), freed when the thread ends.
+struct ThreadFlag {
+  int* p = nullptr;
+  ~ThreadFlag() {
+    if (p) cudaFreeHost(p);
+  }
+};
+int* thread_flag() {
+  static thread_local ThreadFlag f;
+  if (!f.p && cudaHostAlloc((void**)&f.p, sizeof(int), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+    (void)cudaGetLastError();
+    f.p = nullptr;
+  }
+  return f.p;
+}
+
 int launch_err() {
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
@@ -1840,28 +1859,17 @@ int rks_sketch_apply(int64_t n, int d, int zeta, uint64_t seed, const double* x,
   if (n <= 0 || zeta < 1 || zeta > 16 || d < 2 * zeta || d > 8192 || !x || !z) return RKS_EINVAL;
   cudaStream_t st = (cudaStream_t)stream;
   if (rks::configure_kernels() != cudaSuccess) return RKS_ECUDA;
-  int* flag = nullptr;
-  int rc = dalloc(&flag, 1);
-  if (rc) return rc;
-  cudaMemsetAsync(flag, 0, sizeof(int), st);
-  cudaMemsetAsync(z, 0, d * sizeof(double), st);
-  rks::launch_sketch_vec(n, x, 1.0, d, zeta, seed, z, flag, st);
-  // the kernel sums sign * x_i; the 1/sqrt(zeta) scale is applied here
-  std::vector<double> h(d);
-  int f = 0;
-  cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess) e = cudaMemcpyAsync(h.data(), z, d * sizeof(double), cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&f, flag, sizeof(int), cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  int* flag = thread_flag();
+  if (!flag) return RKS_ENOMEM;
+  *flag = 0;
+  cudaError_t e = cudaMemsetAsync(z, 0, d * sizeof(double), st);
   if (e == cudaSuccess) {
-    const double sc = 1.0 / std::sqrt((double)zeta);
-    for (double& v : h) v *= sc;
-    e = cudaMemcpyAsync(z, h.data(), d * sizeof(double), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    rks::launch_sketch_vec(n, x, 1.0 / std::sqrt((double)zeta), d, zeta, seed, z, flag, st);
+    e = cudaGetLastError();
   }
-  cudaFree(flag);
-  if (e != cudaSuccess) return RKS_ECUDA;
-  return f ? RKS_EINVAL : RKS_OK;
+  const cudaError_t es = cudaStreamSynchronize(st);
+  if (e != cudaSuccess || es != cudaSuccess) return RKS_ECUDA;
+  return *flag ? RKS_EINVAL : RKS_OK;
 }
 
 }  // extern "C"

@@ -176,7 +176,8 @@ void launch_tc_restart_df(int64_t n, const float2* in, float2* out, int64_t ldu,
 
 void launch_sketch_pairs(int64_t n, int d, int zeta, uint64_t seed, int32_t* rows, int8_t* signs, int* flag,
                          cudaStream_t st);
-void launch_sketch_vec(int64_t n, const double* x, double xscale, int d, int zeta, uint64_t seed, double* out_raw,
+// out += scale * sum_i sign * x_i
+void launch_sketch_vec(int64_t n, const double* x, double scale, int d, int zeta, uint64_t seed, double* out,
                        int* flag, cudaStream_t st);
 void launch_spmv_sketch(const Csr& A, const double* x, const double* xscale, double* w, int d, int zeta,
                         uint64_t seed, double* out_raw, int* flag, cudaStream_t st);
