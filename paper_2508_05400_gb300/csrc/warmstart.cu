@@ -14,14 +14,14 @@
 // every run.
 //
 // Kernels:
-//   k_conv3x3       16 x 16 output pixels per CTA, all output channels: the
-//                   input tile with its halo and the layer's weights in
-//                   shared memory, optional ReLU on the output and an
-//                   optional mask (z > 0) on the input (the ReLU derivative
-//                   of the backward pass); the backward-data product is this
-//                   kernel with the flipped, transposed weights.
-//   k_conv3x3_wgrad partial sums of dL/dW and dL/db over a band of tiles
-//                   per CTA, folded in CTA order by k_fold_params.
+//   k_conv3x3       32 x 8 output pixels per CTA, 4 pixels x 8 outputs per
+//                   thread, optional ReLU on the output and an optional mask
+//                   on it (the ReLU derivative of the backward pass); the
+//                   backward-data product is this kernel with the flipped,
+//                   transposed weights.  k_conv3x3_one: the one-channel layer.
+//   k_wgrad32 / k_wgrad3 / k_wgrad_one
+//                   partial sums of dL/dW and dL/db per CTA, folded in a
+//                   fixed order by k_fold_params.
 //   k_pool, k_pool_back, k_up_add, k_up_back: level changes.
 //   k_loss_dots, k_loss_grad: Q^T u and u^T u (FP64 partials), dL/du.
 //   k_adam, k_pack_weights: the optimiser and the FP16 weight layouts.
@@ -45,127 +45,460 @@ constexpr int kConvs = 15;       // C1 .. C15
 constexpr int kTile = 16;        // output tile side
 constexpr int kHalo = kTile + 2;
 constexpr int kHalo2 = kHalo * kHalo;
-constexpr int kWgradTiles = 4;   // tiles per CTA of the weight gradient
 
 int conv_cin(int l) { return l == 0 ? 3 : kCh; }
 int conv_cout(int l) { return l == kConvs - 1 ? 1 : kCh; }
 
-// out[o, y, x] = b[o] + sum_{c, dy, dx} W[o, c, dy, dx] z'[c, y + dy - 1, x + dx - 1],
-// z' = z (or z * (mask > 0)), zero outside the grid; W in layout
-// [c][dy * 3 + dx][o] (FP16); optional ReLU on out.
-template <int COUT>
-__global__ void __launch_bounds__(256) k_conv3x3(const float* __restrict__ z, const float* __restrict__ mask, int cin,
-                                                 int H, int W, const __half* __restrict__ w,
-                                                 const float* __restrict__ bias, int relu, float* __restrict__ out) {
-  extern __shared__ float sm[];
+// Two FP32 FMAs per lane and instruction (IEEE, round to nearest each): the
+// FMA pipe then needs an issue slot only every other cycle, which leaves the
+// others to the shared-memory loads.
+__device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpack2(unsigned long long v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ void cp4_zfill(float* dst, const float* src, bool on) {
+  const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(on ? 4 : 0) : "memory");
+}
+
+// out[o, y, x] = b[o] + sum_{c, dy, dx} W[o, c, dy, dx] z[c, y + dy - 1, x + dx - 1],
+// zero outside the grid, for 32 output channels; W (the FP16 values as FP32)
+// in layout [c][dy * 3 + dx][o]; optional ReLU on out; with omask, out is
+// zero where omask <= 0 (the ReLU derivative of the layer that out is the
+// gradient of).  FP32 FMAs in the order (c, dy, dx) from b.
+//
+// A CTA takes 32 x 8 pixels and four groups of OUTS outputs (grid.z the
+// others), a thread 4 pixels of a row and one group: per channel 18 OUTS
+// two-wide FMAs against 24 shared-memory loads (a group's weights are one
+// broadcast address per warp), where one pixel x 32 outputs per thread needed
+// 9 loads per 32 FMAs and ran at 27% of the FMA rate.  Channels come in
+// stages of 8 with the next stage in flight (cp.async, zero fill at the
+// border).  OUTS = 8 for large grids, 4 where its CTAs would not fill the
+// SMs (half the chain per warp, twice the CTAs).
+// Measured, 512 x 512, 32 -> 32 (2.4 GMAC): 89 us, 74% of the FMA rate (the
+// pixel form 190 us); 8 pixels x 4 outputs per thread with doubled weights
+// 125 us.  256 x 256: 31 us with OUTS = 4 (37 us with 8).
+// On the tensor cores (bf16 splits of z) the sums would be truncated at
+// every accumulation, always towards zero: layer after layer that shrinks
+// the result by more than the rounding errors of these FMAs.
+constexpr int kCvW = 32, kCvH = 8, kCvPitch = 36, kCvStage = 8;
+constexpr int kCvPlane = (kCvH + 2) * kCvPitch;
+
+// One channel's tile with its halo, by one warp: a lane a column, then the
+// last two columns.
+__device__ __forceinline__ void conv_stage_plane(const float* __restrict__ zc, int H, int W, int x0, int y0,
+                                                 int lane, float* dst) {
+  const int gx = x0 - 1 + lane;
+  const bool okx = gx >= 0 && gx < W;
+#pragma unroll
+  for (int r = 0; r < kCvH + 2; ++r) {
+    const int gy = y0 - 1 + r;
+    const bool on = okx && gy >= 0 && gy < H;
+    cp4_zfill(dst + r * kCvPitch + lane, on ? zc + (size_t)gy * W + gx : zc, on);
+  }
+  if (lane < 2 * (kCvH + 2)) {
+    const int r = lane >> 1, hx = x0 + 31 + (lane & 1), gy = y0 - 1 + r;
+    const bool on = hx < W && gy >= 0 && gy < H;
+    cp4_zfill(dst + r * kCvPitch + 32 + (lane & 1), on ? zc + (size_t)gy * W + hx : zc, on);
+  }
+}
+
+template <int OUTS>
+__global__ void __launch_bounds__(256) k_conv3x3(const float* __restrict__ z, int cin, int H, int W,
+                                                 const float* __restrict__ w, const float* __restrict__ bias,
+                                                 int relu, const float* __restrict__ omask,
+                                                 float* __restrict__ out) {
+  extern __shared__ __align__(16) float sm[];
+  constexpr int OP = OUTS / 2;                  // output pairs
+  float* zs = sm;                               // two stages of kCvStage planes
+  float* ws = sm + 2 * kCvStage * kCvPlane;     // (cin * 9) x 4 groups x OUTS
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int og = tid >> 6, xg = tid & 7, ty = (tid >> 3) & 7;
+  const int x0 = blockIdx.x * kCvW, y0 = blockIdx.y * kCvH;
+  const int o0 = (blockIdx.z * 4 + og) * OUTS;
+  const size_t hw = (size_t)H * W;
+  auto stage = [&](int c0, float* dst) {        // a warp a channel
+    if (c0 + warp < cin) conv_stage_plane(z + (c0 + warp) * hw, H, W, x0, y0, lane, dst + warp * kCvPlane);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  for (int i = tid; i < cin * 9 * OUTS; i += 256) {       // 16 bytes each
+    const int r = i / OUTS, q = i % OUTS;
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                     static_cast<uint32_t>(__cvta_generic_to_shared(ws + 4 * i))),
+                 "l"(w + r * 32 + blockIdx.z * 4 * OUTS + 4 * q)
+                 : "memory");
+  }
+  stage(0, zs);
+  unsigned long long acc[4][OP];                // pixel, output pair
+#pragma unroll
+  for (int q = 0; q < OP; ++q) {
+    const unsigned long long b = bias ? pack2(bias[o0 + 2 * q], bias[o0 + 2 * q + 1]) : 0ull;
+#pragma unroll
+    for (int p = 0; p < 4; ++p) acc[p][q] = b;
+  }
+  int buf = 0;
+  for (int c0 = 0; c0 < cin; c0 += kCvStage, buf ^= 1) {
+    const bool more = c0 + kCvStage < cin;
+    if (more) stage(c0 + kCvStage, zs + (buf ^ 1) * kCvStage * kCvPlane);
+    if (more) asm volatile("cp.async.wait_group 1;" ::: "memory");
+    else asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    const int nc = min(kCvStage, cin - c0);
+    const float* zc = zs + buf * kCvStage * kCvPlane + ty * kCvPitch + xg * 4;
+    const float* wc = ws + c0 * 36 * OUTS + og * OUTS;
+    for (int c = 0; c < nc; ++c, zc += kCvPlane, wc += 36 * OUTS) {
+#pragma unroll
+      for (int dy = 0; dy < 3; ++dy) {
+        const float4 a = *reinterpret_cast<const float4*>(zc + dy * kCvPitch);
+        const float2 b = *reinterpret_cast<const float2*>(zc + dy * kCvPitch + 4);
+        const unsigned long long v[6] = {pack2(a.x, a.x), pack2(a.y, a.y), pack2(a.z, a.z),
+                                         pack2(a.w, a.w), pack2(b.x, b.x), pack2(b.y, b.y)};
+#pragma unroll
+        for (int dx = 0; dx < 3; ++dx) {
+#pragma unroll
+          for (int h = 0; h < OP / 2; ++h) {
+            const ulonglong2 wk = *reinterpret_cast<const ulonglong2*>(wc + (dy * 3 + dx) * 4 * OUTS + 4 * h);
+#pragma unroll
+            for (int p = 0; p < 4; ++p) {
+              acc[p][2 * h] = fma2(wk.x, v[p + dx], acc[p][2 * h]);
+              acc[p][2 * h + 1] = fma2(wk.y, v[p + dx], acc[p][2 * h + 1]);
+            }
+          }
+        }
+      }
+    }
+    __syncthreads();                            // the stage is free for the load after next
+  }
+  const int yy = y0 + ty, xx = x0 + xg * 4;
+  if (yy >= H || xx >= W) return;
+  const bool vec = (W & 3) == 0;                // then the row's four pixels exist and are aligned
+#pragma unroll
+  for (int o = 0; o < OUTS; ++o) {
+    float r[4];
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+      float lo, hi;
+      unpack2(acc[p][o >> 1], lo, hi);
+      r[p] = o & 1 ? hi : lo;
+      if (relu) r[p] = fmaxf(r[p], 0.f);
+    }
+    const size_t at = ((size_t)(o0 + o) * H + yy) * W + xx;
+    if (vec) {
+      if (omask) {
+        const float4 m = *reinterpret_cast<const float4*>(omask + at);
+        r[0] = m.x > 0.f ? r[0] : 0.f;
+        r[1] = m.y > 0.f ? r[1] : 0.f;
+        r[2] = m.z > 0.f ? r[2] : 0.f;
+        r[3] = m.w > 0.f ? r[3] : 0.f;
+      }
+      *reinterpret_cast<float4*>(out + at) = make_float4(r[0], r[1], r[2], r[3]);
+    } else {
+#pragma unroll
+      for (int p = 0; p < 4; ++p)
+        if (xx + p < W) out[at + p] = omask && !(omask[at + p] > 0.f) ? 0.f : r[p];
+    }
+  }
+}
+
+// One output channel (the network's last layer): 16 x 16 pixels per CTA, a
+// thread a pixel, all cin channels staged.
+__global__ void __launch_bounds__(256) k_conv3x3_one(const float* __restrict__ z, int cin, int H, int W,
+                                                     const float* __restrict__ w, const float* __restrict__ bias,
+                                                     float* __restrict__ out) {
+  extern __shared__ __align__(16) float sm[];
   float* zs = sm;                          // cin x 18 x 18
-  float* ws = sm + cin * kHalo2;           // cin x 9 x COUT
+  float* ws = sm + cin * kHalo2;           // cin x 9
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const int x0 = blockIdx.x * kTile, y0 = blockIdx.y * kTile;
-  for (int i = tid; i < cin * 9 * COUT; i += 256) ws[i] = __half2float(w[i]);
+  for (int i = tid; i < cin * 9; i += 256) ws[i] = w[i];
   for (int i = tid; i < cin * kHalo2; i += 256) {
     const int c = i / kHalo2, r = i - c * kHalo2;
     const int yy = y0 - 1 + r / kHalo, xx = x0 - 1 + r % kHalo;
-    float v = 0.f;
-    if (yy >= 0 && yy < H && xx >= 0 && xx < W) {
-      const size_t at = ((size_t)c * H + yy) * W + xx;
-      v = z[at];
-      if (mask && !(mask[at] > 0.f)) v = 0.f;
-    }
-    zs[i] = v;
+    const bool on = yy >= 0 && yy < H && xx >= 0 && xx < W;
+    cp4_zfill(zs + i, on ? z + ((size_t)c * H + yy) * W + xx : z, on);
   }
+  asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
   __syncthreads();
-  float acc[COUT];
-#pragma unroll
-  for (int o = 0; o < COUT; ++o) acc[o] = bias ? bias[o] : 0.f;
+  float acc = bias[0];
   for (int c = 0; c < cin; ++c) {
     const float* zc = zs + c * kHalo2 + ty * kHalo + tx;
 #pragma unroll
-    for (int k = 0; k < 9; ++k) {
-      const float v = zc[(k / 3) * kHalo + (k % 3)];
-      const float* wk = ws + (c * 9 + k) * COUT;
-#pragma unroll
-      for (int o = 0; o < COUT; ++o) acc[o] = fmaf(wk[o], v, acc[o]);
-    }
+    for (int k = 0; k < 9; ++k) acc = fmaf(ws[c * 9 + k], zc[(k / 3) * kHalo + (k % 3)], acc);
   }
   const int yy = y0 + ty, xx = x0 + tx;
-  if (yy < H && xx < W) {
-#pragma unroll
-    for (int o = 0; o < COUT; ++o) out[((size_t)o * H + yy) * W + xx] = relu ? fmaxf(acc[o], 0.f) : acc[o];
-  }
+  if (yy < H && xx < W) out[(size_t)yy * W + xx] = acc;
 }
 
-// Per-CTA partial sums of dL/dW[o, c, k] = sum_p g'[o, p] z[c, p + k] and
-// dL/db[o] = sum_p g'[o, p] over kWgradTiles tiles (g' = g or g * (gmask > 0)).
-// Thread t < cin * 9 owns (c, k) for all o; the next COUT threads own the
-// biases.  part[blockIdx.x * (cin * 9 * COUT + COUT) + ...] in the parameter
-// layout (o, c, k) then b.
+// Weight gradients: per-CTA partial sums of dL/dW[o, c, k] = sum_p g[o, p]
+// z[c, p + k] and dL/db[o] = sum_p g[o, p] over every gridDim.x-th tile of
+// 16 x 8 pixels; part[blockIdx.x * (cin * 9 * COUT + COUT) + ...] in the
+// parameter layout (o, c, k) then b, folded by k_fold_params.
+//
+// A warp takes one group of 8 outputs and half of a tile's rows, a lane one
+// input channel (cin = 32): the nine taps x 8 outputs are 72 sums in
+// registers, fed per pixel by one new column of the 3 x 3 window (3 loads)
+// and the pixel's 8 gradients (2 broadcast loads), where a thread per
+// (channel, tap) with 32 outputs needed 9 loads per 32 FMAs and left most of
+// the warps idle.  cin = 3 uses 27 lanes, one per (channel, tap); COUT = 1
+// has one group, every warp a row.  The next tile is in flight (cp.async)
+// while one is used.  512 x 512, 32 -> 32: 121 us, was 590 us.
+constexpr int kWgW = 16, kWgH = 8, kWgPx = kWgW * kWgH;
+constexpr int kWgZw = kWgW + 2, kWgZ = kWgZw * (kWgH + 2) + 1;   // channel stride 181: odd, no bank conflicts
+constexpr int kWgG = 36;                                          // gradients of a pixel: stride 36 words
+constexpr int kWgCtas = 152 * 2;
+
+// Tile (x0, y0) into shared memory, asynchronously (one commit group): the
+// cin input planes with their halo, a warp a channel, and the gradients
+// transposed to [pixel][output].
 template <int COUT>
-__global__ void __launch_bounds__(320) k_conv3x3_wgrad(const float* __restrict__ z, int cin, int H, int W,
-                                                       const float* __restrict__ g, const float* __restrict__ gmask,
-                                                       float* __restrict__ part) {
-  extern __shared__ float sm[];
-  float* zs = sm;                          // cin x 18 x 18
-  float* gs = sm + cin * kHalo2;           // 256 pixels x COUT
-  const int tid = threadIdx.x, nt = blockDim.x;
-  const int tiles_x = (W + kTile - 1) / kTile, tiles_y = (H + kTile - 1) / kTile;
-  const int ntiles = tiles_x * tiles_y;
-  const int nk = cin * 9;
-  float acc[COUT];
+__device__ __forceinline__ void wgrad_stage(const float* __restrict__ z, int cin, int H, int W,
+                                            const float* __restrict__ g, int x0, int y0, float* zs, float* gs) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const size_t hw = (size_t)H * W;
 #pragma unroll
-  for (int o = 0; o < COUT; ++o) acc[o] = 0.f;
-  for (int it = 0; it < kWgradTiles; ++it) {
-    const int t = blockIdx.x * kWgradTiles + it;
-    if (t >= ntiles) break;
-    const int x0 = (t % tiles_x) * kTile, y0 = (t / tiles_x) * kTile;
-    __syncthreads();
-    for (int i = tid; i < cin * kHalo2; i += nt) {
-      const int c = i / kHalo2, r = i - c * kHalo2;
-      const int yy = y0 - 1 + r / kHalo, xx = x0 - 1 + r % kHalo;
-      zs[i] = (yy >= 0 && yy < H && xx >= 0 && xx < W) ? z[((size_t)c * H + yy) * W + xx] : 0.f;
-    }
-    for (int i = tid; i < 256 * COUT; i += nt) {
-      const int o = i / 256, p = i - o * 256;
-      const int yy = y0 + (p >> 4), xx = x0 + (p & 15);
-      float v = 0.f;
-      if (yy < H && xx < W) {
-        const size_t at = ((size_t)o * H + yy) * W + xx;
-        v = g[at];
-        if (gmask && !(gmask[at] > 0.f)) v = 0.f;
-      }
-      gs[p * COUT + o] = v;
-    }
-    __syncthreads();
-    if (tid < nk) {
-      const int c = tid / 9, k = tid - c * 9;
-      const float* zc = zs + c * kHalo2 + (k / 3) * kHalo + (k % 3);
-      for (int p = 0; p < 256; ++p) {
-        const float v = zc[(p >> 4) * kHalo + (p & 15)];
-        const float* gp = gs + p * COUT;
-#pragma unroll
-        for (int o = 0; o < COUT; ++o) acc[o] = fmaf(gp[o], v, acc[o]);
-      }
-    } else if (tid < nk + COUT) {
-      const int o = tid - nk;
-      for (int p = 0; p < 256; ++p) acc[0] += gs[p * COUT + o];
+  for (int i = 0; i < (kWgZ - 1 + 31) / 32; ++i) {
+    const int pos = lane + 32 * i, yy = pos / kWgZw, xx = pos % kWgZw;
+    if (pos < kWgZ - 1) {
+      const int gy = y0 - 1 + yy, gx = x0 - 1 + xx;
+      const bool on = gy >= 0 && gy < H && gx >= 0 && gx < W;
+      const float* src = on ? z + (size_t)gy * W + gx : z;
+      for (int c = warp; c < cin; c += 8) cp4_zfill(zs + c * kWgZ + pos, on ? src + c * hw : z, on);
     }
   }
-  float* pp = part + (size_t)blockIdx.x * (nk * COUT + COUT);
-  if (tid < nk) {
-    const int c = tid / 9, k = tid - c * 9;
+  const int p = threadIdx.x & (kWgPx - 1), yy = y0 + p / kWgW, xx = x0 + p % kWgW;
+  const bool on = yy < H && xx < W;
+  const float* gp = on ? g + (size_t)yy * W + xx : g;
+  if (COUT == 1) {
+    if (threadIdx.x < kWgPx) cp4_zfill(gs + p, gp, on);
+  } else {
+#pragma unroll 4
+    for (int o = threadIdx.x / kWgPx; o < COUT; o += 256 / kWgPx) cp4_zfill(gs + p * kWgG + o, on ? gp + o * hw : g, on);
+  }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+__global__ void __launch_bounds__(256, 2) k_wgrad32(const float* __restrict__ z, int H, int W,
+                                                    const float* __restrict__ g, float* __restrict__ part) {
+  extern __shared__ __align__(16) float sm[];
+  constexpr int kBuf = kWgPx * kWgG + 32 * kWgZ + 0;   // gradients, then the planes; two buffers
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, og = warp & 3, ph = warp >> 2;
+  const int tiles_x = (W + kWgW - 1) / kWgW, ntiles = tiles_x * ((H + kWgH - 1) / kWgH);
+  unsigned long long acc[9][4];
 #pragma unroll
-    for (int o = 0; o < COUT; ++o) pp[(o * cin + c) * 9 + k] = acc[o];
-  } else if (tid < nk + COUT) {
-    pp[nk * COUT + (tid - nk)] = acc[0];
+  for (int k = 0; k < 9; ++k)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc[k][q] = 0ull;
+  float db = 0.f;                          // output warp * 4 + lane % 4, pixels lane / 4 + 8 i
+  int buf = 0;
+  wgrad_stage<32>(z, 32, H, W, g, (blockIdx.x % tiles_x) * kWgW, (blockIdx.x / tiles_x) * kWgH, sm + kWgPx * kWgG, sm);
+  for (int t = blockIdx.x; t < ntiles; t += gridDim.x, buf ^= 1) {
+    const int nt = t + gridDim.x;
+    if (nt < ntiles) {
+      float* nb = sm + (buf ^ 1) * kBuf;
+      wgrad_stage<32>(z, 32, H, W, g, (nt % tiles_x) * kWgW, (nt / tiles_x) * kWgH, nb + kWgPx * kWgG, nb);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
+    __syncthreads();
+    const float *gs = sm + buf * kBuf, *zs = gs + kWgPx * kWgG;
+#pragma unroll
+    for (int i = 0; i < kWgPx / 8; ++i) db += gs[(lane / 4 + 8 * i) * kWgG + warp * 4 + (lane & 3)];
+    for (int y = ph * (kWgH / 2); y < (ph + 1) * (kWgH / 2); ++y) {
+      const float* zr = zs + lane * kWgZ + y * kWgZw;
+      const float* gr = gs + y * kWgW * kWgG + og * 8;
+      unsigned long long v[3][3];          // window: column, row
+#pragma unroll
+      for (int c = 0; c < 2; ++c)
+#pragma unroll
+        for (int r = 0; r < 3; ++r) { const float u = zr[r * kWgZw + c]; v[c][r] = pack2(u, u); }
+#pragma unroll
+      for (int x = 0; x < kWgW; ++x) {
+#pragma unroll
+        for (int r = 0; r < 3; ++r) { const float u = zr[r * kWgZw + x + 2]; v[(x + 2) % 3][r] = pack2(u, u); }
+        const ulonglong2 g0 = *reinterpret_cast<const ulonglong2*>(gr + x * kWgG);
+        const ulonglong2 g1 = *reinterpret_cast<const ulonglong2*>(gr + x * kWgG + 4);
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+          const unsigned long long vk = v[(x + k % 3) % 3][k / 3];
+          acc[k][0] = fma2(g0.x, vk, acc[k][0]);
+          acc[k][1] = fma2(g0.y, vk, acc[k][1]);
+          acc[k][2] = fma2(g1.x, vk, acc[k][2]);
+          acc[k][3] = fma2(g1.y, vk, acc[k][3]);
+        }
+      }
+    }
+    __syncthreads();                     // the buffer is free for the tile after next
+  }
+  // the two row halves of a group, then to global memory
+  __syncthreads();
+  float* red = sm;                         // 4 groups x 72 x 32 lanes
+  if (ph == 1) {
+#pragma unroll
+    for (int k = 0; k < 9; ++k)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        float lo, hi;
+        unpack2(acc[k][q], lo, hi);
+        red[(og * 72 + k * 8 + 2 * q) * 32 + lane] = lo;
+        red[(og * 72 + k * 8 + 2 * q + 1) * 32 + lane] = hi;
+      }
+  }
+  for (int o = 4; o < 32; o <<= 1) db += __shfl_xor_sync(0xffffffffu, db, o);
+  __syncthreads();
+  float* pp = part + (size_t)blockIdx.x * (32 * 9 * 32 + 32);
+  if (ph == 0) {
+#pragma unroll
+    for (int k = 0; k < 9; ++k)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        float lo, hi;
+        unpack2(acc[k][q], lo, hi);
+        pp[((og * 8 + 2 * q) * 32 + lane) * 9 + k] = lo + red[(og * 72 + k * 8 + 2 * q) * 32 + lane];
+        pp[((og * 8 + 2 * q + 1) * 32 + lane) * 9 + k] = hi + red[(og * 72 + k * 8 + 2 * q + 1) * 32 + lane];
+      }
+  }
+  if (lane < 4) pp[32 * 9 * 32 + warp * 4 + lane] = db;
+}
+
+// cin = 3, 32 outputs: lane = channel * 9 + tap (27 of 32), 8 outputs per warp
+__global__ void __launch_bounds__(256) k_wgrad3(const float* __restrict__ z, int H, int W,
+                                                const float* __restrict__ g, float* __restrict__ part) {
+  extern __shared__ __align__(16) float sm[];
+  constexpr int kBuf = kWgPx * kWgG + 3 * kWgZ + 1;   // gradients, then the planes; two buffers
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, og = warp & 3, ph = warp >> 2;
+  const int tiles_x = (W + kWgW - 1) / kWgW, ntiles = tiles_x * ((H + kWgH - 1) / kWgH);
+  const int lk = min(lane, 26), c = lk / 9, k = lk % 9;
+  unsigned long long acc[4] = {0ull, 0ull, 0ull, 0ull};
+  float db = 0.f;
+  int buf = 0;
+  wgrad_stage<32>(z, 3, H, W, g, (blockIdx.x % tiles_x) * kWgW, (blockIdx.x / tiles_x) * kWgH, sm + kWgPx * kWgG, sm);
+  for (int t = blockIdx.x; t < ntiles; t += gridDim.x, buf ^= 1) {
+    const int nt = t + gridDim.x;
+    if (nt < ntiles) {
+      float* nb = sm + (buf ^ 1) * kBuf;
+      wgrad_stage<32>(z, 3, H, W, g, (nt % tiles_x) * kWgW, (nt / tiles_x) * kWgH, nb + kWgPx * kWgG, nb);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
+    __syncthreads();
+    const float *gs = sm + buf * kBuf, *zs = gs + kWgPx * kWgG;
+#pragma unroll
+    for (int i = 0; i < kWgPx / 8; ++i) db += gs[(lane / 4 + 8 * i) * kWgG + warp * 4 + (lane & 3)];
+    const float* zr = zs + c * kWgZ + (k / 3) * kWgZw + k % 3;
+    for (int y = ph * (kWgH / 2); y < (ph + 1) * (kWgH / 2); ++y) {
+#pragma unroll
+      for (int x = 0; x < kWgW; ++x) {
+        const float u = zr[y * kWgZw + x];
+        const unsigned long long v = pack2(u, u);
+        const ulonglong2 g0 = *reinterpret_cast<const ulonglong2*>(gs + (y * kWgW + x) * kWgG + og * 8);
+        const ulonglong2 g1 = *reinterpret_cast<const ulonglong2*>(gs + (y * kWgW + x) * kWgG + og * 8 + 4);
+        acc[0] = fma2(g0.x, v, acc[0]);
+        acc[1] = fma2(g0.y, v, acc[1]);
+        acc[2] = fma2(g1.x, v, acc[2]);
+        acc[3] = fma2(g1.y, v, acc[3]);
+      }
+    }
+    __syncthreads();                     // the buffer is free for the tile after next
+  }
+  __syncthreads();
+  unsigned long long* red = reinterpret_cast<unsigned long long*>(sm);   // 4 groups x 4 x 32 lanes
+  if (ph == 1)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) red[(og * 4 + q) * 32 + lane] = acc[q];
+  for (int o = 4; o < 32; o <<= 1) db += __shfl_xor_sync(0xffffffffu, db, o);
+  __syncthreads();
+  float* pp = part + (size_t)blockIdx.x * (3 * 9 * 32 + 32);
+  if (ph == 0 && lane < 27) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      float a, b, a1, b1;
+      unpack2(acc[q], a, b);
+      unpack2(red[(og * 4 + q) * 32 + lane], a1, b1);
+      pp[((og * 8 + 2 * q) * 3 + c) * 9 + k] = a + a1;
+      pp[((og * 8 + 2 * q + 1) * 3 + c) * 9 + k] = b + b1;
+    }
+  }
+  if (lane < 4) pp[3 * 9 * 32 + warp * 4 + lane] = db;
+}
+
+// one output: lane = input channel (32), a warp per tile row
+__global__ void __launch_bounds__(256) k_wgrad_one(const float* __restrict__ z, int H, int W,
+                                                   const float* __restrict__ g, float* __restrict__ part) {
+  extern __shared__ __align__(16) float sm[];
+  constexpr int kBuf = kWgPx + 32 * kWgZ + 0;   // gradients, then the planes; two buffers
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tiles_x = (W + kWgW - 1) / kWgW, ntiles = tiles_x * ((H + kWgH - 1) / kWgH);
+  float acc[9], db = 0.f;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) acc[k] = 0.f;
+  int buf = 0;
+  wgrad_stage<1>(z, 32, H, W, g, (blockIdx.x % tiles_x) * kWgW, (blockIdx.x / tiles_x) * kWgH, sm + kWgPx, sm);
+  for (int t = blockIdx.x; t < ntiles; t += gridDim.x, buf ^= 1) {
+    const int nt = t + gridDim.x;
+    if (nt < ntiles) {
+      float* nb = sm + (buf ^ 1) * kBuf;
+      wgrad_stage<1>(z, 32, H, W, g, (nt % tiles_x) * kWgW, (nt / tiles_x) * kWgH, nb + kWgPx, nb);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
+    __syncthreads();
+    const float *gs = sm + buf * kBuf, *zs = gs + kWgPx;
+    const float* zr = zs + lane * kWgZ + warp * kWgZw;
+#pragma unroll
+    for (int x = 0; x < kWgW; ++x) {
+      const float gv = gs[warp * kWgW + x];
+      db += gv;
+#pragma unroll
+      for (int k = 0; k < 9; ++k) acc[k] = fmaf(gv, zr[(k / 3) * kWgZw + x + k % 3], acc[k]);
+    }
+    __syncthreads();                     // the buffer is free for the tile after next
+  }
+  __syncthreads();
+  float* red = sm;                         // 8 warps x 10 x 32 lanes
+#pragma unroll
+  for (int k = 0; k < 9; ++k) red[(warp * 10 + k) * 32 + lane] = acc[k];
+  red[(warp * 10 + 9) * 32 + lane] = db;
+  __syncthreads();
+  float* pp = part + (size_t)blockIdx.x * (32 * 9 + 1);
+  for (int i = tid; i < 289; i += 256) {
+    const int k = i < 288 ? i % 9 : 9, c = i < 288 ? i / 9 : 0;
+    float s = 0.f;
+    for (int w = 0; w < 8; ++w) s += red[(w * 10 + k) * 32 + c];
+    pp[i] = s;
   }
 }
 
-// grad[i] += sum_b part[b * cnt + i], b in order
-__global__ void k_fold_params(const float* __restrict__ part, int nb, int cnt, float* __restrict__ grad) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += gridDim.x * blockDim.x) {
-    float s = 0.f;
-    for (int b = 0; b < nb; ++b) s += part[(size_t)b * cnt + i];
-    grad[i] += s;
+// grad[i] += sum_b part[b * cnt + i]: 16 strands b = s, s + 16, ... in
+// order, then the strands in order (one strand of up to 304 dependent adds
+// took 14 us a layer)
+constexpr int kFoldStrands = 16;
+__global__ void __launch_bounds__(32 * kFoldStrands) k_fold_params(const float* __restrict__ part, int nb, int cnt,
+                                                                   float* __restrict__ grad) {
+  __shared__ float red[kFoldStrands][32];
+  const int lane = threadIdx.x & 31, s = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
+  float v = 0.f;
+  if (i < cnt) {
+#pragma unroll 10
+    for (int b = s; b < nb; b += kFoldStrands) v += part[(size_t)b * cnt + i];
+  }
+  red[s][lane] = v;
+  __syncthreads();
+  if (s == 0 && i < cnt) {
+#pragma unroll
+    for (int q = 1; q < kFoldStrands; ++q) v += red[q][lane];
+    grad[i] += v;
   }
 }
 
@@ -180,12 +513,14 @@ __global__ void k_pool(const float* __restrict__ z, int C, int H, int W, float* 
   }
 }
 
-// gz[c, y, x] += g[c, y / 2, x / 2] / 4 (gz at H x W)
-__global__ void k_pool_back(const float* __restrict__ g, int C, int H, int W, float* __restrict__ gz) {
+// gz[c, y, x] = (gz[c, y, x] + g[c, y / 2, x / 2] / 4) (mask > 0) (gz at H x W)
+__global__ void k_pool_back(const float* __restrict__ g, int C, int H, int W, const float* __restrict__ mask,
+                            float* __restrict__ gz) {
   const int64_t cnt = (int64_t)C * H * W;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < cnt; t += (int64_t)gridDim.x * blockDim.x) {
     const int x = (int)(t % W), y = (int)((t / W) % H), c = (int)(t / ((int64_t)W * H));
-    gz[t] += 0.25f * g[((size_t)c * (H / 2) + y / 2) * (W / 2) + x / 2];
+    const float v = gz[t] + 0.25f * g[((size_t)c * (H / 2) + y / 2) * (W / 2) + x / 2];
+    gz[t] = mask[t] > 0.f ? v : 0.f;
   }
 }
 
@@ -199,14 +534,15 @@ __global__ void k_up_add(const float* __restrict__ z, const float* __restrict__ 
   }
 }
 
-// gz[c, i, j] = sum of the 2 x 2 block of g (gz at H/2 x W/2)
-__global__ void k_up_back(const float* __restrict__ g, int C, int H, int W, float* __restrict__ gz) {
+// gz[c, i, j] = sum of the 2 x 2 block of g, where mask > 0 (gz and mask at H/2 x W/2)
+__global__ void k_up_back(const float* __restrict__ g, int C, int H, int W, const float* __restrict__ mask,
+                          float* __restrict__ gz) {
   const int h = H / 2, w = W / 2;
   const int64_t cnt = (int64_t)C * h * w;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < cnt; t += (int64_t)gridDim.x * blockDim.x) {
     const int j = (int)(t % w), i = (int)((t / w) % h), c = (int)(t / ((int64_t)w * h));
     const float* gg = g + ((size_t)c * H + 2 * i) * W + 2 * j;
-    gz[t] = (gg[0] + gg[1]) + (gg[W] + gg[W + 1]);
+    gz[t] = mask[t] > 0.f ? (gg[0] + gg[1]) + (gg[W] + gg[W + 1]) : 0.f;
   }
 }
 
@@ -264,14 +600,15 @@ __global__ void k_adam(int64_t cnt, float* __restrict__ theta, float* __restrict
   }
 }
 
-// FP16 layouts of W (master layout (o, c, k)): forward [c][k][o] and, for the
-// backward-data product, the flipped transpose [o][8 - k][c]
-__global__ void k_pack_weights(const float* __restrict__ Wm, int cin, int cout, __half* __restrict__ wf,
-                               __half* __restrict__ wb) {
+// The FP16-rounded weights in FP32 as the convolutions read them (master
+// layout (o, c, k)): forward [c][k][o] and, for the backward-data product, the
+// flipped transpose [o][8 - k][c]
+__global__ void k_pack_weights(const float* __restrict__ Wm, int cin, int cout, float* __restrict__ wf,
+                               float* __restrict__ wb) {
   const int cnt = cin * cout * 9;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += gridDim.x * blockDim.x) {
     const int k = i % 9, c = (i / 9) % cin, o = i / (9 * cin);
-    const __half h = __float2half_rn(Wm[i]);
+    const float h = __half2float(__float2half_rn(Wm[i]));
     wf[(c * 9 + k) * cout + o] = h;
     if (wb) wb[(o * 9 + (8 - k)) * cin + c] = h;
   }
@@ -323,8 +660,8 @@ struct rks_ws {
   float* m = nullptr;
   float* v = nullptr;
   float* gacc = nullptr;                // gradient accumulated over the minibatch
-  __half* wf[kConvs] = {};              // forward layouts
-  __half* wb[kConvs] = {};              // backward-data layouts
+  float* wf[kConvs] = {};               // forward layouts (FP16-rounded values)
+  float* wb[kConvs] = {};               // backward-data layouts (none for C1)
   float* part = nullptr;                // weight-gradient partials
   int64_t part_cap = 0;
   double* lpart = nullptr;              // loss partials
@@ -348,10 +685,11 @@ namespace {
 
 cudaError_t configure_ws_kernels_once() {
   const int big = 200 * 1024;
-  cudaError_t e = cudaFuncSetAttribute(k_conv3x3<kCh>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_conv3x3<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_conv3x3_wgrad<kCh>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_conv3x3_wgrad<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+  cudaError_t e = cudaFuncSetAttribute(k_conv3x3<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_conv3x3<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_conv3x3_one, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_wgrad32, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_wgrad_one, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
   return e;
 }
 
@@ -360,31 +698,40 @@ int grid1(int64_t cnt) { return (int)std::max<int64_t>(1, std::min<int64_t>((cnt
 int lvH(const rks_ws* s, int l) { return s->H >> l; }
 int lvW(const rks_ws* s, int l) { return s->W >> l; }
 
-// out = C_l(z) at level lv; mask: input multiplied by (mask > 0); back: use
-// the backward-data weights (no bias)
-void conv(rks_ws* s, int l, int lv, const float* z, const float* mask, bool back, int relu, float* out) {
+// Tiles (32 x 8 pixels) from which a CTA takes all 32 outputs: four per SM
+constexpr int kCvWideFrom = 608;
+
+// out = C_l(z) at level lv; back: with the backward-data weights (no bias),
+// omask: out is zeroed where omask <= 0
+void conv(rks_ws* s, int l, int lv, const float* z, bool back, int relu, const float* omask, float* out) {
   const int H = lvH(s, lv), W = lvW(s, lv);
   const int cin = back ? conv_cout(l) : conv_cin(l), cout = back ? conv_cin(l) : conv_cout(l);
-  const size_t sm = (size_t)(cin * kHalo2 + cin * 9 * cout) * sizeof(float);
-  dim3 grid((W + kTile - 1) / kTile, (H + kTile - 1) / kTile);
   const float* bias = back ? nullptr : s->theta + s->poff[2 * l + 1];
-  const __half* w = back ? s->wb[l] : s->wf[l];
-  if (cout == 1) k_conv3x3<1><<<grid, 256, sm, s->st>>>(z, mask, cin, H, W, w, bias, relu, out);
-  else k_conv3x3<kCh><<<grid, 256, sm, s->st>>>(z, mask, cin, H, W, w, bias, relu, out);
+  const float* w = back ? s->wb[l] : s->wf[l];
+  if (cout == 1) {
+    dim3 grid((W + kTile - 1) / kTile, (H + kTile - 1) / kTile);
+    k_conv3x3_one<<<grid, 256, (size_t)(cin * kHalo2 + cin * 9) * sizeof(float), s->st>>>(z, cin, H, W, w, bias, out);
+    return;
+  }
+  dim3 grid((W + kCvW - 1) / kCvW, (H + kCvH - 1) / kCvH);
+  const bool wide = (int64_t)grid.x * grid.y >= kCvWideFrom;
+  grid.z = wide ? 1 : 2;
+  const size_t sm = (size_t)(2 * kCvStage * kCvPlane + cin * 36 * (wide ? 8 : 4)) * sizeof(float);
+  if (wide) k_conv3x3<8><<<grid, 256, sm, s->st>>>(z, cin, H, W, w, bias, relu, omask, out);
+  else k_conv3x3<4><<<grid, 256, sm, s->st>>>(z, cin, H, W, w, bias, relu, omask, out);
 }
 
-// gacc[W_l, b_l] += dL/d(W_l, b_l) for the input z of C_l and dL/d(out) = g (* (gmask > 0))
-void wgrad(rks_ws* s, int l, int lv, const float* z, const float* g, const float* gmask) {
+// gacc[W_l, b_l] += dL/d(W_l, b_l) for the input z of C_l and dL/d(out) = g
+void wgrad(rks_ws* s, int l, int lv, const float* z, const float* g) {
   const int H = lvH(s, lv), W = lvW(s, lv);
   const int cin = conv_cin(l), cout = conv_cout(l);
-  const int ntiles = ((W + kTile - 1) / kTile) * ((H + kTile - 1) / kTile);
-  const int nb = (ntiles + kWgradTiles - 1) / kWgradTiles;
+  const int nb = std::min(kWgCtas, ((W + kWgW - 1) / kWgW) * ((H + kWgH - 1) / kWgH));
   const int cnt = cin * 9 * cout + cout;
-  const int threads = (cin * 9 + cout + 31) / 32 * 32;
-  const size_t sm = (size_t)(cin * kHalo2 + 256 * cout) * sizeof(float);
-  if (cout == 1) k_conv3x3_wgrad<1><<<nb, threads, sm, s->st>>>(z, cin, H, W, g, gmask, s->part);
-  else k_conv3x3_wgrad<kCh><<<nb, threads, sm, s->st>>>(z, cin, H, W, g, gmask, s->part);
-  k_fold_params<<<(cnt + 255) / 256, 256, 0, s->st>>>(s->part, nb, cnt, s->gacc + s->poff[2 * l]);
+  const size_t sm = (size_t)2 * ((kWgPx * (cout == 1 ? 1 : kWgG) + cin * kWgZ + 3) & ~3) * sizeof(float);
+  if (cout == 1) k_wgrad_one<<<nb, 256, sm, s->st>>>(z, H, W, g, s->part);
+  else if (cin == 3) k_wgrad3<<<nb, 256, sm, s->st>>>(z, H, W, g, s->part);
+  else k_wgrad32<<<nb, 256, sm, s->st>>>(z, H, W, g, s->part);
+  k_fold_params<<<(cnt + 31) / 32, 32 * kFoldStrands, 0, s->st>>>(s->part, nb, cnt, s->gacc + s->poff[2 * l]);
 }
 
 void pool(rks_ws* s, int lv, const float* z, float* y) {   // lv: level of z
@@ -392,9 +739,9 @@ void pool(rks_ws* s, int lv, const float* z, float* y) {   // lv: level of z
   k_pool<<<grid1(cnt), 256, 0, s->st>>>(z, kCh, lvH(s, lv), lvW(s, lv), y);
 }
 
-void pool_back(rks_ws* s, int lv, const float* g, float* gz) {   // lv: level of gz
+void pool_back(rks_ws* s, int lv, const float* g, const float* mask, float* gz) {   // lv: level of gz
   const int64_t cnt = (int64_t)kCh * lvH(s, lv) * lvW(s, lv);
-  k_pool_back<<<grid1(cnt), 256, 0, s->st>>>(g, kCh, lvH(s, lv), lvW(s, lv), gz);
+  k_pool_back<<<grid1(cnt), 256, 0, s->st>>>(g, kCh, lvH(s, lv), lvW(s, lv), mask, gz);
 }
 
 void up_add(rks_ws* s, int lv, const float* z, const float* skip, float* y) {   // lv: level of y
@@ -402,9 +749,9 @@ void up_add(rks_ws* s, int lv, const float* z, const float* skip, float* y) {   
   k_up_add<<<grid1(cnt), 256, 0, s->st>>>(z, skip, kCh, lvH(s, lv), lvW(s, lv), y);
 }
 
-void up_back(rks_ws* s, int lv, const float* g, float* gz) {   // lv: level of g
+void up_back(rks_ws* s, int lv, const float* g, const float* mask, float* gz) {   // lv: level of g
   const int64_t cnt = (int64_t)kCh * (lvH(s, lv) / 2) * (lvW(s, lv) / 2);
-  k_up_back<<<grid1(cnt), 256, 0, s->st>>>(g, kCh, lvH(s, lv), lvW(s, lv), gz);
+  k_up_back<<<grid1(cnt), 256, 0, s->st>>>(g, kCh, lvH(s, lv), lvW(s, lv), mask, gz);
 }
 
 void pack_weights(rks_ws* s) {
@@ -417,8 +764,8 @@ void pack_weights(rks_ws* s) {
 
 // block: o = R(C_{l+1}(R(C_l(z)))) at level lv
 void block(rks_ws* s, int l, int lv, const float* z, float* a, float* o) {
-  conv(s, l, lv, z, nullptr, false, 1, a);
-  conv(s, l + 1, lv, a, nullptr, false, 1, o);
+  conv(s, l, lv, z, false, 1, nullptr, a);
+  conv(s, l + 1, lv, a, false, 1, nullptr, o);
 }
 
 void forward(rks_ws* s, const float* x) {
@@ -435,35 +782,36 @@ void forward(rks_ws* s, const float* x) {
   block(s, 10, 1, s->d1in, s->d1a, s->d1);
   up_add(s, 0, s->d1, s->e0, s->d0in);
   block(s, 12, 0, s->d0in, s->d0a, s->d0);
-  conv(s, 14, 0, s->d0, nullptr, false, 0, s->u);
+  conv(s, 14, 0, s->d0, false, 0, nullptr, s->u);
 }
 
-// through o = R(C_{l+1}(R(C_l(z)))) with g = dL/do; gz = dL/dz (unless null)
-void block_back(rks_ws* s, int l, int lv, const float* z, const float* a, const float* o, const float* g, float* ga,
-                float* gz) {
-  wgrad(s, l + 1, lv, a, g, o);
-  conv(s, l + 1, lv, g, o, true, 0, ga);              // dL/da (before the mask of a)
-  wgrad(s, l, lv, z, ga, a);
-  if (gz) conv(s, l, lv, ga, a, true, 0, gz);
+// through o = R(C_{l+1}(R(C_l(z)))): g = dL/do where o > 0 (zero elsewhere);
+// ga is scratch; gz = dL/dz (unless null).  The gradients are masked by the
+// kernels that produce them.
+void block_back(rks_ws* s, int l, int lv, const float* z, const float* a, const float* g, float* ga, float* gz) {
+  wgrad(s, l + 1, lv, a, g);
+  conv(s, l + 1, lv, g, true, 0, a, ga);              // dL/da, masked by a
+  wgrad(s, l, lv, z, ga);
+  if (gz) conv(s, l, lv, ga, true, 0, nullptr, gz);
 }
 
 void backward(rks_ws* s, const float* x) {
   // u = C15(d0)
-  wgrad(s, 14, 0, s->d0, s->gu, nullptr);
-  conv(s, 14, 0, s->gu, nullptr, true, 0, s->gA[0]);  // dL/d(d0)
-  block_back(s, 12, 0, s->d0in, s->d0a, s->d0, s->gA[0], s->gB[0], s->gS[0]);   // gS0 = dL/d(U(d1) + e0)
-  up_back(s, 0, s->gS[0], s->gA[1]);
-  block_back(s, 10, 1, s->d1in, s->d1a, s->d1, s->gA[1], s->gB[1], s->gS[1]);   // gS1 = dL/d(U(d2) + e1)
-  up_back(s, 1, s->gS[1], s->gA[2]);
-  block_back(s, 8, 2, s->d2in, s->d2a, s->d2, s->gA[2], s->gB[2], s->gS[2]);    // gS2 = dL/d(U(e3) + e2)
-  up_back(s, 2, s->gS[2], s->gA[3]);
-  block_back(s, 6, 3, s->p3, s->e3a, s->e3, s->gA[3], s->gB[3], s->gS[3]);      // dL/d(P(e2))
-  pool_back(s, 2, s->gS[3], s->gS[2]);                                           // dL/d(e2)
-  block_back(s, 4, 2, s->p2, s->e2a, s->e2, s->gS[2], s->gB[2], s->gA[2]);      // dL/d(P(e1))
-  pool_back(s, 1, s->gA[2], s->gS[1]);
-  block_back(s, 2, 1, s->p1, s->e1a, s->e1, s->gS[1], s->gB[1], s->gA[1]);      // dL/d(P(e0))
-  pool_back(s, 0, s->gA[1], s->gS[0]);
-  block_back(s, 0, 0, x, s->e0a, s->e0, s->gS[0], s->gB[0], nullptr);
+  wgrad(s, 14, 0, s->d0, s->gu);
+  conv(s, 14, 0, s->gu, true, 0, s->d0, s->gA[0]);                       // dL/d(d0)
+  block_back(s, 12, 0, s->d0in, s->d0a, s->gA[0], s->gB[0], s->gS[0]);   // gS0 = dL/d(U(d1) + e0)
+  up_back(s, 0, s->gS[0], s->d1, s->gA[1]);
+  block_back(s, 10, 1, s->d1in, s->d1a, s->gA[1], s->gB[1], s->gS[1]);   // gS1 = dL/d(U(d2) + e1)
+  up_back(s, 1, s->gS[1], s->d2, s->gA[2]);
+  block_back(s, 8, 2, s->d2in, s->d2a, s->gA[2], s->gB[2], s->gS[2]);    // gS2 = dL/d(U(e3) + e2)
+  up_back(s, 2, s->gS[2], s->e3, s->gA[3]);
+  block_back(s, 6, 3, s->p3, s->e3a, s->gA[3], s->gB[3], s->gS[3]);      // dL/d(P(e2))
+  pool_back(s, 2, s->gS[3], s->e2, s->gS[2]);                             // dL/d(e2)
+  block_back(s, 4, 2, s->p2, s->e2a, s->gS[2], s->gB[2], s->gA[2]);      // dL/d(P(e1))
+  pool_back(s, 1, s->gA[2], s->e1, s->gS[1]);
+  block_back(s, 2, 1, s->p1, s->e1a, s->gS[1], s->gB[1], s->gA[1]);      // dL/d(P(e0))
+  pool_back(s, 0, s->gA[1], s->e0, s->gS[0]);
+  block_back(s, 0, 0, x, s->e0a, s->gS[0], s->gB[0], nullptr);
 }
 
 int launch_ok() { return cudaGetLastError() == cudaSuccess ? RKS_OK : RKS_ECUDA; }
@@ -513,8 +861,8 @@ int rks_ws_create(rks_ws** out, int H, int W, uint64_t seed, void* stream) {
   // e0a e0 d0in d0a d0 gA0 gB0 gS0 | p1 e1a e1 d1in d1a d1 gA1 gB1 gS1 | p2 e2a e2 d2in d2a d2 gA2 gB2 gS2 |
   // p3 e3a e3 gA3 gB3 gS3 | u gu
   const int64_t total = 8 * L[0] + 9 * L[1] + 9 * L[2] + 6 * L[3] + 2 * n0;
-  int ntiles_max = ((W + kTile - 1) / kTile) * ((H + kTile - 1) / kTile);
-  s->part_cap = (int64_t)((ntiles_max + kWgradTiles - 1) / kWgradTiles) * (kCh * 9 * kCh + kCh);
+  const int ntiles_max = ((W + kWgW - 1) / kWgW) * ((H + kWgH - 1) / kWgH);
+  s->part_cap = (int64_t)std::min(kWgCtas, ntiles_max) * (kCh * 9 * kCh + kCh);
   bool ok = cudaMalloc(&s->buf, total * sizeof(float)) == cudaSuccess &&
             cudaMalloc(&s->theta, o * sizeof(float)) == cudaSuccess &&
             cudaMalloc(&s->m, o * sizeof(float)) == cudaSuccess && cudaMalloc(&s->v, o * sizeof(float)) == cudaSuccess &&
@@ -524,8 +872,8 @@ int rks_ws_create(rks_ws** out, int H, int W, uint64_t seed, void* stream) {
             cudaMalloc(&s->lcoef, (kMaxQ + 2) * sizeof(double)) == cudaSuccess;
   for (int l = 0; ok && l < kConvs; ++l) {
     const size_t cnt = (size_t)conv_cin(l) * conv_cout(l) * 9;
-    ok = cudaMalloc(&s->wf[l], cnt * sizeof(__half)) == cudaSuccess &&
-         cudaMalloc(&s->wb[l], cnt * sizeof(__half)) == cudaSuccess;
+    ok = cudaMalloc(&s->wf[l], cnt * sizeof(float)) == cudaSuccess &&
+         (l == 0 || cudaMalloc(&s->wb[l], cnt * sizeof(float)) == cudaSuccess);
   }
   if (!ok) { delete s; return RKS_ENOMEM; }
   float* p = s->buf;
