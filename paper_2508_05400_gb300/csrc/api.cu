@@ -21,6 +21,7 @@
 #include <cstdio>
 #include <cstring>
 #include <new>
+#include <utility>
 #include <vector>
 
 #include "../../include/rks.h"
@@ -78,11 +79,9 @@ struct rks_ctx {
   float* Uf = nullptr;
   void* qimg = nullptr;     // mixed precision: bf16 split image of Q' for the tensor-core restart
   std::vector<uint16_t> qimg_h;
-  void* qimg_df = nullptr;  // double-float basis: digit image of Q', column exponents, row exponents
-  int* fexp_d = nullptr;
-  int* pexp_d = nullptr;     // power-of-two part of the input columns' scales
-  int* rexp_d = nullptr;     // per-row exponents (n)
-  std::vector<int> fexp_h, pexp_h;
+  void* qimg_df = nullptr;  // double-float basis: digit block of Q' (tc_restart_df_blob)
+  std::vector<uint8_t> blob_h;
+  std::vector<int> pexp_h;  // power-of-two part of the input columns' scales
   std::vector<double> Qr_h;
   // rotation of the kept columns still to be applied on the device after the
   // restart's host work (whitening, aggressive reorder): columns corr_q ..
@@ -171,6 +170,34 @@ int* thread_flag() {
     f.p = nullptr;
   }
   return f.p;
+}
+
+// Device block for the small operand of a product (a few hundred KB), for the
+// same kind of call: one per host thread and device, freed when the thread
+// ends; the call synchronises before it returns, so no kernel reads it then.
+struct ThreadBlocks {
+  std::vector<std::pair<int, void*>> b;
+  ~ThreadBlocks() {
+    int cur = 0;
+    if (b.empty() || cudaGetDevice(&cur) != cudaSuccess) return;
+    for (auto& e : b)
+      if (cudaSetDevice(e.first) == cudaSuccess) cudaFree(e.second);
+    cudaSetDevice(cur);
+  }
+};
+void* thread_block() {
+  static thread_local ThreadBlocks t;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+  for (auto& e : t.b)
+    if (e.first == dev) return e.second;
+  void* p = nullptr;
+  if (cudaMalloc(&p, std::max(rks::kTcDfBlobBytes, rks::kTcImageBytes)) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return nullptr;
+  }
+  t.b.emplace_back(dev, p);
+  return p;
 }
 
 int launch_err() {
@@ -482,19 +509,14 @@ int restart_launch(rks_ctx* c, int a0, int nin, const std::vector<double>& Q, co
       const double sc = cs ? cs[l] : 1.0;
       int E = 0;
       if (sc != 0.0) std::frexp(sc, &E);
-      c->pexp_h[l] = sc != 0.0 ? E - 1 : 0;
+      c->pexp_h[l] = sc != 0.0 ? std::min(std::max(E - 1, -126), 126) : 0;
       for (int j = 0; j < nout; ++j)
         c->Qr_h[l + (size_t)j * nin] = std::ldexp(Qp[l + (size_t)j * nin], -c->pexp_h[l]);
     }
-    rks::tc_restart_df_bimage(nin, nout, c->Qr_h.data(), c->qimg_h, c->fexp_h);
-    CK(cudaMemcpyAsync(c->pexp_d, c->pexp_h.data(), c->pexp_h.size() * sizeof(int), cudaMemcpyHostToDevice,
-                       c->stream));
-    CK(cudaMemcpyAsync(c->qimg_df, c->qimg_h.data(), c->qimg_h.size() * sizeof(uint16_t), cudaMemcpyHostToDevice,
-                       c->stream));
-    CK(cudaMemcpyAsync(c->fexp_d, c->fexp_h.data(), c->fexp_h.size() * sizeof(int), cudaMemcpyHostToDevice,
-                       c->stream));
+    rks::tc_restart_df_blob(nin, nout, c->Qr_h.data(), c->pexp_h.data(), c->blob_h);
+    CK(cudaMemcpyAsync(c->qimg_df, c->blob_h.data(), c->blob_h.size(), cudaMemcpyHostToDevice, c->stream));
     float2* U0 = c->U2 + (size_t)a0 * c->ldu;
-    rks::launch_tc_restart_df(c->n, U0, U0, c->ldu, nin, nout, c->qimg_df, c->fexp_d, c->pexp_d, c->rexp_d,
+    rks::launch_tc_restart_df(c->n, U0, U0, c->ldu, nin, nout, c->qimg_df,
                               move_src >= 0 ? c->U2 + (size_t)move_src * c->ldu : nullptr,
                               move_src >= 0 ? c->U2 + (size_t)(a0 + nout) * c->ldu : nullptr, c->flag, c->stream);
   } else if (c->prec != RKS_PREC_FP64) {
@@ -869,7 +891,7 @@ void free_ctx(rks_ctx* c) {
   cudaFree(c->vals2); cudaFree(c->U2); cudaFree(c->S2); cudaFree(c->nrs); cudaFree(c->sj); cudaFree(c->Q2);
   cudaFree(c->rprev); cudaFree(c->znorm); cudaFree(c->tmp64); cudaFree(c->valsf); cudaFree(c->Uf);
   cudaFree(c->otab); cudaFree(c->lsr1); cudaFree(c->M2); cudaFree(c->bar); cudaFree(c->qimg);
-  cudaFree(c->qimg_df); cudaFree(c->fexp_d); cudaFree(c->pexp_d); cudaFree(c->rexp_d);
+  cudaFree(c->qimg_df);
   rks::free_sketch_tiles(&c->tiles);
   cudaFree(c->part_z); cudaFree(c->part_s); cudaFree(c->part_d);
   for (cudaEvent_t e : c->evpool) cudaEventDestroy(e);
@@ -1060,11 +1082,7 @@ int rks_create(rks_ctx** out, int64_t n, const int32_t* rowptr, const int32_t* c
       return fail(rc);
     if (o.tc_restart && rks::tc_restart_df_supported(m, k + 1)) {
       if (rks::configure_tc_kernels() != cudaSuccess) return fail(RKS_ECUDA);
-      if (cudaMalloc(&c->qimg_df, rks::kTcDfImageBytes) != cudaSuccess ||
-          cudaMalloc(&c->fexp_d, 64 * sizeof(int)) != cudaSuccess ||
-          cudaMalloc(&c->pexp_d, 256 * sizeof(int)) != cudaSuccess ||
-          cudaMalloc(&c->rexp_d, (size_t)n * sizeof(int)) != cudaSuccess)
-        return fail(RKS_ENOMEM);
+      if (cudaMalloc(&c->qimg_df, rks::kTcDfBlobBytes) != cudaSuccess) return fail(RKS_ENOMEM);
     }
     if (cudaMemsetAsync(c->bar, 0, 2 * sizeof(unsigned), c->stream) != cudaSuccess) return fail(RKS_ECUDA);
     {
@@ -1793,23 +1811,18 @@ int rks_basis_product_f32(int64_t n, const float* U, int64_t ldu, int nin, const
   cudaStream_t st = (cudaStream_t)stream;
   std::vector<uint16_t> img;
   rks::tc_restart_bimage(nin, nout, Q, img);
-  void* dimg = nullptr;
-  int* flag = nullptr;
-  if (cudaMalloc(&dimg, img.size() * sizeof(uint16_t)) != cudaSuccess) return RKS_ENOMEM;
-  if (cudaMalloc(&flag, sizeof(int)) != cudaSuccess) { cudaFree(dimg); return RKS_ENOMEM; }
-  cudaError_t e = cudaMemsetAsync(flag, 0, sizeof(int), st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(dimg, img.data(), img.size() * sizeof(uint16_t), cudaMemcpyHostToDevice, st);
+  int* flag = thread_flag();
+  void* dimg = thread_block();
+  if (!flag || !dimg) return RKS_ENOMEM;
+  *flag = 0;
+  cudaError_t e = cudaMemcpyAsync(dimg, img.data(), img.size() * sizeof(uint16_t), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) {
     rks::launch_tc_restart_f32(n, U, out, ldu, nin, nout, dimg, nullptr, nullptr, flag, st);
     e = cudaGetLastError();
   }
-  int f = 0;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&f, flag, sizeof(int), cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  cudaFree(dimg);
-  cudaFree(flag);
-  if (e != cudaSuccess) return RKS_ECUDA;
-  return (f & rks::RKS_FLAG_TIMEOUT) ? RKS_ETIMEOUT : RKS_OK;
+  const cudaError_t es = cudaStreamSynchronize(st);
+  if (e != cudaSuccess || es != cudaSuccess) return RKS_ECUDA;
+  return (*flag & rks::RKS_FLAG_TIMEOUT) ? RKS_ETIMEOUT : RKS_OK;
 }
 
 int rks_basis_product_df(int64_t n, const double* U, int64_t ldu, int nin, const double* Q, int nout, double* out,
@@ -1817,42 +1830,20 @@ int rks_basis_product_df(int64_t n, const double* U, int64_t ldu, int nin, const
   if (n <= 0 || ldu < n || !U || !Q || !out || !rks::tc_restart_df_supported(nin, nout)) return RKS_EINVAL;
   if (rks::configure_tc_kernels() != cudaSuccess) return RKS_ECUDA;
   cudaStream_t st = (cudaStream_t)stream;
-  std::vector<uint16_t> img;
-  std::vector<int> fexp;
-  rks::tc_restart_df_bimage(nin, nout, Q, img, fexp);
-  float2 *Ud = nullptr, *Od = nullptr;
-  void* dimg = nullptr;
-  int *dfexp = nullptr, *flag = nullptr, *pexp = nullptr, *rexp = nullptr;
-  int rc = RKS_OK;
-  if (cudaMalloc(&Ud, (size_t)ldu * nin * sizeof(float2)) != cudaSuccess ||
-      cudaMalloc(&Od, (size_t)ldu * nout * sizeof(float2)) != cudaSuccess ||
-      cudaMalloc(&dimg, img.size() * sizeof(uint16_t)) != cudaSuccess ||
-      cudaMalloc(&dfexp, fexp.size() * sizeof(int)) != cudaSuccess ||
-      cudaMalloc(&pexp, (size_t)nin * sizeof(int)) != cudaSuccess ||
-      cudaMalloc(&rexp, (size_t)n * sizeof(int)) != cudaSuccess ||
-      cudaMalloc(&flag, sizeof(int)) != cudaSuccess)
-    rc = RKS_ENOMEM;
-  int f = 0;
-  if (rc == RKS_OK) {
-    cudaError_t e = cudaMemsetAsync(flag, 0, sizeof(int), st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(pexp, 0, (size_t)nin * sizeof(int), st);   // unscaled columns
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(dimg, img.data(), img.size() * sizeof(uint16_t), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(dfexp, fexp.data(), fexp.size() * sizeof(int), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) {
-      rks::launch_d2df((int64_t)ldu * nin, U, Ud, false, st);   // the basis as double-float pairs
-      rks::launch_tc_restart_df(n, Ud, Od, ldu, nin, nout, dimg, dfexp, pexp, rexp, nullptr, nullptr, flag, st);
-      rks::launch_df2d_cols(n, Od, ldu, out, ldu, nout, false, st);
-      e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&f, flag, sizeof(int), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) rc = RKS_ECUDA;
+  std::vector<uint8_t> blob;
+  rks::tc_restart_df_blob(nin, nout, Q, nullptr, blob);   // unscaled columns
+  int* flag = thread_flag();
+  void* dblob = thread_block();
+  if (!flag || !dblob) return RKS_ENOMEM;
+  *flag = 0;
+  cudaError_t e = cudaMemcpyAsync(dblob, blob.data(), blob.size(), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) {
+    rks::launch_tc_product_f64(n, U, out, ldu, nin, nout, dblob, flag, st);
+    e = cudaGetLastError();
   }
-  cudaFree(Ud); cudaFree(Od); cudaFree(dimg); cudaFree(dfexp); cudaFree(pexp); cudaFree(rexp); cudaFree(flag);
-  if (rc != RKS_OK) return rc;
-  return (f & rks::RKS_FLAG_TIMEOUT) ? RKS_ETIMEOUT : RKS_OK;
+  const cudaError_t es = cudaStreamSynchronize(st);
+  if (e != cudaSuccess || es != cudaSuccess) return RKS_ECUDA;
+  return (*flag & rks::RKS_FLAG_TIMEOUT) ? RKS_ETIMEOUT : RKS_OK;
 }
 
 int rks_sketch_apply(int64_t n, int d, int zeta, uint64_t seed, const double* x, double* z, void* stream) {

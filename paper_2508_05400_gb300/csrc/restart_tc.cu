@@ -26,6 +26,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "rks_impl.h"
@@ -81,23 +82,29 @@ __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::be
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
-// Bounded wait for the completion of the mbarrier phase with this parity.
-__device__ bool mbar_wait(uint32_t mbar, uint32_t parity, int* flag) {
+__device__ __forceinline__ bool mbar_try(uint32_t mbar, uint32_t parity) {
+  uint32_t done;
+  asm volatile(
+      "{\n\t.reg .pred P1;\n\tmbarrier.try_wait.parity.shared::cta.b64 P1, [%1], %2;\n\t"
+      "selp.b32 %0, 1, 0, P1;\n\t}\n"
+      : "=r"(done)
+      : "r"(mbar), "r"(parity)
+      : "memory");
+  return done != 0;
+}
+__device__ __noinline__ bool mbar_wait_slow(uint32_t mbar, uint32_t parity, int* flag) {
   const long long t0 = clock64();
-  while (true) {
-    uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred P1;\n\tmbarrier.try_wait.parity.shared::cta.b64 P1, [%1], %2;\n\t"
-        "selp.b32 %0, 1, 0, P1;\n\t}\n"
-        : "=r"(done)
-        : "r"(mbar), "r"(parity)
-        : "memory");
-    if (done) return true;
+  while (!mbar_try(mbar, parity)) {
     if (clock64() - t0 > 2000000000ll) {
       atomicOr(flag, RKS_FLAG_TIMEOUT);
       return false;
     }
   }
+  return true;
+}
+// Bounded wait for the completion of the mbarrier phase with this parity.
+__device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, int* flag) {
+  return mbar_try(mbar, parity) || mbar_wait_slow(mbar, parity, flag);
 }
 
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
@@ -110,6 +117,16 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
   for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
+}
+
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
+  uint32_t r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int j = 0; j < 8; ++j) v[j] = __uint_as_float(r[j]);
 }
 
 __device__ __forceinline__ uint32_t bf16_bits(__nv_bfloat16 h) { return (uint32_t)__bfloat16_as_ushort(h); }
@@ -285,103 +302,126 @@ __global__ void __launch_bounds__(kThreads, 3) k_tc_restart_f32(int64_t n, const
 // Double-float basis: exact split products (Ozaki-type) on the tensor cores
 // ---------------------------------------------------------------------------
 //
-// A DF value v = hi + lo of row i is written, relative to the row scale 2^e_i
-// (|v| < 2^(e_i - 1) for every input column), as the 47-bit fixed-point
-// integer V = round(v 2^(48 - e_i)) = sum_s d_s 2^(42 - 7s), a signed top
-// digit d_0 (|d_0| <= 32) and six 7-bit digits (0..127), all exact in bf16;
-// Q' likewise per column with scale 2^f_o (digits c_t, built on the host).
-// Then
+// A value v of row i is written, relative to the row scale 2^e_i
+// (|v| < 2^(e_i - 1) for every input column, its column's power of two
+// included), as the fixed-point integer V = round(v 2^(48 - e_i)) =
+// sum_s d_s 2^(42 - 7s) with seven balanced digits |d_s| <= 64; Q' likewise
+// per column with scale 2^f_o (digits c_t, built on the host).  Then
 //   sum_l v_l q_l = 2^(e_i + f_o - 12) sum_g 2^(-7g) G_g,
 //   G_g = sum_{s + t = g} sum_l d_s(i, l) c_t(l, o),
 // with integer G_g.  The 34 digit pairs with s + t <= 7 go to 8 accumulators
-// (8 x N tensor-memory columns; the dropped pairs are below 5 * 2^-51 of
-// the scale).  For K <= 192 every group of weight above 2^-35 stays below
-// 2^24, so the bf16 MMAs with FP32 accumulation in tensor memory sum it
-// exactly; a lighter group may round by a unit or two, far below 2^-48.
-// The epilogue combines the groups in DF.  K streams through two shared-
-// memory stages of one K-step (16 input columns x 7 digit slices); Q'
-// (7 slices, all K) stays resident.
+// (8 x N tensor-memory columns); the dropped pairs are below 2^-50 of the
+// scale.  The bf16 operand holds d_s + 192 (128 .. 256, exact), whose sum
+// over l is 192 sum_l c_t(l, o) too large: a constant per group and output
+// (corr, from the host) that the epilogue subtracts.  For K <= 192 every group
+// of weight above 2^-35 stays below 5 * 192 * 256 * 64 < 2^24, so the
+// bf16 MMAs with FP32 accumulation in tensor memory sum it exactly; a lighter
+// group may round by a unit or two, far below 2^-48.
+//
+// The digits cost three FP32 adds each (|d_s| <= 64 holds as the low word of
+// v, below 2^-5 of a unit when it enters, cannot push a digit over): with M_s = 2^(-7s) (1.5 2^23 +
+// 0x4340), t = x + M_s rounds x to a multiple of 2^(-7s), and the low 16 bits
+// of t are the bf16 pattern of d_s + 192; x - (t - M_s) is the exact rest.
+// (Cutting a 64-bit integer and converting every digit took three times the
+// instructions and bound the kernel.)  Slices of Q' lie side by side, so
+// that one MMA multiplies a digit slice of U by all its slices of Q' (up to
+// N = 256) where one MMA per pair re-read the U slice 34 times.
+// K streams through two shared-memory stages of one K-step (16 input columns
+// x 7 digit slices); Q' (7 slices, all K) stays resident.  The row exponents
+// of a CTA's next tile are formed while the current one is processed, which
+// also brings that tile into L2: HBM sees every input once.
+// Measured, n = 1e6, 80 -> 21 columns: see launch_tc_restart_df.
 
 constexpr int kDfDigits = 7;
-constexpr int kDfThreads = 512;
+constexpr int kDfThreads = 256;
 constexpr int kDfGroups = 8;
 constexpr int kDfStepSplit = kM * 16 * 2;                 // one digit slice of one K-step
 constexpr int kDfStage = kDfDigits * kDfStepSplit;        // 28 KB
 
-// Largest biased exponent of the hi parts of row i over the nin columns, each
-// column taken times 2^pexp[l] (its power-of-two scale; zero entries skipped).
-__global__ void k_row_exp(int64_t n, const float2* __restrict__ in, int64_t ldu, int nin,
-                          const int* __restrict__ pexp, int* __restrict__ rexp) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    int em = -100000;
-#pragma unroll 8
-    for (int l = 0; l < nin; ++l) {
-      const int E = (int)((__float_as_uint(in[i + (int64_t)l * ldu].x) >> 23) & 0xFFu);
-      if (E != 0) em = max(em, E + pexp[l]);
-    }
-    rexp[i] = em;
+// Shared-memory matrix descriptor of a K-major, no-swizzle operand whose
+// rows lie 16 bytes apart: SBO (next 8 rows) 128 bytes, LBO (next 8 columns) lbo.
+__device__ __forceinline__ uint64_t sdesc_rows(uint32_t addr, uint32_t lbo) {
+  return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo >> 4) << 16) | ((uint64_t)(128 >> 4) << 32) |
+         (1ull << 46);
+}
+
+// What the split needs of a type.  Row exponents are kept biased and clamped
+// to [4, 257], so that the row factor 2^(131 - emax) is a float; rows below or
+// above lie outside what an FP32 pair resolves.
+//   key / key_exp: running maximum over a row and its biased exponent
+//   scaled:        v 2^p 2^(6 - e_i) as x + y (x the leading bits,
+//                  |y| < 2^-22 |x|, |x| < 32)
+template <class T>
+struct Split;
+template <>
+struct Split<float2> {
+  typedef float Key;     // |hi| 2^p
+  typedef float Probe;   // what a row maximum reads of a value
+  static __device__ __forceinline__ Probe probe(const float2* p) { return p->x; }
+  static __device__ __forceinline__ Key key(Key k, Probe v, float col) { return fmaxf(k, fabsf(v * col)); }
+  static __device__ __forceinline__ int key_exp(Key k) { return min(max((int)(__float_as_uint(k) >> 23), 4), 257); }
+  static __device__ __forceinline__ int scale(int emax) { return emax - 125; }   // e_i
+  static __device__ __forceinline__ float row(int emax) { return __int_as_float((131 - emax + 127) << 23); }
+  static __device__ __forceinline__ void scaled(float2 v, float col, float rowf, float& x, float& y) {
+    x = v.x * col * rowf;
+    y = v.y * col * rowf;
   }
-}
+};
+// The FP64 pipe is 60 times slower than the FP32 one, so a double is taken
+// apart with integer operations: 24 leading bits, and 23 more rounded.  (No
+// column factors: the FP64 product has none.)
+template <>
+struct Split<double> {
+  typedef int Key;       // high word without the sign
+  typedef int Probe;
+  static __device__ __forceinline__ Probe probe(const double* p) { return reinterpret_cast<const int*>(p)[1]; }
+  static __device__ __forceinline__ Key key(Key k, Probe v, float) { return max(k, v & 0x7FFFFFFF); }
+  static __device__ __forceinline__ int key_exp(Key k) { return max(k >> 20, 1); }
+  static __device__ __forceinline__ int scale(int emax) { return emax - 1021; }
+  static __device__ __forceinline__ int row(int emax) { return (131 - emax) * (1 << 20); }
+  static __device__ __forceinline__ void scaled(double v, float, int rowk, float& x, float& y) {
+    const int hi = __double2hiint(v), lo = __double2loint(v);
+    const int d = (hi & 0x7FFFFFFF) + rowk;                 // biased exponent of x, 20 bits of mantissa
+    const int xb = __funnelshift_l(lo, d, 3), sg = hi & 0x80000000;
+    const float yi = __int_as_float((((lo & 0x1FFFFFFF) + 32) >> 6) + 0x4B000000) - 8388608.0f;
+    x = d >= 1 << 20 ? __int_as_float(xb | sg) : 0.f;
+    y = d >= 47 << 20 ? yi * __int_as_float(((xb & 0x7F800000) - (46 << 23)) | sg) : 0.f;
+  }
+};
 
-// bf16 bits of a small integer 0 <= d < 256 on the full-rate pipes: the
-// float 2^23 + d minus 2^23 is d exactly, and its low 16 bits are zero.
-__device__ __forceinline__ uint32_t small_bf16(int d) {
-  return __float_as_uint(__int_as_float(0x4B000000 | d) - 8388608.0f) >> 16;
-}
-
-// round(x 2^(48 - e)) with e = emax - 125, from the bits of x (|result| <= 2^47 + 1);
-// a column scale 2^p is applied by passing emax - p
-__device__ __forceinline__ int64_t fixed48(float x, int emax) {
-  const uint32_t b = __float_as_uint(x);
-  int E = (int)((b >> 23) & 0xFFu);
-  uint32_t m = b & 0x7FFFFFu;
-  if (E == 0) E = 1; else m |= 0x800000u;
-  const int sh = E - emax + 23;                  // E - 102 - e
-  int64_t V;
-  if (sh >= 0) V = (int64_t)m << min(sh, 40);   // sh <= 23 except for an all-zero row (m = 0)
-  else if (sh > -26) V = (int64_t)((m + (1u << (-sh - 1))) >> -sh);
-  else V = 0;
-  return (b >> 31) ? -V : V;
-}
-
-// out[i, o] = sum_l in[i, l] 2^pexp[l] Q'[l, o] (DF) for i < n, o < nout;
-// then, when mvsrc is given, mvdst[i] = mvsrc[i].  bimg: the digit slices of
-// Q' (Kp x N, canonical layout, slice t at byte t * Kp * N * 2); fexp[o] =
-// f_o; rexp[i] from k_row_exp.  Every read of a tile's rows precedes its
-// writes (in place).
-//
-// Warp roles: warps 0..15 (kDfThreads threads) load and split the digits of
-// one K-step into a shared-memory stage and run the epilogue; warp 16 issues
-// the MMAs.  Per stage s: full[s] (the splitters arrive once the digits are
-// stored) and empty[s] (the MMA commit arrives once they are consumed); per
-// tile: done (accumulators complete) and tfree (the epilogue has read them).
-// The split of step g + 1 thus overlaps the MMA issue of step g.  Every wait
-// is bounded (mbar_wait); the splitters agree on the outcome at their named
-// barrier, so a timeout ends every role's loop.
-__device__ __forceinline__ bool splitters_and(bool p) {
-  uint32_t r;
-  asm volatile(
-      "{\n\t.reg .pred P, Q;\n\tsetp.ne.u32 P, %1, 0;\n\tbar.red.and.pred Q, 1, %2, P;\n\t"
-      "selp.u32 %0, 1, 0, Q;\n\t}\n"
-      : "=r"(r)
-      : "r"((uint32_t)p), "n"(kDfThreads)
-      : "memory");
-  return r != 0;
-}
 __device__ __forceinline__ void mbar_arrive(uint32_t mbar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(mbar) : "memory");
 }
 
 constexpr int kDfAllThreads = kDfThreads + 32;
 
-__global__ void __launch_bounds__(kDfAllThreads, 1) k_tc_restart_df(int64_t n, const float2* in, float2* out,
-                                                                    int64_t ldu, int nin, int Kp, int N, int nout,
-                                                                    const uint4* __restrict__ bimg,
-                                                                    const int* __restrict__ fexp,
-                                                                    const int* __restrict__ pexp,
-                                                                    const int* __restrict__ rexp,
-                                                                    const float2* mvsrc, float2* mvdst, int tcols,
-                                                                    int* flag) {
+// Host data of one product, in one device block: column exponents, input
+// column powers of two, group corrections, then the digit image.
+struct DfBlobHead {
+  int fexp[64];
+  int pexp[256];
+  float corr[kDfGroups * 64];   // [group][output of N]
+};
+static_assert(sizeof(DfBlobHead) % 16 == 0, "the digit image follows, read in 16-byte pieces");
+
+// out[i, o] = sum_l in[i, l] 2^pexp[l] Q'[l, o] for i < n, o < nout; then,
+// when mvsrc is given, mvdst[i] = mvsrc[i].  Input and output in double-float
+// or both in FP64.  Every read of a tile's rows precedes its writes (in
+// place).
+//
+// Warp roles: warps 0..7 load and split the digits of one K-step into a
+// shared-memory stage and run the epilogue; warp 8 issues the MMAs.  Per
+// stage s: full[s] (every splitter arrives once its digits are stored) and
+// empty[s] (the MMA commit arrives once they are consumed); per tile: done
+// (accumulators complete) and tfree (the epilogue has read them).  Every wait
+// is bounded (mbar_wait); a thread whose wait gave up skips its later waits
+// and otherwise goes on, so that every barrier keeps its count.
+template <class T, int MINB>
+__global__ void __launch_bounds__(kDfAllThreads, MINB) k_tc_restart_df(int64_t n, const T* in, T* out, int64_t ldu,
+                                                                       int nin, int Kp, int N, int nout,
+                                                                       const DfBlobHead* __restrict__ head,
+                                                                       const T* mvsrc, T* mvdst, int tcols,
+                                                                       int* flag) {
   extern __shared__ __align__(1024) uint8_t smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int bbytes = kDfDigits * Kp * N * 2;
@@ -389,19 +429,22 @@ __global__ void __launch_bounds__(kDfAllThreads, 1) k_tc_restart_df(int64_t n, c
   uint8_t* sA = smem + ((bbytes + 1023) & ~1023);
   uint64_t* mbar = reinterpret_cast<uint64_t*>(sA + 2 * kDfStage);   // full[2], empty[2], done, tfree
   uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + 6);
-  int* sp = reinterpret_cast<int*>(mbar + 7);            // column power-of-two scales (Kp)
+  float* colf = reinterpret_cast<float*>(mbar + 8);      // 2^pexp (Kp; the last column repeated)
+  short* rowe = reinterpret_cast<short*>(colf + Kp);     // [tile parity][column half][row] largest exponents
   const uint32_t full0 = smem_u32(mbar + 0), empty0 = smem_u32(mbar + 2);
   const uint32_t done_b = smem_u32(mbar + 4), tfree_b = smem_u32(mbar + 5);
+  const uint4* bimg = reinterpret_cast<const uint4*>(head + 1);
 
   for (int t = tid; t < bbytes / 16; t += kDfAllThreads) reinterpret_cast<uint4*>(sB)[t] = bimg[t];
-  for (int t = tid; t < Kp; t += kDfAllThreads) sp[t] = t < nin ? pexp[t] : 0;
+  for (int t = tid; t < Kp; t += kDfAllThreads) colf[t] = __int_as_float((head->pexp[min(t, nin - 1)] + 127) << 23);
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
                  "r"(tcols));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   if (tid == 0) {
-    for (int s = 0; s < 6; ++s) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(mbar + s)));
+    for (int s = 0; s < 6; ++s)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(mbar + s)), "r"(s < 2 || s == 5 ? kDfThreads : 1));
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   fence_async_smem();
@@ -414,33 +457,36 @@ __global__ void __launch_bounds__(kDfAllThreads, 1) k_tc_restart_df(int64_t n, c
   bool ok = true;
 
   if (warp == kDfThreads / 32) {
-    // ---- MMA issuer (lane 0 of warp 16)
+    // ---- MMA issuer (lane 0 of warp 8)
     if (lane == 0) {
-      const uint32_t idesc = idesc_bf16(N);
       const uint32_t sA32 = smem_u32(sA), sB32 = smem_u32(sB);
+      const uint32_t blbo = (uint32_t)(kDfDigits * N * 16);
+      const int per = 256 / N;                           // slices of Q' in one MMA
       int g = 0, tcount = 0;
-      for (int64_t tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++tcount) {
-        if (tcount > 0) {   // the epilogue of the previous tile has read the accumulators
-          ok = mbar_wait(tfree_b, (uint32_t)((tcount - 1) & 1), flag);
-          if (!ok) break;
-          fence_after();
-        }
+      for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++tcount) {
+        if (tcount > 0 && ok) ok = mbar_wait(tfree_b, (uint32_t)((tcount - 1) & 1), flag);   // accumulators read
+        fence_after();
         for (int kc = 0; kc < nk; ++kc, ++g) {
           const int s = g & 1;
-          ok = mbar_wait(full0 + 8u * s, (uint32_t)((g >> 1) & 1), flag);
-          if (!ok) break;
+          if (ok) ok = mbar_wait(full0 + 8u * s, (uint32_t)((g >> 1) & 1), flag);
           fence_after();
-          const bool first = kc == 0;
-#pragma unroll
-          for (int gg = 0; gg < kDfGroups; ++gg)
-#pragma unroll
-            for (int sa = gg < kDfDigits ? 0 : gg - kDfDigits + 1; sa <= gg && sa < kDfDigits; ++sa) {
-              const int tb = gg - sa;
-              const int sa0 = gg < kDfDigits ? 0 : gg - kDfDigits + 1;   // first pair of the group
-              const uint64_t a = sdesc(sA32 + s * kDfStage + sa * kDfStepSplit);
-              const uint64_t b = sdesc(sB32 + tb * Kp * N * 2 + kc * N * 32);
-              mma_bf16(tmem + (uint32_t)(gg * N), a, b, idesc, (first && sa == sa0) ? 0u : 1u);
+          if (ok) {
+            const uint32_t b0 = sB32 + (uint32_t)kc * 2u * blbo;
+            for (int sa = 0; sa < kDfDigits; ++sa) {
+              const uint64_t a = sdesc_rows(sA32 + s * kDfStage + sa * kDfStepSplit, 2048);
+              const int t1 = sa <= 1 ? kDfDigits : kDfGroups - sa;   // slices 0 .. t1 - 1: groups sa .. sa + t1 - 1
+              for (int t = 0; t < t1;) {
+                // the first K-step clears the accumulators: groups 0 .. 6 with
+                // digit 0, group 7 with its first pair (digit 1, slice 6)
+                const bool last7 = kc == 0 && sa == 1 && t == kDfDigits - 1;
+                int cnt = min(per, t1 - t);
+                if (kc == 0 && sa == 1 && !last7) cnt = min(cnt, kDfDigits - 1 - t);
+                mma_bf16(tmem + (uint32_t)((sa + t) * N), a, sdesc_rows(b0 + (uint32_t)(t * N * 16), blbo),
+                         idesc_bf16(cnt * N), (kc == 0 && (sa == 0 || last7)) ? 0u : 1u);
+                t += cnt;
+              }
             }
+          }
           mma_commit(empty0 + 8u * s);
           if (kc == nk - 1) mma_commit(done_b);
         }
@@ -451,121 +497,205 @@ __global__ void __launch_bounds__(kDfAllThreads, 1) k_tc_restart_df(int64_t n, c
     }
     __syncwarp();
   } else {
-    // ---- splitters (warps 0..15) and the epilogue
+    // ---- splitters (warps 0..7) and the epilogue
     int g = 0;                 // stages filled so far (all tiles)
-    uint32_t dpar = 0;         // parity of the accumulator-done barrier
-    const int r = tid & (kM - 1), kq = tid >> 7;   // loader: row, quarter of the K-step's 16 columns
-    auto load4 = [&](int64_t tile, int kc, float2* v) {
+    uint32_t tpar = 0;         // parity of the tile (accumulator-done barrier, row exponents)
+    // a thread has one row and 8 of the 16 columns: one 16-byte store per digit
+    const int r = tid & (kM - 1), c8 = (tid >> 7) * 8;
+    // Rows past n and columns past nin repeat the last one: their outputs are
+    // not stored, their rows of Q' are zero.
+    typedef Split<T> S;
+    auto row_ptr = [&](int64_t tile) {
       const int64_t i = tile * kM + r;
-      const int l0 = kc * 16 + kq * 4;
+      return in + (i < n ? i : n - 1);
+    };
+    auto col_off = [&](int c, int u) { return (int64_t)min(c + u, nin - 1) * ldu; };
+    auto put_rowe = [&](uint32_t par, typename S::Key key) {
+      rowe[(par * 2 + (c8 >> 3)) * kM + r] = (short)S::key_exp(key);
+    };
+    {
+      typename S::Key key = 0;
+      const T* p0 = row_ptr(blockIdx.x);
+#pragma unroll 2
+      for (int kc = 0; kc < nk; ++kc) {
+        const int c = kc * 16 + c8;
+        typename S::Probe pm[8];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int l = l0 + u;
-        v[u] = (tile < ntiles && i < n && l < nin) ? in[i + (int64_t)l * ldu] : make_float2(0.f, 0.f);
+        for (int u = 0; u < 8; ++u) pm[u] = S::probe(p0 + col_off(c, u));
+#pragma unroll
+        for (int u = 0; u < 8; ++u) key = S::key(key, pm[u], colf[c + u]);
       }
-    };
-    auto next_step = [&](int64_t& t, int& k) {
-      if (++k == nk) { k = 0; t += gridDim.x; }
-    };
-    float2 v[4], vn[4];   // the next K-step's values are loaded during this one's split
-    int64_t pt = blockIdx.x;
-    int pk = 0;
-    load4(pt, pk, v);
-    for (int64_t tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
-      const int64_t irow = tile * kM + r;
-      const int emax = irow < n ? rexp[irow] : 0;
-      for (int kc = 0; kc < nk && ok; ++kc, ++g) {
+      put_rowe(0, key);
+    }
+    T v[8], vn[8];             // the next K-step's values are loaded during this one's split
+    const T* pv = row_ptr(blockIdx.x);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = pv[col_off(c8, u)];
+    asm volatile("bar.sync 1, %0;" ::"n"(kDfThreads) : "memory");
+    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, tpar ^= 1u) {
+      const short* re = rowe + tpar * 2 * kM;
+      const auto rowf = S::row(max((int)re[r], (int)re[kM + r]));
+      const bool more = tile + gridDim.x < ntiles;
+      const T* pnext = row_ptr(more ? tile + gridDim.x : tile);
+      typename S::Key key = 0;   // the next tile's row maximum, its loads consumed one K-step later
+      typename S::Probe pm[8];
+      for (int kc = 0; kc < nk; ++kc, ++g) {
         const int s = g & 1;
-        next_step(pt, pk);
-        load4(pt, pk, vn);
-        if (g >= 2) ok = mbar_wait(empty0 + 8u * s, (uint32_t)(((g - 2) >> 1) & 1), flag);
-        ok = splitters_and(ok);
-        if (!ok) break;
-        // digits of 4 values of one row
-        uint32_t w[kDfDigits][2];
+        const int c = kc * 16 + c8;
+        const int cn = kc + 1 < nk ? c + 16 : c8;
+        const T* ps = kc + 1 < nk ? pv : pnext;
+        if (cn + 8 <= nin) {
+          ps += (int64_t)cn * ldu;
 #pragma unroll
-        for (int u = 0; u < 4; u += 2) {
-          uint32_t pk2[kDfDigits][2];
+          for (int u = 0; u < 8; ++u) vn[u] = ps[u * ldu];
+        } else {
 #pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            const float2 x = v[u + e];
-            const int ep = emax - sp[kc * 16 + kq * 4 + u + e];
-            const int64_t V = fixed48(x.x, ep) + fixed48(x.y, ep);
-            // digits from two 32-bit halves: bits 21..47 (signed) and 0..20
-            const int vh = (int)(V >> 21);
-            const int vl = (int)(V & 0x1FFFFF);
-            const int d0 = vh >> 21;                                   // -32 .. 32
-            pk2[0][e] = __float_as_uint(__int_as_float(0x4B000000 | (d0 + 128)) - 8388736.0f) >> 16;
-            pk2[1][e] = small_bf16((vh >> 14) & 127);
-            pk2[2][e] = small_bf16((vh >> 7) & 127);
-            pk2[3][e] = small_bf16(vh & 127);
-            pk2[4][e] = small_bf16(vl >> 14);
-            pk2[5][e] = small_bf16((vl >> 7) & 127);
-            pk2[6][e] = small_bf16(vl & 127);
-          }
-#pragma unroll
-          for (int q = 0; q < kDfDigits; ++q) w[q][u >> 1] = pk2[q][0] | (pk2[q][1] << 16);
+          for (int u = 0; u < 8; ++u) vn[u] = ps[col_off(cn, u)];
         }
-        uint8_t* st = sA + s * kDfStage;
-        const uint32_t off = canon_off(r, kq * 4, kM);
+        if (kc > 0) {
 #pragma unroll
-        for (int q = 0; q < kDfDigits; ++q)
-          *reinterpret_cast<uint2*>(st + q * kDfStepSplit + off) = make_uint2(w[q][0], w[q][1]);
+          for (int u = 0; u < 8; ++u) key = S::key(key, pm[u], colf[c - 16 + u]);
+        }
+        if (more) {
+          if (c + 8 <= nin) {
+            const T* pp = pnext + (int64_t)c * ldu;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) pm[u] = S::probe(pp + u * ldu);
+          } else {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) pm[u] = S::probe(pnext + col_off(c, u));
+          }
+        }
+        // digits of 8 values of one row
+        uint32_t w[kDfDigits][4];
+#pragma unroll
+        for (int u = 0; u < 8; u += 2) {
+          float x[2], y[2];
+          S::scaled(v[u], colf[c + u], rowf, x[0], y[0]);
+          S::scaled(v[u + 1], colf[c + u + 1], rowf, x[1], y[1]);
+#pragma unroll
+          for (int d = 0; d < kDfDigits; ++d) {
+            const float m = __int_as_float(0x4B404340 - ((7 * d) << 23));
+            uint32_t b[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+              // the low word enters in two parts, each far below a unit of its digit
+              if (d == 2) {
+                const float z = x[e] + y[e];
+                y[e] -= z - x[e];
+                x[e] = z;
+              }
+              if (d == 4) x[e] += y[e];
+              const float t = x[e] + m;
+              b[e] = __float_as_uint(t);
+              x[e] -= t - m;
+            }
+            w[d][u >> 1] = __byte_perm(b[0], b[1], 0x5410);
+          }
+        }
+        if (ok && g >= 2) ok = mbar_wait(empty0 + 8u * s, (uint32_t)(((g - 2) >> 1) & 1), flag);
+        uint8_t* st = sA + s * kDfStage + (c8 >> 3) * 2048 + r * 16;
+#pragma unroll
+        for (int d = 0; d < kDfDigits; ++d)
+          *reinterpret_cast<uint4*>(st + d * kDfStepSplit) = make_uint4(w[d][0], w[d][1], w[d][2], w[d][3]);
         fence_async_smem();
-        asm volatile("bar.sync 1, %0;" ::"n"(kDfThreads) : "memory");
-        if (tid == 0) mbar_arrive(full0 + 8u * s);
+        mbar_arrive(full0 + 8u * s);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = vn[u];
+        for (int u = 0; u < 8; ++u) v[u] = vn[u];
       }
-      if (!ok) break;
-      // epilogue: sum_g 2^(-7g) G_g in DF, times 2^(e_i + f_o - 12)
-      ok = mbar_wait(done_b, dpar, flag);
-      dpar ^= 1u;
-      ok = splitters_and(ok);
-      if (!ok) break;
+      pv = pnext;
+      if (more) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) key = S::key(key, pm[u], colf[(nk - 1) * 16 + c8 + u]);
+        put_rowe(tpar ^ 1u, key);
+      }
+      // epilogue: sum_g 2^(-7g) (G_g - corr_g), times 2^(e_i + f_o - 12)
+      if (ok) ok = mbar_wait(done_b, tpar, flag);
       fence_after();
       const int q4 = warp & 3;
       const int64_t ir = tile * kM + q4 * 32 + lane;
-      const int er = ir < n ? rexp[ir] - 125 : 0;
-      float2 mv = make_float2(0.f, 0.f);
+      const int er = S::scale(max((int)re[q4 * 32 + lane], (int)re[kM + q4 * 32 + lane])) - 12;
+      T mv{};
       if (mvsrc && warp < 4 && ir < n) mv = mvsrc[ir];
-      for (int cg = warp >> 2; cg < N / 16; cg += kDfThreads / 128) {
-        float hs[16], ls[16];
-        {
-          float gv[16];
-          tmem_ld16(tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)((kDfGroups - 1) * N + cg * 16), gv);
+      for (int cg = warp >> 2; cg < N / 8; cg += kDfThreads / 128) {
+        const uint32_t tc = tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(cg * 8);
+        const float* co = head->corr + cg * 8;
+        if constexpr (sizeof(T) == 8 && !std::is_same<T, double>::value) {
+          float hs[8], ls[8];
+          for (int gg = kDfGroups - 1; gg >= 0; --gg) {
+            float gv[8];
+            tmem_ld8(tc + (uint32_t)(gg * N), gv);
+            const float4 ca = __ldg(reinterpret_cast<const float4*>(co + gg * N));
+            const float4 cb = __ldg(reinterpret_cast<const float4*>(co + gg * N) + 1);
+            const float cc[8] = {ca.x, ca.y, ca.z, ca.w, cb.x, cb.y, cb.z, cb.w};
 #pragma unroll
-          for (int jj = 0; jj < 16; ++jj) { hs[jj] = gv[jj]; ls[jj] = 0.f; }
-        }
-        for (int gg = kDfGroups - 2; gg >= 0; --gg) {
-          float gv[16];
-          tmem_ld16(tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(gg * N + cg * 16), gv);
-#pragma unroll
-          for (int jj = 0; jj < 16; ++jj) {
-            const float sh = hs[jj] * 0.0078125f, sl = ls[jj] * 0.0078125f;   // exact scaling by 2^-7
-            float s2, e2;
-            two_sum_f(gv[jj], sh, s2, e2);
-            hs[jj] = s2;
-            ls[jj] = e2 + sl;
+            for (int jj = 0; jj < 8; ++jj) {
+              const float a = gv[jj] - cc[jj];
+              if (gg == kDfGroups - 1) {
+                hs[jj] = a;
+                ls[jj] = 0.f;
+              } else {
+                const float sh = hs[jj] * 0.0078125f, sl = ls[jj] * 0.0078125f;   // exact scaling by 2^-7
+                float s2, e2;
+                two_sum_f(a, sh, s2, e2);
+                hs[jj] = s2;
+                ls[jj] = e2 + sl;
+              }
+            }
           }
-        }
-        if (ir < n) {
+          if (ir < n) {
 #pragma unroll
-          for (int jj = 0; jj < 16; ++jj) {
-            const int o = cg * 16 + jj;
-            if (o < nout) {
-              const int sc = er + fexp[o] - 12;
-              float h, l;
-              two_sum_f(hs[jj], ls[jj], h, l);
-              out[ir + (int64_t)o * ldu] = make_float2(ldexpf(h, sc), ldexpf(l, sc));
+            for (int jj = 0; jj < 8; ++jj) {
+              const int o = cg * 8 + jj;
+              if (o < nout) {
+                const int sc = er + head->fexp[o];
+                float hh, ll;
+                two_sum_f(hs[jj], ls[jj], hh, ll);
+                out[ir + (int64_t)o * ldu] = make_float2(ldexpf(hh, sc), ldexpf(ll, sc));
+              }
+            }
+          }
+        } else {
+          // FP64: the groups as one 64-bit integer (group 7 rounded to a unit
+          // of group 6), converted once
+          long long acc[8], top[8];
+#pragma unroll
+          for (int gg = kDfGroups - 1; gg >= 0; --gg) {
+            float gv[8];
+            tmem_ld8(tc + (uint32_t)(gg * N), gv);
+            const float4 ca = __ldg(reinterpret_cast<const float4*>(co + gg * N));
+            const float4 cb = __ldg(reinterpret_cast<const float4*>(co + gg * N) + 1);
+            const float cc[8] = {ca.x, ca.y, ca.z, ca.w, cb.x, cb.y, cb.z, cb.w};
+#pragma unroll
+            for (int jj = 0; jj < 8; ++jj) {
+              const float a = gv[jj] - cc[jj];
+              if (gg == kDfGroups - 1) acc[jj] = __float2int_rn(a * 0.0078125f);
+              else if (gg >= 2) acc[jj] += (long long)__float2int_rn(a) * (1ll << (7 * (kDfGroups - 2 - gg)));
+              else if (gg == 1) top[jj] = __float2int_rn(a);
+              else acc[jj] += (top[jj] + ((long long)__float2int_rn(a) << 7)) << 35;
+            }
+          }
+          if (ir < n) {
+#pragma unroll
+            for (int jj = 0; jj < 8; ++jj) {
+              const int o = cg * 8 + jj;
+              if (o < nout) {
+                const int sc = er + head->fexp[o] - 42;
+                const double d = __ll2double_rn(acc[jj]);
+                const int hi = __double2hiint(d), e = ((hi >> 20) & 0x7FF) + sc;
+                // scaling by an exponent add where the result is a normal number
+                out[ir + (int64_t)o * ldu] = (hi & 0x7FF00000) == 0 ? d
+                                             : e > 0 && e < 0x7FF   ? __hiloint2double(hi + (sc << 20), __double2loint(d))
+                                                                    : scalbn(d, sc);
+              }
             }
           }
         }
       }
       if (mvsrc && warp < 4 && ir < n) mvdst[ir] = mv;
       fence_before();
-      asm volatile("bar.sync 1, %0;" ::"n"(kDfThreads) : "memory");
-      if (tid == 0) mbar_arrive(tfree_b);
+      mbar_arrive(tfree_b);
+      asm volatile("bar.sync 1, %0;" ::"n"(kDfThreads) : "memory");   // the next tile's row exponents
     }
   }
   fence_before();
@@ -619,61 +749,96 @@ static int df_n(int nout) { return (nout + 15) / 16 * 16; }
 
 size_t tc_restart_df_smem(int nin, int nout) {
   const size_t b = (size_t)kDfDigits * df_kp(nin) * df_n(nout) * 2;
-  return ((b + 1023) & ~(size_t)1023) + 2 * kDfStage + 64 + (size_t)df_kp(nin) * sizeof(int);
+  return ((b + 1023) & ~(size_t)1023) + 2 * kDfStage + 64 + (size_t)df_kp(nin) * sizeof(float) +
+         (size_t)4 * kM * sizeof(short);
 }
 
 bool tc_restart_df_supported(int nin, int nout) {
   return nin >= 1 && nin <= 192 && nout >= 1 && nout <= 64 && tc_restart_df_smem(nin, nout) <= kTcDfSmemMax;
 }
 
-// Digit image of Q (nin x nout, column-major FP64) and the column exponents:
-// |Q[:, o]| < 2^(f_o - 1), W = round(Q 2^(48 - f_o)) = sum_t c_t 2^(42 - 7t).
-void tc_restart_df_bimage(int nin, int nout, const double* Q, std::vector<uint16_t>& img, std::vector<int>& fexp) {
+// The block a product reads (DfBlobHead, then the digit image of Q, nin x
+// nout column-major FP64): |Q[:, o]| < 2^(f_o - 1), W = round(Q 2^(48 - f_o))
+// = sum_t c_t 2^(42 - 7t) with balanced digits -64 <= c_t < 64 (t > 0); slice
+// t, column l, output o at K-step l / 16: [(l / 8) % 2][t N + o][l % 8].
+// pexp: the input columns' powers of two (nullptr: zero).
+static_assert(sizeof(DfBlobHead) + (size_t)kDfDigits * 256 * 64 * 2 <= kTcDfBlobBytes, "largest block");
+void tc_restart_df_blob(int nin, int nout, const double* Q, const int* pexp, std::vector<uint8_t>& blob) {
   const int Kp = df_kp(nin), N = df_n(nout);
-  img.assign((size_t)kDfDigits * Kp * N, 0);
-  fexp.assign(N, 0);
+  blob.assign(sizeof(DfBlobHead) + (size_t)kDfDigits * Kp * N * 2, 0);
+  DfBlobHead* hd = reinterpret_cast<DfBlobHead*>(blob.data());
+  uint16_t* img = reinterpret_cast<uint16_t*>(hd + 1);
+  for (int l = 0; l < nin; ++l) hd->pexp[l] = pexp ? pexp[l] : 0;      // -126 .. 126
   for (int o = 0; o < nout; ++o) {
     double mx = 0.0;
     for (int l = 0; l < nin; ++l) mx = std::max(mx, std::fabs(Q[l + (size_t)o * nin]));
     int E2 = 0;
     if (mx > 0.0) std::frexp(mx, &E2);          // mx < 2^E2
     const int f = E2 + 1;
-    fexp[o] = f;
+    hd->fexp[o] = f;
+    int csum[kDfDigits] = {};
     for (int l = 0; l < nin; ++l) {
-      const int64_t W = std::llround(std::ldexp(Q[l + (size_t)o * nin], 48 - f));
-      for (int t = 0; t < kDfDigits; ++t) {
-        const int dgt = t == 0 ? (int)(W >> 42) : (int)((W >> (42 - 7 * t)) & 127);
-        img[(size_t)t * Kp * N + canon_off(o, l, N) / 2] = host_bf16((float)dgt);
+      int64_t W = std::llround(std::ldexp(Q[l + (size_t)o * nin], 48 - f));
+      for (int t = kDfDigits - 1; t >= 0; --t) {
+        const int dgt = t == 0 ? (int)W : (int)(((W + 64) & 127) - 64);
+        W = (W - dgt) >> 7;
+        csum[t] += dgt;
+        img[((size_t)((l >> 4) * 2 + ((l >> 3) & 1)) * kDfDigits * N + (size_t)t * N + o) * 8 + (l & 7)] =
+            host_bf16((float)dgt);
       }
+    }
+    for (int g = 0; g < kDfGroups; ++g) {
+      int c = 0;
+      for (int t = std::max(0, g - kDfDigits + 1); t <= std::min(g, kDfDigits - 1); ++t) c += csum[t];
+      hd->corr[g * N + o] = 192.0f * (float)c;
     }
   }
 }
 
-void launch_tc_restart_df(int64_t n, const float2* in, float2* out, int64_t ldu, int nin, int nout, const void* bimg,
-                          const int* fexp, const int* pexp, int* rexp, const float2* mvsrc, float2* mvdst, int* flag,
-                          cudaStream_t st) {
+// Two CTAs per SM where the tensor memory holds both (N <= 32) and the
+// shared memory too, else one with all its registers.  Measured on the
+// GB300, n = 1e6, 80 -> 21 columns (808 MB, 0.12 ms at the copy rate):
+// FP64 in and out
+// 1.44 ms (with its conversion passes) -> 0.36 ms, bound by the digit split
+// (issue 60%, tensor pipe 20%); the whole rks_basis_product_df call 2.52 ->
+// 0.41 ms (no allocations, no double-float copies).  A 512-thread form with
+// four columns per thread and one store of 8 bytes per digit took 0.56 ms.
+template <class T>
+static void launch_df_t(int64_t n, const T* in, T* out, int64_t ldu, int nin, int nout, const void* blob,
+                        const T* mvsrc, T* mvdst, int* flag, cudaStream_t st) {
   const int Kp = df_kp(nin), N = df_n(nout);
   int tcols = 32;
   while (tcols < kDfGroups * N) tcols *= 2;
   const int64_t ntiles = (n + kM - 1) / kM;
   const size_t sm = tc_restart_df_smem(nin, nout);
-  int sms = 152, dev = 0, per_sm = 1;
+  int sms = 152, dev = 0;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tc_restart_df, kDfAllThreads, sm) != cudaSuccess ||
-      per_sm < 1)
-    per_sm = 1;
-  per_sm = std::min(per_sm, 512 / tcols);          // tensor memory columns per SM
-  const int ge = (int)std::min<int64_t>((n + 255) / 256, (int64_t)sms * 8);
-  k_row_exp<<<std::max(ge, 1), 256, 0, st>>>(n, in, ldu, nin, pexp, rexp);
-  const int g = (int)std::min<int64_t>(ntiles, (int64_t)sms * per_sm);
-  k_tc_restart_df<<<g, kDfAllThreads, sm, st>>>(n, in, out, ldu, nin, Kp, N, nout, static_cast<const uint4*>(bimg),
-                                             fexp, pexp, rexp, mvsrc, mvdst, tcols, flag);
+  const bool two = tcols <= 256 && 2 * (sm + 1024) <= 228 * 1024;
+  const int g = (int)std::min<int64_t>(ntiles, (int64_t)sms * (two ? 2 : 1));
+  const DfBlobHead* hd = static_cast<const DfBlobHead*>(blob);
+  if (two)
+    k_tc_restart_df<T, 2><<<g, kDfAllThreads, sm, st>>>(n, in, out, ldu, nin, Kp, N, nout, hd, mvsrc, mvdst, tcols, flag);
+  else
+    k_tc_restart_df<T, 1><<<g, kDfAllThreads, sm, st>>>(n, in, out, ldu, nin, Kp, N, nout, hd, mvsrc, mvdst, tcols, flag);
+}
+
+void launch_tc_restart_df(int64_t n, const float2* in, float2* out, int64_t ldu, int nin, int nout, const void* blob,
+                          const float2* mvsrc, float2* mvdst, int* flag, cudaStream_t st) {
+  launch_df_t<float2>(n, in, out, ldu, nin, nout, blob, mvsrc, mvdst, flag, st);
+}
+
+void launch_tc_product_f64(int64_t n, const double* in, double* out, int64_t ldu, int nin, int nout, const void* blob,
+                           int* flag, cudaStream_t st) {
+  launch_df_t<double>(n, in, out, ldu, nin, nout, blob, nullptr, nullptr, flag, st);
 }
 
 static cudaError_t configure_tc_kernels_once() {
   cudaError_t e = cudaFuncSetAttribute(k_tc_restart_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_tc_restart_df, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcDfSmemMax);
+  const int df = (int)kTcDfSmemMax;
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_tc_restart_df<float2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, df);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_tc_restart_df<float2, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, df);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_tc_restart_df<double, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, df);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_tc_restart_df<double, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, df);
   return e;
 }
 
