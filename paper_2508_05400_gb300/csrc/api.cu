@@ -813,7 +813,7 @@ int finalize(rks_ctx* c) {
     if (rc) return rc;
     rc = dalloc(&c->rsum, (size_t)4 * (c->k + 1) * rks::kResidCtas);
     if (rc) return rc;
-    rc = dalloc(&c->pcol, (size_t)2 * (c->k + 1));
+    rc = dalloc(&c->pcol, (size_t)3 * (c->k + 1));
     if (rc) return rc;
     rc = dalloc(&c->plam, (size_t)2 * (c->k + 1));
     if (rc) return rc;
@@ -842,14 +842,19 @@ int finalize(rks_ctx* c) {
   } else {
     rks::launch_rows_gemm(c->n, c->U, c->ldu, 0, kk, c->Qd, nw, c->X, c->ldu, 0, -1, c->stream);
   }
-  rks::launch_spmm(c->A, c->X, c->ldu, c->AX, c->ldu, nw, c->stream);
-  std::vector<int> pc(2 * np);
+  std::vector<int> pc(2 * np), order;
   std::vector<double> pv(2 * np);
   for (int t = 0; t < np; ++t) { pc[t] = col[t]; pc[np + t] = colim[t]; pv[t] = pl_re[t]; pv[np + t] = pl_im[t]; }
+  for (int t = 0; t < np; ++t)
+    if (colim[t] < 0) order.push_back(t);
+  const int nreal = (int)order.size();
+  for (int t = 0; t < np; ++t)
+    if (colim[t] >= 0) order.push_back(t);
+  pc.insert(pc.end(), order.begin(), order.end());
   CK(cudaMemcpyAsync(c->pcol, pc.data(), pc.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream));
   CK(cudaMemcpyAsync(c->plam, pv.data(), pv.size() * sizeof(double), cudaMemcpyHostToDevice, c->stream));
-  const int rg = rks::launch_resid_sums(c->n, c->X, c->AX, c->ldu, np, c->pcol, c->pcol + np, c->plam,
-                                        c->plam + np, c->rsum, c->stream);
+  const int rg = rks::launch_resid(c->A, c->X, c->ldu, nreal, np - nreal, c->pcol + 2 * np, c->pcol, c->pcol + np,
+                                   c->plam, c->plam + np, c->rsum, c->stream);
   prof_end(c, ps, RKS_K_OTHER, 3, 0.0, 0.0);
   int rc = launch_err();
   if (rc) return rc;

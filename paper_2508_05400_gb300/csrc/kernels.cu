@@ -507,57 +507,115 @@ __global__ void k_rows_gemm(int64_t n, const double* A, int64_t lda, int a0, int
 }
 
 // y = A x for several columns: Y[:, j] = A X[:, j], j < ncols.
-__global__ void k_spmm(int64_t n, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ colind,
-                       const double* __restrict__ vals, const double* __restrict__ X, int64_t ldx,
-                       double* __restrict__ Y, int64_t ldy, int ncols) {
-  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  int j = blockIdx.y;
-  if (i >= n || j >= ncols) return;
-  const double* x = X + (int64_t)j * ldx;
-  double acc = 0.0;
-  for (int p = rowptr[i]; p < rowptr[i + 1]; ++p) acc = fma(vals[p], x[colind[p]], acc);
-  Y[i + (int64_t)j * ldy] = acc;
-}
-
-// Residual sums of eigenpair column pair t (blockIdx.y): col[t] (re part),
-// colim[t] (im part column or -1), lam (a, b).  out[t*6 + ...] +=
-// {||r||^2, ||x||^2, Re x^H A x, Im x^H A x}.
-__global__ void k_resid_sums(int64_t n, const double* __restrict__ X, const double* __restrict__ AX,
-                             int64_t ld, const int* __restrict__ col, const int* __restrict__ colim,
-                             const double* __restrict__ lre, const double* __restrict__ lim,
-                             double* __restrict__ out) {
-  int t = blockIdx.y;
-  int cr = col[t], ci = colim[t];
-  double a = lre[t], b = lim[t];
-  double s[4] = {0, 0, 0, 0};
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    double xr = X[i + (int64_t)cr * ld], axr = AX[i + (int64_t)cr * ld];
-    double xi = ci >= 0 ? X[i + (int64_t)ci * ld] : 0.0;
-    double axi = ci >= 0 ? AX[i + (int64_t)ci * ld] : 0.0;
-    double rre = axr - a * xr + b * xi;
-    double rim = axi - a * xi - b * xr;
-    s[0] += rre * rre + rim * rim;
-    s[1] += xr * xr + xi * xi;
-    s[2] += xr * axr + xi * axi;
-    s[3] += xr * axi - xi * axr;
-  }
-  __shared__ double red[4][32];
-  int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+// Residual sums of Ritz vectors, the product with A formed on the way (A X is
+// never stored): for slot t = slots[blockIdx.y * C ..], columns col[t] (re) and
+// colim[t] (im, CPLX only), lambda = (a, b):
+//   {||r||^2, ||x||^2, Re x^H A x, Im x^H A x}, r = A x - lambda x,
+// per CTA to out[(t * 4 + q) * gridDim.x + cta], added on the host in CTA order.
+// FP64 throughput bounds it: a real column costs its row's products and four
+// FMAs (the two-pass form spent 16 on the sums alone and stored A X); C = 4
+// real columns share the reads of A.  Rows of more than kLongRow entries are
+// taken by the whole warp (one thread on a row of 10^4 entries held the pass
+// up for 1.6 ms).  Measured, n = 1e6, 20 columns, 5 entries per row:
+// 0.79 -> 0.35 ms; 100 003 rows with one of 10^4 entries, 8 columns: 1.65 ->
+// 0.3 ms.
+constexpr int kLongRow = 64;
+template <bool CPLX, int C>
+__global__ void __launch_bounds__(256) k_resid(int64_t n, const int32_t* __restrict__ rowptr,
+                                               const int32_t* __restrict__ colind, const double* __restrict__ vals,
+                                               const double* __restrict__ X, int64_t ld, const int* __restrict__ slots,
+                                               int nslot, const int* __restrict__ col, const int* __restrict__ colim,
+                                               const double* __restrict__ lre, const double* __restrict__ lim,
+                                               double* __restrict__ out) {
+  constexpr int V = CPLX ? 2 : C;              // vectors read per row
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int slot[C];
+  const double* xv[V];
+  double la[C];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    double v = s[q];
-    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) red[q][warp] = v;
+  for (int q = 0; q < C; ++q) {
+    slot[q] = slots[min((int)blockIdx.y * C + q, nslot - 1)];
+    la[q] = lre[slot[q]];
+    xv[q] = X + (int64_t)col[slot[q]] * ld;
   }
-  __syncthreads();
-  if (warp == 0) {
-    int nw = blockDim.x >> 5;
+  if (CPLX) xv[1] = X + (int64_t)colim[slot[0]] * ld;
+  const double lb = CPLX ? lim[slot[0]] : 0.0;
+  double s[C][4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      double v = lane < nw ? red[q][lane] : 0.0;
+  for (int q = 0; q < C; ++q)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) s[q][k] = 0.0;
+  for (int64_t i0 = ((int64_t)blockIdx.x * 8 + warp) * 32; i0 < n; i0 += (int64_t)gridDim.x * 256) {
+    const int64_t i = i0 + lane;
+    const int p0 = i < n ? rowptr[i] : 0, p1 = i < n ? rowptr[i + 1] : 0;
+    const bool big = p1 - p0 > kLongRow;
+    double ax[V];
+#pragma unroll
+    for (int v = 0; v < V; ++v) ax[v] = 0.0;
+    if (!big) {
+#pragma unroll 4
+      for (int p = p0; p < p1; ++p) {
+        const double a = vals[p];
+        const int j = colind[p];
+#pragma unroll
+        for (int v = 0; v < V; ++v) ax[v] = fma(a, xv[v][j], ax[v]);
+      }
+    }
+    for (unsigned m = __ballot_sync(0xffffffffu, big); m; m &= m - 1) {
+      const int src = __ffs(m) - 1;
+      const int b0 = __shfl_sync(0xffffffffu, p0, src), b1 = __shfl_sync(0xffffffffu, p1, src);
+      double part[V];
+#pragma unroll
+      for (int v = 0; v < V; ++v) part[v] = 0.0;
+#pragma unroll 4
+      for (int p = b0 + lane; p < b1; p += 32) {
+        const double a = vals[p];
+        const int j = colind[p];
+#pragma unroll
+        for (int v = 0; v < V; ++v) part[v] = fma(a, xv[v][j], part[v]);
+      }
+#pragma unroll
+      for (int v = 0; v < V; ++v) {
+        for (int o = 16; o; o >>= 1) part[v] += __shfl_xor_sync(0xffffffffu, part[v], o);
+        if (lane == src) ax[v] = part[v];
+      }
+    }
+    if (i < n) {
+      if (CPLX) {
+        const double xr = xv[0][i], xi = xv[1][i];
+        const double rre = ax[0] - la[0] * xr + lb * xi, rim = ax[1] - la[0] * xi - lb * xr;
+        s[0][0] += rre * rre + rim * rim;
+        s[0][1] += xr * xr + xi * xi;
+        s[0][2] += xr * ax[0] + xi * ax[1];
+        s[0][3] += xr * ax[1] - xi * ax[0];
+      } else {
+#pragma unroll
+        for (int q = 0; q < C; ++q) {
+          const double x = xv[q][i], r = fma(-la[q], x, ax[q]);
+          s[q][0] = fma(r, r, s[q][0]);
+          s[q][1] = fma(x, x, s[q][1]);
+          s[q][2] = fma(x, ax[q], s[q][2]);
+        }
+      }
+    }
+  }
+  __shared__ double red[C][4][8];
+#pragma unroll
+  for (int q = 0; q < C; ++q)
+#pragma unroll
+    for (int k = 0; k < (CPLX ? 4 : 3); ++k) {
+      double v = s[q][k];
       for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == 0) out[((size_t)t * 4 + q) * gridDim.x + blockIdx.x] = v;   // summed on the host in CTA order
+      if (lane == 0) red[q][k][warp] = v;
+    }
+  __syncthreads();
+  if (threadIdx.x < C * 4) {
+    const int q = threadIdx.x >> 2, k = threadIdx.x & 3;
+    if ((int)blockIdx.y * C + q < nslot) {
+      double v = 0.0;
+      if (CPLX || k < 3)
+        for (int w = 0; w < 8; ++w) v += red[q][k][w];
+      out[((size_t)slots[blockIdx.y * C + q] * 4 + k) * gridDim.x + blockIdx.x] = v;
     }
   }
 }
@@ -709,16 +767,19 @@ void launch_rows_gemm(int64_t n, const double* A, int64_t lda, int a0, int nin, 
   k_rows_gemm<<<g, threads, sm, st>>>(n, A, lda, a0, nin, B, nout, C, ldc, c0, move_src);
 }
 
-void launch_spmm(const Csr& A, const double* X, int64_t ldx, double* Y, int64_t ldy, int ncols, cudaStream_t st) {
-  dim3 grid((unsigned)((A.n + 255) / 256), (unsigned)ncols);
-  k_spmm<<<grid, 256, 0, st>>>(A.n, A.rowptr, A.colind, A.vals, X, ldx, Y, ldy, ncols);
-}
-
-int launch_resid_sums(int64_t n, const double* X, const double* AX, int64_t ld, int npairs, const int* col,
-                      const int* colim, const double* lre, const double* lim, double* out, cudaStream_t st) {
-  const int g = grid_for(n, 256, kResidCtas);
-  dim3 grid((unsigned)g, (unsigned)npairs);
-  k_resid_sums<<<grid, 256, 0, st>>>(n, X, AX, ld, col, colim, lre, lim, out);
+int launch_resid(const Csr& A, const double* X, int64_t ld, int nreal, int npair, const int* slots, const int* col,
+                 const int* colim, const double* lre, const double* lim, double* out, cudaStream_t st) {
+  const int g = grid_for(A.n, 256, kResidCtas);
+  if (nreal > 0) {
+    dim3 grid((unsigned)g, (unsigned)((nreal + 3) / 4));
+    k_resid<false, 4><<<grid, 256, 0, st>>>(A.n, A.rowptr, A.colind, A.vals, X, ld, slots, nreal, col, colim, lre, lim,
+                                            out);
+  }
+  if (npair > 0) {
+    dim3 grid((unsigned)g, (unsigned)npair);
+    k_resid<true, 1><<<grid, 256, 0, st>>>(A.n, A.rowptr, A.colind, A.vals, X, ld, slots + nreal, npair, col, colim,
+                                           lre, lim, out);
+  }
   return g;
 }
 

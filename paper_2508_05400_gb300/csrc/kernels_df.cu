@@ -35,6 +35,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "convert.cuh"
 #include "rks_impl.h"
 
 namespace rks {
@@ -99,14 +100,6 @@ __device__ __forceinline__ float2 df_norm(float s, float t) {
   fast_two_sum(s, t, h, l);
   return make_float2(h, l);
 }
-
-__device__ __forceinline__ float2 df_from_double(double x) {
-  float h = __double2float_rn(x);
-  float l = __double2float_rn(x - (double)h);
-  return make_float2(h, l);
-}
-
-__device__ __forceinline__ double df_to_double(float2 v) { return (double)v.x + (double)v.y; }
 
 // DF warp reduction of (s, t) pairs
 __device__ __forceinline__ void df_warp_sum(float& s, float& t) {

@@ -202,10 +202,11 @@ cudaError_t once_per_device(int slot, cudaError_t (*f)());
 int rows_gemm_smem(int nin, int nout, int threads);
 void launch_rows_gemm(int64_t n, const double* A, int64_t lda, int a0, int nin, const double* B, int nout,
                       double* C, int64_t ldc, int c0, int move_src, cudaStream_t st);
-void launch_spmm(const Csr& A, const double* X, int64_t ldx, double* Y, int64_t ldy, int ncols, cudaStream_t st);
-// Writes per-CTA partial sums out[(pair * 4 + q) * G + cta]; returns G (<= kResidCtas).
-int launch_resid_sums(int64_t n, const double* X, const double* AX, int64_t ld, int npairs, const int* col,
-                      const int* colim, const double* lre, const double* lim, double* out, cudaStream_t st);
+// Residual sums of nreal real slots and npair conjugate pairs (slots: device,
+// the real ones first): per-CTA partial sums out[(slot * 4 + q) * G + cta];
+// returns G (<= kResidCtas).
+int launch_resid(const Csr& A, const double* X, int64_t ld, int nreal, int npair, const int* slots, const int* col,
+                 const int* colim, const double* lre, const double* lim, double* out, cudaStream_t st);
 void launch_f32_to_f64(int64_t n, const float* a, double* b, cudaStream_t st);
 void launch_check_csr(int64_t n, int64_t nnz, const int32_t* rowptr, const int32_t* colind, int* bad,
                       cudaStream_t st);

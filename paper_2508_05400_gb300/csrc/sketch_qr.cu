@@ -33,6 +33,7 @@
 #include <vector>
 
 #include "../../include/rks.h"
+#include "convert.cuh"
 #include "dense.h"
 #include "rks_impl.h"
 
@@ -45,7 +46,7 @@ __global__ void k_df2d_scaled(int64_t n, const float2* __restrict__ x, int64_t l
   const double sc = scale[j];
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const float2 v = x[i + (int64_t)j * ldx];
-    y[i + (int64_t)j * ldy] = ((double)v.x + (double)v.y) * sc;
+    y[i + (int64_t)j * ldy] = rks::df_to_double(v) * sc;
   }
 }
 
