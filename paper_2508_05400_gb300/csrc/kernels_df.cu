@@ -1213,13 +1213,14 @@ __device__ __forceinline__ double fold_row(const double* __restrict__ part, int 
   return v;
 }
 
-// out = the CTA-ordered sum of the sketch kernels' partials (warp per row)
+// out = the CTA-ordered sum of the sketch kernels' partials (warp per row;
+// blockIdx.y: several vectors, G x d partials and d sums each)
 __global__ void __launch_bounds__(256) k_df_fold(const double* __restrict__ part, int d, int G,
                                                  double* __restrict__ out) {
   const int r = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (r >= d) return;
-  const double v = fold_row(part, d, G, r, lane);
-  if (lane == 0) out[r] = v;
+  const double v = fold_row(part + (size_t)blockIdx.y * G * d, d, G, r, lane);
+  if (lane == 0) out[(size_t)blockIdx.y * d + r] = v;
 }
 
 // Least squares b = S^+ z of one Arnoldi step (Alg. 2, Thm 4.3: against the
@@ -1593,6 +1594,14 @@ __global__ void k_d2df(int64_t n, const double* __restrict__ x, TU* __restrict__
     stv(y + i, df_from_double(x[i]));
 }
 
+__global__ void k_d2df_cols(int64_t n, const double* __restrict__ x, int64_t ldx, float2* __restrict__ y,
+                            int64_t ldy) {
+  const int j = blockIdx.y;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x)
+    y[i + (int64_t)j * ldy] = df_from_double(x[i + (int64_t)j * ldx]);
+}
+
 // stored columns -> FP64 columns (ncols, with leading dimensions)
 template <class TU>
 __global__ void k_df2d_cols(int64_t n, const TU* __restrict__ x, int64_t ldx, double* __restrict__ y,
@@ -1627,6 +1636,156 @@ __global__ void __launch_bounds__(512) k_df_sketch_vec(const TU* __restrict__ x,
     tile_gather<sizeof(TU) == 8>(d, tv.H, v, of, ms, es, acc);
   }
   tile_write_part(acc, d, part);
+}
+
+// part[col][cta] = the CTA's Omega-sums of column col, for a block of columns
+// given in FP64 or double-float; with U, the double-float columns are also
+// written there.  A CTA takes up to NC columns (grid.y the others), so that a
+// tile's bin lists (16 bytes a row, twice a column's bytes) are staged once
+// for NC columns, and FP64 input is converted on the way: a launch, a
+// conversion pass and a staging per column took 36 us a column at n = 1e6,
+// d = 320; here 14 us.  The next column's values are loaded while one is
+// summed; the sums are those of k_df_sketch_vec.
+constexpr int kSkCols = kPanelCols;
+template <class TS>
+__global__ void __launch_bounds__(512, 2) k_df_sketch_cols(const TS* __restrict__ x, int64_t ldx, int ncols, int nc,
+                                                           float2* __restrict__ U, int64_t ldu, const SketchTiles tv,
+                                                           double* __restrict__ part) {
+  extern __shared__ __align__(16) uint8_t smraw[];
+  const int d = tv.d, L1 = tv.L + 1;
+  float2* vb = reinterpret_cast<float2*>(smraw);                             // two value buffers
+  uint16_t* es = reinterpret_cast<uint16_t*>(vb + 2 * kTileRows);
+  uint32_t* ms = reinterpret_cast<uint32_t*>(es + (size_t)kTileRows * tv.zeta);
+  int* of = reinterpret_cast<int*>(ms + d);
+  float2* acc = reinterpret_cast<float2*>(of + L1 + (L1 + d & 1));           // nc x d
+  const int q0 = blockIdx.y * nc, nq = min(nc, ncols - q0);
+  for (int r = threadIdx.x; r < nq * d; r += blockDim.x) acc[r] = make_float2(0.f, 0.f);
+  x += (int64_t)q0 * ldx;
+  if (U) U += (int64_t)q0 * ldu;
+  const int la = threadIdx.x, lb = threadIdx.x + 512;
+  const int t0 = tv.ctile[blockIdx.x], t1 = tv.ctile[blockIdx.x + 1];
+  auto as_df = [](TS v) {
+    if constexpr (std::is_same<TS, double>::value) return df_from_double(v);
+    else return v;
+  };
+  for (int t = t0; t < t1; ++t) {
+    const int64_t r0 = tv.row[t];
+    const int rows = (int)(tv.row[t + 1] - r0);
+    const TS* xt = x + r0;
+    TS a{}, b{};
+    if (la < rows) a = xt[la];
+    if (lb < rows) b = xt[lb];
+    __syncthreads();                               // the last tile's lists and values are read
+    tile_stage(tv, t, r0, rows, of, ms, es);
+    for (int q = 0; q < nq; ++q) {
+      float2* v = vb + (q & 1) * kTileRows;
+      const float2 da = as_df(a), db = as_df(b);
+      v[la] = da;
+      v[lb] = db;
+      if (U) {
+        if (la < rows) U[(int64_t)q * ldu + r0 + la] = da;
+        if (lb < rows) U[(int64_t)q * ldu + r0 + lb] = db;
+      }
+      if (q + 1 < nq) {
+        const TS* xn = xt + (int64_t)(q + 1) * ldx;
+        if (la < rows) a = xn[la];
+        if (lb < rows) b = xn[lb];
+      }
+      __syncthreads();
+      tile_gather<true>(d, tv.H, v, of, ms, es, acc + (size_t)q * d);
+    }
+  }
+  __syncthreads();
+  for (int r = threadIdx.x; r < nq * d; r += blockDim.x) {
+    const int q = r / d, i = r - q * d;
+    part[((size_t)(q0 + q) * gridDim.x + blockIdx.x) * d + i] = df_to_double(acc[r]);
+  }
+}
+
+// U[:, p0 + k] += sum_{c < c0} U[:, c] coef[c * kSkCols + k] for k < nb <= kSkCols
+// (double-float): a panel of columns updated by all earlier ones in one pass
+// over them, where a column at a time read them once per column.  Two rows
+// per thread; a column's terms are added in the order of k_df_update_sketch.
+// Bound by the FP32 pipes (12 operations per double-float multiply-add).  The
+// 80-column RGS at n = 1e6: 5.5 ms of updates -> 1.5 ms here and 2.5 ms of
+// updates inside the panels.
+__global__ void __launch_bounds__(256, 2) k_df_panel(int64_t n, float2* __restrict__ U, int64_t ldu, int c0, int p0,
+                                                     int nb, const float2* __restrict__ coef) {
+  extern __shared__ __align__(16) float2 cs[];     // c0 x kSkCols
+  for (int t = threadIdx.x; t < c0 * kSkCols; t += blockDim.x) cs[t] = coef[t];
+  __syncthreads();
+  for (int64_t i = 2 * (blockIdx.x * (int64_t)blockDim.x + threadIdx.x); i < n;
+       i += 2 * (int64_t)gridDim.x * blockDim.x) {
+    float s[2][kSkCols], t[2][kSkCols];
+#pragma unroll
+    for (int k = 0; k < kSkCols; ++k) {
+      float2 a = make_float2(0.f, 0.f), b = a;
+      if (k < nb) ld2(U + i + (int64_t)(p0 + k) * ldu, a, b);
+      s[0][k] = a.x; t[0][k] = a.y;
+      s[1][k] = b.x; t[1][k] = b.y;
+    }
+#pragma unroll 4
+    for (int c = 0; c < c0; ++c) {
+      float2 a, b;
+      ld2(U + i + (int64_t)c * ldu, a, b);
+#pragma unroll
+      for (int k = 0; k < kSkCols; ++k) {
+        const float2 r = cs[c * kSkCols + k];
+        df_mac(a.x, a.y, r.x, r.y, s[0][k], t[0][k]);
+        df_mac(b.x, b.y, r.x, r.y, s[1][k], t[1][k]);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < kSkCols; ++k)
+      if (k < nb) {
+        float2* p = U + i + (int64_t)(p0 + k) * ldu;
+        p[0] = df_norm(s[0][k], t[0][k]);
+        if (i + 1 < n) p[1] = df_norm(s[1][k], t[1][k]);
+      }
+  }
+}
+
+// Gram matrix of s double-float columns, upper triangle in 4 x 4 blocks:
+// part[cta * npair + p], p = the block's number * 16 + 4 i + j, holds the CTA's
+// sum of column (4 bi + i) times column (4 bj + j).  A block reads 8 columns
+// for 16 products where a product per column pair read one for one.
+__global__ void __launch_bounds__(256) k_df_gram(const float2* __restrict__ U, int64_t ldu, int64_t n, int s,
+                                                 double* __restrict__ part, int npair) {
+  __shared__ float2 red[8][16];
+  int bj = 0, q = blockIdx.y;
+  while (q > bj) { q -= bj + 1; ++bj; }            // block (bi = q, bj), bi <= bj
+  const int bi = q;
+  const float2 *pa[4], *pb[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    pa[u] = U + (int64_t)min(4 * bi + u, s - 1) * ldu;
+    pb[u] = U + (int64_t)min(4 * bj + u, s - 1) * ldu;
+  }
+  float sh[16], sl[16];
+#pragma unroll
+  for (int u = 0; u < 16; ++u) { sh[u] = 0.f; sl[u] = 0.f; }
+  const int64_t per = (n + gridDim.x - 1) / gridDim.x, r0 = blockIdx.x * per, r1 = min(n, r0 + per);
+  for (int64_t i = r0 + threadIdx.x; i < r1; i += blockDim.x) {
+    float2 a[4], b[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) { a[u] = pa[u][i]; b[u] = pb[u][i]; }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int v = 0; v < 4; ++v) df_mac(a[u].x, a[u].y, b[v].x, b[v].y, sh[4 * u + v], sl[4 * u + v]);
+  }
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int u = 0; u < 16; ++u) {
+    df_warp_sum(sh[u], sl[u]);
+    if (lane == 0) red[warp][u] = df_norm(sh[u], sl[u]);
+  }
+  __syncthreads();
+  if (threadIdx.x < 16) {
+    double v = 0.0;
+    for (int w = 0; w < 8; ++w) v += df_to_double(red[w][threadIdx.x]);
+    part[(size_t)blockIdx.x * npair + blockIdx.y * 16 + threadIdx.x] = v;
+  }
 }
 
 // U[i, c0 + l] -= coef[l] * U[i, src] for l < ncols (double-float): one
@@ -1899,6 +2058,7 @@ static cudaError_t configure_df_kernels_once() {
   RKS_SMEM((k_df_update_sketch<float2, U8, MB, 1>)); RKS_SMEM((k_df_update_sketch<float, 2 * U8, MB, 1>));
   RKS_SMEM((k_df_update_sketch<float2, U8, MB, 0>)); RKS_SMEM((k_df_update_sketch<float2, U8, MB, 2>));
   RKS_SMEM(k_df_sketch_vec<float2>); RKS_SMEM(k_df_sketch_vec<float>);
+  RKS_SMEM(k_df_sketch_cols<float2>); RKS_SMEM(k_df_sketch_cols<double>); RKS_SMEM(k_df_panel);
   RKS_SMEM(k_tiles_count<4>); RKS_SMEM(k_tiles_count<8>); RKS_SMEM(k_tiles_count<16>);
   RKS_SMEM(k_tiles_build<4>); RKS_SMEM(k_tiles_build<8>); RKS_SMEM(k_tiles_build<16>);
   RKS_SMEM(k_df_ls1);
@@ -2076,8 +2236,41 @@ void launch_df_update_plain(void* U, int64_t ldu, int c, const float2* nrs, cons
   else k_df_update_sketch<float2, U8, MB, 0><<<t.G, 512, sm, st>>>(u, ldu, c, nrs, sj, t, nullptr);
 }
 
-void launch_df_fold(const double* part, int d, int G, double* out, cudaStream_t st) {
-  k_df_fold<<<(d + 7) / 8, 256, 0, st>>>(part, d, G, out);
+void launch_df_fold(const double* part, int d, int G, double* out, cudaStream_t st, int nvec) {
+  k_df_fold<<<dim3((d + 7) / 8, nvec), 256, 0, st>>>(part, d, G, out);
+}
+
+template <class TS>
+static void sketch_cols_t(const TS* x, int64_t ldx, int ncols, float2* U, int64_t ldu, const SketchTiles& t,
+                          double* part, cudaStream_t st) {
+  const size_t fixed = (size_t)2 * kTileRows * sizeof(float2) + (size_t)kTileRows * t.zeta * sizeof(uint16_t) +
+                       (size_t)(t.d + t.L + 2) * sizeof(int) + 16;
+  // columns per CTA: as many accumulators as two CTAs per SM leave room for
+  const size_t room = 100 * 1024 > fixed ? 100 * 1024 - fixed : 0;
+  const int nc = (int)std::min<size_t>({(size_t)kSkCols, (size_t)ncols,
+                                        std::max<size_t>(1, room / ((size_t)t.d * sizeof(float2)))});
+  k_df_sketch_cols<TS><<<dim3(t.G, (ncols + nc - 1) / nc), 512, fixed + (size_t)nc * t.d * sizeof(float2), st>>>(
+      x, ldx, ncols, nc, U, ldu, t, part);
+}
+void launch_df_sketch_cols(const float2* x, int64_t ldx, int ncols, const SketchTiles& t, double* part,
+                           cudaStream_t st) {
+  sketch_cols_t<float2>(x, ldx, ncols, nullptr, 0, t, part, st);
+}
+void launch_sketch_cols_f64(const double* x, int64_t ldx, int ncols, float2* U, int64_t ldu, const SketchTiles& t,
+                            double* part, cudaStream_t st) {
+  sketch_cols_t<double>(x, ldx, ncols, U, ldu, t, part, st);
+}
+
+void launch_df_panel(int64_t n, float2* U, int64_t ldu, int c0, int p0, int nb, const float2* coef, cudaStream_t st) {
+  const int g = (int)std::min<int64_t>((n + 511) / 512, 152 * 2);
+  k_df_panel<<<g, 256, (size_t)c0 * kSkCols * sizeof(float2), st>>>(n, U, ldu, c0, p0, nb, coef);
+}
+
+int gram_ctas(int64_t n) { return (int)std::max<int64_t>(1, std::min<int64_t>(152, (n + 1023) / 1024)); }
+int gram_pairs(int s) { const int b = (s + 3) / 4; return b * (b + 1) / 2 * 16; }
+void launch_df_gram(int64_t n, const float2* U, int64_t ldu, int s, double* part, cudaStream_t st) {
+  const int npair = gram_pairs(s);
+  k_df_gram<<<dim3(gram_ctas(n), npair / 16), 256, 0, st>>>(U, ldu, n, s, part, npair);
 }
 
 void launch_df_dots(const void* U, int64_t ldu, int c, int cv, const SketchTiles& t, double* part, cudaStream_t st) {
@@ -2159,6 +2352,10 @@ void launch_sum_cols_f32(int64_t n, const float* U, int64_t ldu, int ncols, doub
 void launch_d2df(int64_t n, const double* x, void* y, bool f32, cudaStream_t st) {
   if (f32) k_d2df<float><<<df_grid(n, 256) * 2, 256, 0, st>>>(n, x, static_cast<float*>(y));
   else k_d2df<float2><<<df_grid(n, 256) * 2, 256, 0, st>>>(n, x, static_cast<float2*>(y));
+}
+
+void launch_d2df_cols(int64_t n, const double* x, int64_t ldx, float2* y, int64_t ldy, int ncols, cudaStream_t st) {
+  k_d2df_cols<<<dim3((unsigned)df_grid(n, 256), (unsigned)ncols), 256, 0, st>>>(n, x, ldx, y, ldy);
 }
 
 void launch_df2d_cols(int64_t n, const void* x, int64_t ldx, double* y, int64_t ldy, int ncols, bool f32,

@@ -115,8 +115,21 @@ void launch_df_spmv(const CsrDF& A, const void* x, void* w, const SketchTiles& t
 void launch_df_update_plain(void* U, int64_t ldu, int c, const float2* nrs, const float2* sj, const SketchTiles& t,
                             double* norm_part, cudaStream_t st);
 void launch_df_dots(const void* U, int64_t ldu, int c, int cv, const SketchTiles& t, double* part, cudaStream_t st);
-// out[r] = sum over g < G of part[g * d + r] in a fixed order (r < d)
-void launch_df_fold(const double* part, int d, int G, double* out, cudaStream_t st);
+// out[v * d + r] = sum over g < G of part[(v * G + g) * d + r] in a fixed order (r < d, v < nvec)
+void launch_df_fold(const double* part, int d, int G, double* out, cudaStream_t st, int nvec = 1);
+// Blocks of columns (kernels_df.cu): per-CTA partial sketches part[col][G][d]
+// of ncols columns (the FP64 form also writes them to U in double-float); a
+// panel U[:, p0 .. p0+nb) += U[:, 0 .. c0) coef (coef: c0 x 8 device, nb <= 8);
+// the Gram matrix of s columns (gram_ctas(n) x gram_pairs(s) partials).
+constexpr int kPanelCols = 8;
+void launch_df_sketch_cols(const float2* x, int64_t ldx, int ncols, const SketchTiles& t, double* part,
+                           cudaStream_t st);
+void launch_sketch_cols_f64(const double* x, int64_t ldx, int ncols, float2* U, int64_t ldu, const SketchTiles& t,
+                            double* part, cudaStream_t st);
+void launch_df_panel(int64_t n, float2* U, int64_t ldu, int c0, int p0, int nb, const float2* coef, cudaStream_t st);
+int gram_ctas(int64_t n);
+int gram_pairs(int s);
+void launch_df_gram(int64_t n, const float2* U, int64_t ldu, int s, double* part, cudaStream_t st);
 // U[:, c0 + l] -= coef[l] * U[:, src], l < ncols (double-float columns, coef device)
 void launch_df_axpy_cols(int64_t n, float2* U, int64_t ldu, int src, int c0, int ncols, const float2* coef,
                          cudaStream_t st);
@@ -130,6 +143,7 @@ size_t sketch_tile_smem(const SketchTiles& t, int c);
 void launch_omega_table(int64_t n, int d, int zeta, uint64_t seed, uint16_t* tab, int* flag, cudaStream_t st);
 int omega_slots(int zeta);
 void launch_d2df(int64_t n, const double* x, void* y, bool f32, cudaStream_t st);
+void launch_d2df_cols(int64_t n, const double* x, int64_t ldx, float2* y, int64_t ldy, int ncols, cudaStream_t st);
 void launch_sum_cols_f32(int64_t n, const float* U, int64_t ldu, int ncols, double* y, cudaStream_t st);
 void launch_df2d_cols(int64_t n, const void* x, int64_t ldx, double* y, int64_t ldy, int ncols, bool f32,
                       cudaStream_t st);

@@ -4,10 +4,11 @@
 //
 //  * RKS_QR_RGS: randomized Gram-Schmidt, the process of Algorithm 2 without
 //    the product with A.  The sketches z_j = Omega k_j of all columns first
-//    (tile sketch kernel); per column r = S_j^T z_j with a second pass in the
-//    sketch (host, FP64: S_j is d x j),
-//    q~ = k_j - Q_j r fused with the partial sketches of q~ (the solver's
-//    update kernel), beta = ||Omega q~||.  Columns stay unscaled on the
+//    (one launch, which also converts the block); r = S_j^T z_j with a second
+//    pass in the sketch (host, FP64: S_j is d x j), q~ = k_j - Q_j r by panels
+//    of 8 columns against all earlier ones, then column by column inside the
+//    panel fused with the partial sketches of q~ (the solver's update kernel),
+//    beta = ||Omega q~||.  Columns stay unscaled on the
 //    device (their scale 1/beta goes into the next coefficients and the
 //    final conversion), as in the solver.
 //  * RKS_QR_WHITEN: sketch and whiten (the whitening of Sec. 3.3 on a whole
@@ -58,21 +59,21 @@ float2 to_df(double v) {
 // Device state of one call, freed on every exit path.
 struct QrWork {
   int64_t n = 0, ldu = 0;
-  int s = 0, d = 0, zeta = 0;
+  int s = 0, d = 0, zeta = 0, chunk = 1;
   double zscale = 0.0;
   cudaStream_t st = nullptr;
   float2* U = nullptr;        // ldu x 2s double-float columns: [0, s) and [s, 2s)
   uint16_t* otab = nullptr;
   rks::SketchTiles tiles;
   bool have_tiles = false;
-  double* part = nullptr;     // G x max(d, s) partial sums
-  double* sums = nullptr;     // s x max(d, s) folded sums (a column per sketch or dot group)
+  double* part = nullptr;     // per-CTA partial sums (G x d per column; the Gram matrix's)
+  double* sums = nullptr;     // folded sums (d per column; the Gram matrix's pairs)
   float2* Q2 = nullptr;       // s x s double-float factor
-  float2* nrs = nullptr;      // s update coefficients
+  float2* nrs = nullptr;      // update coefficients (s x 8 of a panel, or 2 s)
   float2* sj = nullptr;       // scale of the updated column
   double* scale = nullptr;    // s column scales for the output
   int* flag = nullptr;
-  std::vector<double> host;   // s x max(d, s) sums read back
+  std::vector<double> host;   // sums read back
   ~QrWork() {
     cudaFree(U); cudaFree(otab); cudaFree(part); cudaFree(sums); cudaFree(Q2); cudaFree(nrs); cudaFree(sj);
     cudaFree(scale); cudaFree(flag);
@@ -85,22 +86,23 @@ struct QrWork {
     if ((x) != cudaSuccess) return RKS_ECUDA;   \
   } while (0)
 
-// nsk: rows the sketch covers (n, or n - s for RHQR's Omega' on rows s..n-1)
-int setup(QrWork& w, int64_t n, int s, int d, int zeta, uint64_t seed, cudaStream_t st, int64_t nsk) {
+// nsk: rows the sketch covers (n, or n - s for RHQR's Omega' on rows s..n-1);
+// ncol: double-float columns (s, or 2 s for the methods that form Q beside K)
+int setup(QrWork& w, int64_t n, int s, int d, int zeta, uint64_t seed, cudaStream_t st, int64_t nsk, int ncol) {
   w.n = n; w.s = s; w.d = d; w.zeta = zeta; w.st = st;
   w.zscale = 1.0 / std::sqrt((double)zeta);
   w.ldu = (n + 31) / 32 * 32;
-  const int wide = std::max(d, s);
-  if (cudaMalloc(&w.U, (size_t)w.ldu * 2 * s * sizeof(float2)) != cudaSuccess ||
+  const size_t nsum = std::max((size_t)d * s, (size_t)rks::gram_pairs(s));
+  if (cudaMalloc(&w.U, (size_t)w.ldu * ncol * sizeof(float2)) != cudaSuccess ||
       cudaMalloc(&w.otab, (size_t)nsk * rks::omega_slots(zeta) * sizeof(uint16_t)) != cudaSuccess ||
-      cudaMalloc(&w.sums, (size_t)wide * s * sizeof(double)) != cudaSuccess ||
+      cudaMalloc(&w.sums, nsum * sizeof(double)) != cudaSuccess ||
       cudaMalloc(&w.Q2, (size_t)s * s * sizeof(float2)) != cudaSuccess ||
-      cudaMalloc(&w.nrs, (size_t)2 * s * sizeof(float2)) != cudaSuccess ||
+      cudaMalloc(&w.nrs, (size_t)rks::kPanelCols * s * sizeof(float2)) != cudaSuccess ||
       cudaMalloc(&w.sj, sizeof(float2)) != cudaSuccess ||
       cudaMalloc(&w.scale, (size_t)s * sizeof(double)) != cudaSuccess ||
       cudaMalloc(&w.flag, sizeof(int)) != cudaSuccess)
     return RKS_ENOMEM;
-  w.host.assign((size_t)wide * s, 0.0);
+  w.host.assign(nsum, 0.0);
   QK(cudaMemsetAsync(w.flag, 0, sizeof(int), st));
   rks::launch_omega_table(nsk, d, zeta, seed, w.otab, w.flag, st);
   int bad = 0;
@@ -113,7 +115,10 @@ int setup(QrWork& w, int64_t n, int s, int d, int zeta, uint64_t seed, cudaStrea
   cudaFree(w.otab);
   w.otab = nullptr;
   if (rks::sketch_tile_smem(w.tiles, s) > 200 * 1024) return RKS_EINVAL;
-  if (cudaMalloc(&w.part, (size_t)w.tiles.G * wide * sizeof(double)) != cudaSuccess) return RKS_ENOMEM;
+  // partial sketches of as many columns at a time as 256 MB hold
+  w.chunk = (int)std::max<size_t>(1, std::min<size_t>(s, ((size_t)256 << 20) / ((size_t)w.tiles.G * d * sizeof(double))));
+  const size_t npart = std::max((size_t)w.tiles.G * d * w.chunk, (size_t)rks::gram_ctas(n) * rks::gram_pairs(s));
+  if (cudaMalloc(&w.part, npart * sizeof(double)) != cudaSuccess) return RKS_ENOMEM;
   return RKS_OK;
 }
 
@@ -158,14 +163,15 @@ std::vector<double> upper_inverse(int s, const std::vector<double>& R) {
   return X;
 }
 
-// Sk (d x s) = Omega U[:, c0 .. c0+s): the sketches of s columns, folded on
-// the device one after the other (stream order protects the partials), read
-// back at once
-int sketch_block(QrWork& w, int c0, std::vector<double>& Sk) {
+// Sk (d x s) = the sketches of s columns; launch(j, m) leaves the partials of
+// columns j .. j + m - 1 in w.part
+template <class F>
+int sketches(QrWork& w, std::vector<double>& Sk, F launch) {
   const int s = w.s, d = w.d;
-  for (int j = 0; j < s; ++j) {
-    rks::launch_df_sketch_vec(col(w, c0 + j), w.tiles, w.part, false, w.st);
-    rks::launch_df_fold(w.part, d, w.tiles.G, w.sums + (size_t)j * d, w.st);
+  for (int j = 0; j < s; j += w.chunk) {
+    const int m = std::min(w.chunk, s - j);
+    launch(j, m);
+    rks::launch_df_fold(w.part, d, w.tiles.G, w.sums + (size_t)j * d, w.st, m);
   }
   QK(cudaGetLastError());
   QK(cudaMemcpyAsync(w.host.data(), w.sums, (size_t)d * s * sizeof(double), cudaMemcpyDeviceToHost, w.st));
@@ -175,10 +181,24 @@ int sketch_block(QrWork& w, int c0, std::vector<double>& Sk) {
   return RKS_OK;
 }
 
+// Sk = Omega U[row0:, c0 .. c0+s)
+int sketch_block(QrWork& w, int c0, std::vector<double>& Sk, int row0 = 0) {
+  return sketches(w, Sk, [&](int j, int m) {
+    rks::launch_df_sketch_cols(col(w, c0 + j) + row0, w.ldu, m, w.tiles, w.part, w.st);
+  });
+}
+
+// U[:, 0 .. s) = K in double-float and Sk = Omega K
+int sketch_input(QrWork& w, const double* K, int64_t ldk, std::vector<double>& Sk) {
+  return sketches(w, Sk, [&](int j, int m) {
+    rks::launch_sketch_cols_f64(K + (size_t)j * ldk, ldk, m, col(w, j), w.ldu, w.tiles, w.part, w.st);
+  });
+}
+
 // Omega K = Q_s R1 (host); U[:, s..2s) = K R1^{-1}.  Sk receives Q_s.
-int whiten(QrWork& w, std::vector<double>& R1, std::vector<double>& Sk) {
+int whiten(QrWork& w, const double* K, int64_t ldk, std::vector<double>& R1, std::vector<double>& Sk) {
   const int s = w.s, d = w.d;
-  int rc = sketch_block(w, 0, Sk);
+  int rc = sketch_input(w, K, ldk, Sk);
   if (rc) return rc;
   R1.assign((size_t)s * s, 0.0);
   rks_dense::house_qr(d, s, Sk.data(), R1.data());
@@ -187,52 +207,99 @@ int whiten(QrWork& w, std::vector<double>& R1, std::vector<double>& Sk) {
   return product(w, 0, upper_inverse(s, R1), s);
 }
 
-int rgs(QrWork& w, std::vector<double>& R, std::vector<double>& S) {
+// Randomized Gram-Schmidt by panels of kPanelCols columns: the coefficients of
+// a column against all earlier panels are its projection in the sketch, which
+// does not depend on the panel's own columns, so one pass over the earlier
+// columns updates the whole panel (they were read once per column, 26 GB at
+// n = 1e6, s = 80); inside the panel a column at a time, its sketch measured
+// after its update.  Every projection is made twice (r = S^T z,
+// r += S^T (z - S r): S is sketch-orthonormal); eight columns side by side
+// give the host loops independent sums.
+int rgs(QrWork& w, const double* K, int64_t ldk, std::vector<double>& R, std::vector<double>& S) {
+  constexpr int B = rks::kPanelCols;
   const int s = w.s, d = w.d;
   R.assign((size_t)s * s, 0.0);
   S.assign((size_t)d * s, 0.0);
-  std::vector<double> Z, zr(d), r(s), cs(s, 0.0);
-  std::vector<float2> nrs(s);
+  std::vector<double> Z, z(d), r(B), cs(s, 0.0), P((size_t)d * B), C((size_t)s * B);
+  std::vector<float2> nrs((size_t)s * B);
   const float2 one = make_float2(1.f, 0.f);
   QK(cudaMemcpyAsync(w.sj, &one, sizeof(float2), cudaMemcpyHostToDevice, w.st));
   // z_j = Omega k_j does not depend on the process: all of them at once
-  int rc = sketch_block(w, 0, Z);
+  int rc = sketch_input(w, K, ldk, Z);
   if (rc) return rc;
-  for (int j = 0; j < s; ++j) {
-    if (j > 0) {
-      // r = S_j^+ z: S_j is sketch-orthonormal; its projection twice
-      // (r1 = S^T z, r = r1 + S^T (z - S r1))
-      const double* z = &Z[(size_t)j * d];
-      std::copy(z, z + d, zr.begin());
-      for (int c = 0; c < j; ++c) {
-        const double* sc = &S[(size_t)c * d];
-        double a = 0.0;
-        for (int i = 0; i < d; ++i) a += sc[i] * z[i];
-        r[c] = a;
+  for (int p0 = 0; p0 < s; p0 += B) {
+    const int nb = std::min(B, s - p0);
+    std::fill(P.begin(), P.end(), 0.0);
+    for (int k = 0; k < nb; ++k)
+      for (int i = 0; i < d; ++i) P[(size_t)i * B + k] = Z[i + (size_t)(p0 + k) * d];
+    if (p0 > 0) {
+      std::fill(C.begin(), C.end(), 0.0);
+      for (int pass = 0; pass < 2; ++pass) {
+        std::vector<double> D((size_t)p0 * B, 0.0);
+        for (int c = 0; c < p0; ++c) {
+          const double* sc = &S[(size_t)c * d];
+          double a[B] = {};
+          for (int i = 0; i < d; ++i)
+            for (int k = 0; k < B; ++k) a[k] += sc[i] * P[(size_t)i * B + k];
+          for (int k = 0; k < B; ++k) D[(size_t)c * B + k] = a[k];
+        }
+        for (int c = 0; c < p0; ++c) {
+          const double* sc = &S[(size_t)c * d];
+          const double* dc = &D[(size_t)c * B];
+          for (int i = 0; i < d; ++i)
+            for (int k = 0; k < B; ++k) P[(size_t)i * B + k] -= sc[i] * dc[k];
+          for (int k = 0; k < B; ++k) C[(size_t)c * B + k] += dc[k];
+        }
       }
-      for (int c = 0; c < j; ++c)
-        for (int i = 0; i < d; ++i) zr[i] -= S[i + (size_t)c * d] * r[c];
-      for (int c = 0; c < j; ++c) {
-        const double* sc = &S[(size_t)c * d];
-        double a = 0.0;
-        for (int i = 0; i < d; ++i) a += sc[i] * zr[i];
-        r[c] += a;
-      }
+      for (int c = 0; c < p0; ++c)
+        for (int k = 0; k < B; ++k) {
+          if (k < nb) R[c + (size_t)(p0 + k) * s] = C[(size_t)c * B + k];
+          nrs[(size_t)c * B + k] = to_df(-C[(size_t)c * B + k] * cs[c]);
+        }
+      QK(cudaMemcpyAsync(w.nrs, nrs.data(), (size_t)p0 * B * sizeof(float2), cudaMemcpyHostToDevice, w.st));
+      rks::launch_df_panel(w.n, w.U, w.ldu, p0, p0, nb, w.nrs, w.st);
     }
-    // q~ = k_j - sum_c (q~_c / beta_c) r_c, fused with its partial sketches
-    for (int c = 0; c < j; ++c) nrs[c] = to_df(-r[c] * cs[c]);
-    if (j > 0) QK(cudaMemcpyAsync(w.nrs, nrs.data(), (size_t)j * sizeof(float2), cudaMemcpyHostToDevice, w.st));
-    rks::launch_df_update_sketch(w.U, w.ldu, j, w.nrs, w.sj, w.tiles, w.part, false, w.st);
-    rc = fold_to_host(w, d);
-    if (rc) return rc;
-    double bb = 0.0;
-    for (int i = 0; i < d; ++i) { const double v = w.host[i] * w.zscale; bb += v * v; }
-    const double beta = std::sqrt(bb);
-    if (!(beta > 0.0) || !std::isfinite(beta)) return RKS_EBREAKDOWN;
-    for (int i = 0; i < d; ++i) S[i + (size_t)j * d] = w.host[i] * w.zscale / beta;
-    for (int c = 0; c < j; ++c) R[c + (size_t)j * s] = r[c];
-    R[j + (size_t)j * s] = beta;
-    cs[j] = 1.0 / beta;
+    for (int jj = 0; jj < nb; ++jj) {
+      const int j = p0 + jj;
+      // against the panel's columns, twice
+      for (int i = 0; i < d; ++i) z[i] = P[(size_t)i * B + jj];
+      std::fill(r.begin(), r.end(), 0.0);
+      for (int pass = 0; pass < 2; ++pass) {
+        double a[B] = {};
+        for (int c = 0; c < jj; ++c) {
+          const double* sc = &S[(size_t)(p0 + c) * d];
+          double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
+          int i = 0;
+          for (; i + 4 <= d; i += 4) {
+            a0 += sc[i] * z[i];
+            a1 += sc[i + 1] * z[i + 1];
+            a2 += sc[i + 2] * z[i + 2];
+            a3 += sc[i + 3] * z[i + 3];
+          }
+          for (; i < d; ++i) a0 += sc[i] * z[i];
+          a[c] = (a0 + a1) + (a2 + a3);
+        }
+        for (int c = 0; c < jj; ++c) {
+          const double* sc = &S[(size_t)(p0 + c) * d];
+          for (int i = 0; i < d; ++i) z[i] -= sc[i] * a[c];
+          r[c] += a[c];
+        }
+      }
+      // q~ = k_j - sum_c (q~_c / beta_c) r_c, fused with its partial sketches
+      for (int c = 0; c < jj; ++c) nrs[c] = to_df(-r[c] * cs[p0 + c]);
+      if (jj > 0) QK(cudaMemcpyAsync(w.nrs, nrs.data(), (size_t)jj * sizeof(float2), cudaMemcpyHostToDevice, w.st));
+      rks::launch_df_update_sketch(col(w, p0), w.ldu, jj, w.nrs, w.sj, w.tiles, w.part, false, w.st);
+      rc = fold_to_host(w, d);
+      if (rc) return rc;
+      double bb = 0.0;
+      for (int i = 0; i < d; ++i) { const double v = w.host[i] * w.zscale; bb += v * v; }
+      const double beta = std::sqrt(bb);
+      if (!(beta > 0.0) || !std::isfinite(beta)) return RKS_EBREAKDOWN;
+      for (int i = 0; i < d; ++i) S[i + (size_t)j * d] = w.host[i] * w.zscale / beta;
+      for (int c = 0; c < jj; ++c) R[p0 + c + (size_t)j * s] = r[c];
+      R[j + (size_t)j * s] = beta;
+      cs[j] = 1.0 / beta;
+    }
   }
   QK(cudaMemcpyAsync(w.scale, cs.data(), (size_t)s * sizeof(double), cudaMemcpyHostToDevice, w.st));
   return RKS_OK;
@@ -256,19 +323,15 @@ int rhqr(QrWork& w, std::vector<double>& R, std::vector<double>& scale) {
   // top blocks (rows 0..s-1) and sketches of the bottom rows of every column
   QK(cudaMemcpy2DAsync(top.data(), s * sizeof(float2), w.U, w.ldu * sizeof(float2), s * sizeof(float2), s,
                        cudaMemcpyDeviceToHost, w.st));
-  for (int l = 0; l < s; ++l) {
-    rks::launch_df_sketch_vec(col(w, l) + s, w.tiles, w.part, false, w.st);
-    rks::launch_df_fold(w.part, d, w.tiles.G, w.sums + (size_t)l * d, w.st);
-  }
-  QK(cudaGetLastError());
-  QK(cudaMemcpyAsync(w.host.data(), w.sums, (size_t)d * s * sizeof(double), cudaMemcpyDeviceToHost, w.st));
-  QK(cudaStreamSynchronize(w.st));
+  std::vector<double> Z0;
+  int rc = sketch_block(w, 0, Z0, s);
+  if (rc) return rc;
   for (int l = 0; l < s; ++l) {
     for (int i = 0; i < s; ++i) {
       const float2 t = top[i + (size_t)l * s];
       Y[i + (size_t)l * ns] = (double)t.x + (double)t.y;
     }
-    for (int i = 0; i < d; ++i) Y[s + i + (size_t)l * ns] = w.host[i + (size_t)l * d] * w.zscale;
+    for (int i = 0; i < d; ++i) Y[s + i + (size_t)l * ns] = Z0[i + (size_t)l * d];
   }
   R.assign((size_t)s * s, 0.0);
   for (int j = 0; j < s; ++j) {
@@ -364,52 +427,50 @@ extern "C" int rks_sketch_qr(int64_t n, int s, const double* K, int64_t ldk, int
   if (Q == K && ldq != ldk) return RKS_EINVAL;
   cudaStream_t st = (cudaStream_t)stream;
   QrWork w;
-  int rc = setup(w, n, s, d, zeta, seed, st, method == RKS_QR_RHQR ? n - s : n);
+  int rc = setup(w, n, s, d, zeta, seed, st, method == RKS_QR_RHQR ? n - s : n, method == RKS_QR_RGS ? s : 2 * s);
   if (rc) return rc;
-  for (int j = 0; j < s; ++j) rks::launch_d2df(n, K + (size_t)j * ldk, col(w, j), false, st);
-  QK(cudaGetLastError());
   std::vector<double> Rh, Sh;
   int out0 = 0;                 // first column of the result in U
   std::vector<double> ones(s, 1.0);
   if (method == RKS_QR_RGS) {
-    rc = rgs(w, Rh, Sh);
+    rc = rgs(w, K, ldk, Rh, Sh);
     if (rc) return rc;
   } else if (method == RKS_QR_RHQR) {
     std::vector<double> sc;
+    rks::launch_d2df_cols(n, K, ldk, w.U, w.ldu, s, st);
     rc = rhqr(w, Rh, sc);
     if (rc) return rc;
     out0 = s;
     QK(cudaMemcpyAsync(w.scale, sc.data(), (size_t)s * sizeof(double), cudaMemcpyHostToDevice, st));
     if (S) {                    // Omega' Q[s:, :], measured: the sketched rows of Theta Q
-      Sh.assign((size_t)d * s, 0.0);
-      for (int j = 0; j < s; ++j) {
-        rks::launch_df_sketch_vec(col(w, s + j) + s, w.tiles, w.part, false, st);
-        rks::launch_df_fold(w.part, d, w.tiles.G, w.sums + (size_t)j * d, st);
-      }
-      QK(cudaGetLastError());
-      QK(cudaMemcpyAsync(w.host.data(), w.sums, (size_t)d * s * sizeof(double), cudaMemcpyDeviceToHost, st));
-      QK(cudaStreamSynchronize(st));
+      rc = sketch_block(w, s, Sh, s);
+      if (rc) return rc;
       for (int j = 0; j < s; ++j)
-        for (int i = 0; i < d; ++i) Sh[i + (size_t)j * d] = w.host[i + (size_t)j * d] * w.zscale * sc[j];
+        for (int i = 0; i < d; ++i) Sh[i + (size_t)j * d] *= sc[j];
     }
   } else {
     std::vector<double> R1;
-    rc = whiten(w, R1, Sh);
+    rc = whiten(w, K, ldk, R1, Sh);
     if (rc) return rc;
     out0 = s;
     Rh = R1;
     if (method == RKS_QR_RCHOLQR) {
-      // G = Q1^T Q1 (columns s .. 2s-1), upper triangle by columns
+      // G = Q1^T Q1 (columns s .. 2s-1)
       std::vector<double> G((size_t)s * s, 0.0);
-      for (int cv = 0; cv < s; ++cv) {
-        rks::launch_df_dots(col(w, s), w.ldu, cv + 1, cv, w.tiles, w.part, st);
-        rks::launch_df_fold(w.part, cv + 1, w.tiles.G, w.sums + (size_t)cv * s, st);
-      }
+      const int np = rks::gram_pairs(s);
+      rks::launch_df_gram(n, col(w, s), w.ldu, s, w.part, st);
+      rks::launch_df_fold(w.part, np, rks::gram_ctas(n), w.sums, st);
       QK(cudaGetLastError());
-      QK(cudaMemcpyAsync(w.host.data(), w.sums, (size_t)s * s * sizeof(double), cudaMemcpyDeviceToHost, st));
+      QK(cudaMemcpyAsync(w.host.data(), w.sums, (size_t)np * sizeof(double), cudaMemcpyDeviceToHost, st));
       QK(cudaStreamSynchronize(st));
-      for (int cv = 0; cv < s; ++cv)
-        for (int l = 0; l <= cv; ++l) G[l + (size_t)cv * s] = G[cv + (size_t)l * s] = w.host[l + (size_t)cv * s];
+      for (int q = 0, bj = 0, bi = 0; q < np / 16; ++q) {
+        for (int u = 0; u < 4; ++u)
+          for (int v = 0; v < 4; ++v) {
+            const int l = 4 * bi + u, cv = 4 * bj + v;
+            if (l <= cv && cv < s) G[l + (size_t)cv * s] = G[cv + (size_t)l * s] = w.host[(size_t)q * 16 + 4 * u + v];
+          }
+        if (bi++ == bj) { bi = 0; ++bj; }
+      }
       // Cholesky G = R2^T R2 (R2 upper)
       std::vector<double> R2((size_t)s * s, 0.0);
       for (int j = 0; j < s; ++j) {
