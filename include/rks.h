@@ -187,7 +187,8 @@ enum {
 };
 
 /* Counters of the last rks_solve.  launches counts every kernel the library
- * launched.  ms (event time) is filled for the timed classes when
+ * launched (the whole expansion of a small double-float problem is one
+ * launch, counted under RKS_K_UPDATE).  ms (event time) is filled for the timed classes when
  * opts.profile is set, else 0.  bytes
  * and flops are the algorithmic traffic / work of the launches: SpMV
  * nnz*(P_A + 4) + 4(n+1) + 2 P_V n; update (c + 2) P_V n for c basis

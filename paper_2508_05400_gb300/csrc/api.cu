@@ -91,6 +91,7 @@ struct rks_ctx {
   bool up_M2 = false;      // the Gram matrix changed at the restart: upload it
   void* Ub = nullptr;      // basis in use: U2 or Uf
   bool f32 = false;        // basis in use is FP32
+  bool small = false;      // tiles of the fused expansion (launch_df_expand_small)
   int phase_restarts = 0;
   float2* S2 = nullptr;
   float2* nrs = nullptr;
@@ -291,6 +292,19 @@ void expand_df_launches(rks_ctx* c, int c0) {
   const double PA = (c->A2.dvals && c->A2.dvals_f32 && c->A2.D <= 8) ? 4.0 : PV;
   const double spmv_bytes = c->A2.dvals ? (double)c->A2.D * PA * n + 2 * PV * n
                                         : (double)c->nnz * (PV + 4) + 4.0 * (n + 1) + 2 * PV * n;
+  // a small problem's expansion is one launch (counted as an update), unless
+  // the kernel classes are timed or the barriers' test hook is on
+  if (c->small && !c->opts.profile && !c->opts.debug_stall &&
+      rks::launch_df_expand_small(c->A2, c->U2, c->ldu, c0, c->m, c->tiles, c->tiles.rows_max, c->tiles.tiles_max,
+                                  c->zscale, c->S, c->S2, c->M2, c->m + 1, c->colscale, c->coef, c->m + 1, c->flag,
+                                  c->stream)) {
+    const int steps = c->m - c0;
+    const double cols = 0.5 * steps * (c0 + 1 + c->m);     // basis columns over all steps
+    prof_end(c, -1, RKS_K_UPDATE, 1, steps * spmv_bytes + (cols + 2.0 * steps) * P * n,
+             2.0 * c->nnz * steps + 2.0 * n * cols);
+    c->nmatvec += steps;
+    return;
+  }
   for (int j = c0; j < c->m; ++j) {
     const int col = j + 1;
     int s = prof_begin(c, RKS_K_SPMV);
@@ -1100,7 +1114,11 @@ int rks_create(rks_ctx** out, int64_t n, const int32_t* rowptr, const int32_t* c
       if (bad) return fail(RKS_EINVAL);
     }
     if (rks::configure_df_kernels() != cudaSuccess) return fail(RKS_ECUDA);
-    if (rks::build_sketch_tiles(n, d, o.zeta, c->otab, &c->tiles, c->stream) != 0) return fail(RKS_ECUDA);
+    // a small double-float problem: the tiles of the fused expansion
+    const int small =
+        c->prec == RKS_PREC_DF && o.ortho == RKS_ORTHO_SKETCH ? rks::small_expand_ctas(n, d, m, o.zeta) : 0;
+    if (rks::build_sketch_tiles(n, d, o.zeta, c->otab, &c->tiles, c->stream, small) != 0) return fail(RKS_ECUDA);
+    c->small = small > 0;
     cudaFree(c->otab);
     c->otab = nullptr;
     if (rks::sketch_tile_smem(c->tiles, m + 1) > 200 * 1024) return fail(RKS_EINVAL);

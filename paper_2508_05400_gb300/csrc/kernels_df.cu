@@ -1255,6 +1255,20 @@ __device__ double block_sum_d(double v, double* red) {
   return red[32];
 }
 
+// The same sum, known to thread 0 only (one barrier fewer)
+__device__ double block_sum_0(double v, double* red) {
+  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  __syncthreads();
+  if (lane == 0) red[warp] = v;
+  __syncthreads();
+  if (warp == 0) {
+    v = lane < nw ? red[lane] : 0.0;
+    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  }
+  return v;
+}
+
 // Phase A for one column (one warp): r1[col] = S[:, col]^T z (if want_r1)
 // and, when column j is being finished (sjd = its DF values), the Gram entries
 // M[col, j] = M[j, col] = S[:, col]^T s_j.  Column j itself reads sjd.
@@ -1483,42 +1497,52 @@ __global__ void __launch_bounds__(256) k_df_ls_coop(
   }
   const double* zsrc = stage ? zst : z_raw;
   const double* ssrc = stage ? sst : s_raw;
+  // FP64 runs at two lanes a clock: a square root or a division by every
+  // thread of the CTA costs thousands of cycles, so thread 0 forms them
+  __shared__ double bsh[2];
   double inv = 0.0;
   if (finish) {
     double ss = 0.0;
     for (int r = tid; r < d; r += nt) { double v = ssrc[r] * zscale; ss = fma(v, v, ss); }
-    ss = block_sum_d(ss, red);
-    const double beta = sqrt(ss);
-    const bool finite = isfinite(beta);
-    const bool brk = finite && !(beta > 1e-14 * zn_prev);
-    inv = (finite && !brk) ? 1.0 / beta : 0.0;
-    for (int r = tid; r < d; r += nt) sjd[r] = df_from_double(ssrc[r] * zscale * inv);
-    if (blockIdx.x == 0) {
-      for (int r = tid; r < d; r += nt) {
-        double v = ssrc[r] * zscale * inv;
-        S64[r + (size_t)j * d] = v;
-        S2[r + (size_t)j * d] = df_from_double(v);
-      }
-      if (j >= 1) {
-        double* cc = coef + (size_t)(j - 1) * ldcoef;
-        for (int i = tid; i < j; i += nt) cc[i] = rprev[i];
-        if (tid == 0) cc[j] = beta;
-      }
-      if (tid == 0) {
-        colscale[j] = inv;
+    ss = block_sum_0(ss, red);
+    if (tid == 0) {
+      const double beta = sqrt(ss);
+      const bool finite = isfinite(beta);
+      const bool brk = finite && !(beta > 1e-14 * zn_prev);
+      bsh[0] = (finite && !brk) ? 1.0 / beta : 0.0;
+      if (blockIdx.x == 0) {
+        bsh[1] = beta;
+        colscale[j] = bsh[0];
         if (!finite) atomicOr(flag, RKS_FLAG_NAN);
         else if (brk) atomicOr(flag, RKS_FLAG_BREAKDOWN);
       }
+    }
+    __syncthreads();
+    inv = bsh[0];
+    for (int r = tid; r < d; r += nt) {
+      const double v = ssrc[r] * zscale * inv;
+      const float2 w = df_from_double(v);
+      sjd[r] = w;
+      if (blockIdx.x == 0) {
+        S64[r + (size_t)j * d] = v;
+        S2[r + (size_t)j * d] = w;
+      }
+    }
+    if (blockIdx.x == 0 && j >= 1) {
+      double* cc = coef + (size_t)(j - 1) * ldcoef;
+      for (int i = tid; i < j; i += nt) cc[i] = rprev[i];
+      if (tid == 0) cc[j] = bsh[1];
     }
   }
   const double scj = finish ? inv : cs_j;
   double zz = 0.0;
   for (int r = tid; r < d; r += nt) {
     double v = zsrc[r] * zscale * scj;
-    zz = fma(v, v, zz);
+    if (blockIdx.x == 0) zz = fma(v, v, zz);    // ||z|| is CTA 0's to store
     zd[r] = df_from_double(v);
   }
-  zz = block_sum_d(zz, red);            // also orders the zd and sjd writes before their use
+  if (blockIdx.x == 0) zz = block_sum_0(zz, red);
+  __syncthreads();                      // orders the zd and sjd writes before their use
   // phase A: r1[col] = S[:, col]^T z and, when finishing, M[col, j] = S[:, col]^T s_j
   float2 mnew = make_float2(0.f, 0.f);  // M[j, col0] computed here (finishing)
   for (int col = gw; col < c; col += tw) {
@@ -2027,6 +2051,390 @@ __global__ void k_df_add_f32_cols(int64_t n, float2* __restrict__ U2, int64_t ld
 }
 
 // ---------------------------------------------------------------------------
+// Small problems: the whole expansion in one launch of one cluster
+// ---------------------------------------------------------------------------
+//
+// At a few thousand rows an Arnoldi step is three launches of 6 to 16 us whose
+// work would take one (2000 rows, 40 columns: 45 us a step with the gaps).
+// Here the CTAs of one thread-block cluster (at most 16) own the row ranges of
+// the sketch tiles and run all steps c0 .. m - 1 of Algorithm 2: per step the
+// product with A and its sketch, the least squares (by every CTA, from the
+// same data), the update and its sketch.  Partial sketches go to every CTA
+// through distributed shared memory, so a step has two cluster barriers.
+// The bin lists, S and M stay in shared memory, the CTA's rows of the basis too
+// where they fit.  The arithmetic and the order of every sum are those of
+// k_df_spmv_* / k_df_ls_coop / k_df_update_sketch on the same tiles: the same
+// bits.  Sixteen SMs suffice while a step's row work stays below its barriers
+// and latencies: kSmallRows.  Measured per step, d = 80, 30 to 40 columns: 12 us
+// at 2000 rows (31 with the separate kernels, 45 with their launches queued
+// from the host), 18 at 16 000 (24), 24 at 32 000 (24).
+struct SmallArgs {
+  const int32_t *rowptr, *colind;
+  const float2* vals;          // CSR (D = 0)
+  const float2* dvals;         // by diagonals (D > 0)
+  DiaOffs offs;
+  int D;
+  int64_t ldd;
+  int n, c0, m;
+  float2* U;
+  int64_t ldu;
+  SketchTiles tv;
+  double zscale;
+  double* S64;
+  const float2 *S2, *M2;
+  double *colscale, *coef;
+  int ldcoef, ldm;
+  int* flag;
+  int rows_max, tiles_max;     // of a CTA
+  int slab;                    // the CTA's basis rows in shared memory
+};
+
+__device__ __forceinline__ uint32_t cl_addr(const void* p, int rank) {
+  uint32_t a = (uint32_t)__cvta_generic_to_shared(p), r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void cl_put(uint32_t a, double v) {
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+}
+__device__ __forceinline__ void cl_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+struct SmallSmem {
+  size_t zx, sx, csc, rp, zd, sjd, acc, v, r1, nrs, mcol, es, ms, of, slab, S, M, total;
+};
+__host__ __device__ inline SmallSmem small_smem(int G, int d, int m, int rows, int tiles, int L, int zeta,
+                                                int slab) {
+  SmallSmem s;
+  size_t o = 0;
+  auto take = [&](size_t bytes) { size_t r = o; o += (bytes + 15) & ~(size_t)15; return r; };
+  s.zx = take((size_t)G * d * 8);
+  s.sx = take((size_t)G * d * 8);
+  s.csc = take((size_t)(m + 1) * 8);
+  s.rp = take((size_t)(m + 1) * 8);
+  s.zd = take((size_t)d * 8);
+  s.sjd = take((size_t)d * 8);
+  s.acc = take((size_t)d * 8);
+  s.v = take((size_t)rows * 8);
+  s.r1 = take((size_t)(m + 1) * 8);
+  s.nrs = take((size_t)(m + 1) * 8);
+  s.mcol = take((size_t)(m + 1) * 8);
+  s.es = take((size_t)rows * zeta * 2);
+  s.ms = take((size_t)tiles * d * 4);
+  s.of = take((size_t)tiles * (L + 1) * 4);
+  s.slab = take(slab ? (size_t)rows * (m + 1) * 8 : 0);
+  s.S = take((size_t)d * (m + 1) * 8);
+  s.M = take((size_t)(m + 1) * (m + 1) * 8);
+  s.total = o;
+  return s;
+}
+
+// sum over g < G <= 16 of p[g * d] in the tree of fold_row
+__device__ __forceinline__ double fold16(const double* p, int d, int G) {
+  double v[16];
+#pragma unroll
+  for (int g = 0; g < 16; ++g) v[g] = g < G ? p[(size_t)g * d] : 0.0;
+#pragma unroll
+  for (int o = 8; o; o >>= 1)
+#pragma unroll
+    for (int g = 0; g < o; ++g) v[g] += v[g + o];
+  return v[0];
+}
+
+__global__ void __launch_bounds__(512) k_df_expand_small(const SmallArgs a) {
+  extern __shared__ __align__(16) uint8_t sraw[];
+  __shared__ double red[64];
+  const SketchTiles& tv = a.tv;
+  const int d = tv.d, m = a.m, G = gridDim.x, rank = blockIdx.x, L1 = tv.L + 1;
+  const SmallSmem lay = small_smem(G, d, m, a.rows_max, a.tiles_max, tv.L, tv.zeta, a.slab);
+  double* zx = reinterpret_cast<double*>(sraw + lay.zx);
+  double* sx = reinterpret_cast<double*>(sraw + lay.sx);
+  double* csc = reinterpret_cast<double*>(sraw + lay.csc);
+  double* rp = reinterpret_cast<double*>(sraw + lay.rp);
+  float2* zd = reinterpret_cast<float2*>(sraw + lay.zd);
+  float2* sjd = reinterpret_cast<float2*>(sraw + lay.sjd);
+  float2* acc = reinterpret_cast<float2*>(sraw + lay.acc);
+  float2* v = reinterpret_cast<float2*>(sraw + lay.v);
+  float2* r1 = reinterpret_cast<float2*>(sraw + lay.r1);
+  float2* nrs = reinterpret_cast<float2*>(sraw + lay.nrs);
+  float2* mcol = reinterpret_cast<float2*>(sraw + lay.mcol);
+  uint16_t* es = reinterpret_cast<uint16_t*>(sraw + lay.es);
+  uint32_t* ms = reinterpret_cast<uint32_t*>(sraw + lay.ms);
+  int* of = reinterpret_cast<int*>(sraw + lay.of);
+  float2* slab = reinterpret_cast<float2*>(sraw + lay.slab);
+  float2* Ss = reinterpret_cast<float2*>(sraw + lay.S);
+  float2* Ms = reinterpret_cast<float2*>(sraw + lay.M);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  constexpr int NT = 512, NW = 16;
+  const int t0 = tv.ctile[rank], t1 = tv.ctile[rank + 1];
+  const int row0 = (int)tv.row[t0], rows = (int)tv.row[t1] - row0;
+  for (int t = t0; t < t1; ++t) {
+    const int r0 = (int)tv.row[t];
+    tile_stage(tv, t, r0, (int)tv.row[t + 1] - r0, of + (t - t0) * L1, ms + (t - t0) * d,
+               es + (size_t)(r0 - row0) * tv.zeta);
+  }
+  for (int c = tid; c <= a.c0; c += NT) csc[c] = a.colscale[c];
+  if (a.slab)
+    for (int c = warp; c <= a.c0; c += NW)
+      for (int l = lane; l < rows; l += 32) slab[c * a.rows_max + l] = a.U[row0 + l + (int64_t)c * a.ldu];
+  for (int t = tid; t < d * (a.c0 + 1); t += NT) Ss[t] = a.S2[t];
+  for (int c = warp; c <= a.c0; c += NW)
+    for (int l = lane; l <= a.c0; l += 32) Ms[l + c * (m + 1)] = a.M2[l + (size_t)c * a.ldm];
+  // the CTA's Omega-sums of its rows' values in v, to every CTA's dst[rank]
+  // (tiles last to first when rev: the update kernel's second half of the grid)
+  auto sketch_out = [&](double* dst, bool rev) {
+    for (int r = tid; r < d; r += NT) acc[r] = make_float2(0.f, 0.f);
+    for (int q = 0; q < t1 - t0; ++q) {
+      const int t = rev ? t1 - t0 - 1 - q : q;
+      __syncthreads();
+      tile_gather<true>(d, tv.H, v + t * kTileRows, of + t * L1, ms + t * d, es + (size_t)t * kTileRows * tv.zeta, acc);
+    }
+    __syncthreads();
+    for (int r = tid; r < d; r += NT) {
+      const double x = df_to_double(acc[r]);
+      const double* p = dst + (size_t)rank * d + r;
+      for (int k = 0; k < G; ++k) cl_put(cl_addr(p, k), x);
+    }
+    cl_sync();
+  };
+  double zz = 0.0;                 // this thread's part of ||z||^2
+  cl_sync();                       // every CTA runs before the first remote store
+  for (int j = a.c0; j <= m; ++j) {
+    const bool fin = j > a.c0;
+    double inv = 0.0;
+    if (fin) {                     // column j: beta_j = ||s~_j||, S, scale, coefficients
+      double ss = 0.0;
+      double sv[2] = {0.0, 0.0};   // this thread's entries r = tid, tid + 512 of s~ (d <= 1024)
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+        if (tid + u * NT < d) sv[u] = fold16(sx + tid + u * NT, d, G) * a.zscale;
+      // strands of 256 as in the least-squares kernel: entries through shared memory
+      double* st = reinterpret_cast<double*>(acc);   // free until this step's sketches
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+        if (tid + u * NT < d) st[tid + u * NT] = sv[u];
+      __syncthreads();
+      if (tid < 256)
+        for (int r = tid; r < d; r += 256) { const double x = st[r]; ss = fma(x, x, ss); }
+      // a warp's sums where it has entries (the others' are zeros); ||z||^2 of
+      // the last step goes along.  Roots and quotients by thread 0 only (FP64
+      // runs at two lanes a clock)
+      if (warp < 8 && warp * 32 < d) {
+        for (int o = 16; o; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+      }
+      if (warp * 32 < d) {
+        for (int o = 16; o; o >>= 1) zz += __shfl_xor_sync(0xffffffffu, zz, o);
+      }
+      if (lane == 0) { red[warp] = warp < 8 && warp * 32 < d ? ss : 0.0; red[32 + warp] = warp * 32 < d ? zz : 0.0; }
+      __syncthreads();
+      if (warp == 0) {
+        double x = lane < 8 ? red[lane] : 0.0, zq = lane < NW ? red[32 + lane] : 0.0;
+        for (int o = 16; o; o >>= 1) {
+          x += __shfl_xor_sync(0xffffffffu, x, o);
+          zq += __shfl_xor_sync(0xffffffffu, zq, o);
+        }
+        if (lane == 0) {
+          const double beta = sqrt(x);
+          const bool finite = isfinite(beta), brk = finite && !(beta > 1e-14 * sqrt(zq));
+          const double iv = (finite && !brk) ? 1.0 / beta : 0.0;
+          red[60] = iv;
+          csc[j] = iv;
+          if (rank == 0) {
+            a.coef[(size_t)(j - 1) * a.ldcoef + j] = beta;
+            a.colscale[j] = iv;
+            if (!finite) atomicOr(a.flag, RKS_FLAG_NAN);
+            else if (brk) atomicOr(a.flag, RKS_FLAG_BREAKDOWN);
+          }
+        }
+      }
+      __syncthreads();
+      inv = red[60];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int r = tid + u * NT;
+        if (r < d) {
+          const double x = sv[u] * inv;
+          const float2 w = df_from_double(x);
+          sjd[r] = w;
+          Ss[r + j * d] = w;
+          if (rank == 0) a.S64[r + (size_t)j * d] = x;
+        }
+      }
+      if (rank == 0) {
+        double* cc = a.coef + (size_t)(j - 1) * a.ldcoef;
+        for (int i = tid; i < j; i += NT) cc[i] = rp[i];
+      }
+    }
+    if (j == m) break;
+    // w = A u~_j on the CTA's rows (u~_j was written by all CTAs: from L2)
+    const float2* x = a.U + (int64_t)j * a.ldu;
+    for (int l = tid; l < rows; l += NT) {
+      const int i = row0 + l;
+      float sh = 0.f, sl = 0.f;
+      if (a.D > 0) {
+        for (int e0 = 0; e0 < a.D; e0 += 4) {
+          float2 av[4], xv[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int e = e0 + u, jx = e < a.D ? i + a.offs.o[e] : -1;
+            const bool on = jx >= 0 && jx < a.n;
+            av[u] = e < a.D ? a.dvals[e * a.ldd + i] : make_float2(0.f, 0.f);
+            xv[u] = on ? __ldcg(x + jx) : make_float2(0.f, 0.f);
+          }
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            if (e0 + u < a.D) df_mac(av[u].x, av[u].y, xv[u].x, xv[u].y, sh, sl);
+        }
+      } else {
+        const int p1 = a.rowptr[i + 1];
+#pragma unroll 4
+        for (int p = a.rowptr[i]; p < p1; ++p) {
+          const float2 av = a.vals[p], xv = __ldcg(x + a.colind[p]);
+          df_mac(av.x, av.y, xv.x, xv.y, sh, sl);
+        }
+      }
+      v[l] = df_norm(sh, sl);
+    }
+    __syncthreads();               // v complete, st (acc) read
+    sketch_out(zx, false);
+    // z = Omega w / beta_j, r1 = S^T z and the new row of M
+    const double scj = fin ? inv : csc[j];
+    zz = 0.0;
+    for (int r = tid; r < d; r += NT) {
+      const double q = fold16(zx + r, d, G) * a.zscale * scj;
+      zz = fma(q, q, zz);
+      zd[r] = df_from_double(q);
+    }
+    __syncthreads();
+    for (int col = warp; col <= j; col += NW) {
+      float s_ = 0.f, t_ = 0.f, g = 0.f, ge = 0.f;
+      for (int r = lane; r < d; r += 32) {
+        const float2 sc = fin && col == j ? sjd[r] : Ss[r + col * d], b = zd[r];
+        df_mac(sc.x, sc.y, b.x, b.y, s_, t_);
+        if (fin) { const float2 e = sjd[r]; df_mac(sc.x, sc.y, e.x, e.y, g, ge); }
+      }
+      df_warp_sum(s_, t_);
+      if (fin) df_warp_sum(g, ge);
+      if (lane == 0) {
+        r1[col] = df_norm(s_, t_);
+        if (fin) {
+          const float2 mv = df_norm(g, ge);
+          mcol[col] = mv;
+          Ms[col + j * (m + 1)] = mv;
+          Ms[j + col * (m + 1)] = mv;
+        }
+      }
+    }
+    __syncthreads();
+    // r = 2 r1 - M r1, the update's coefficients
+    for (int col = warp; col <= j; col += NW) {
+      float s_ = 0.f, t_ = 0.f;
+      for (int l = lane; l <= j; l += 32) {
+        const float2 mv = fin && l == j ? mcol[col] : (fin && col == j ? mcol[l] : Ms[l + col * (m + 1)]), b = r1[l];
+        df_mac(mv.x, mv.y, b.x, b.y, s_, t_);
+      }
+      df_warp_sum(s_, t_);
+      if (lane == 0) {
+        const float2 rc = r1[col];
+        float hs = 2.f * rc.x, ht = 2.f * rc.y;   // exact doubling
+        df_add(-s_, -t_, hs, ht);
+        nrs[col] = df_norm(hs, ht);
+      }
+    }
+    __syncthreads();
+    for (int col = tid; col <= j; col += NT) {    // FP64 side by side, not one lane a warp
+      const double rd = df_to_double(nrs[col]);
+      rp[col] = rd;
+      nrs[col] = df_from_double(-rd * (col == j ? scj : csc[col]));
+    }
+    const float2 sj = df_from_double(scj);
+    __syncthreads();
+    // u~ = w / beta_j - U b on the CTA's rows
+    for (int l = tid; l < rows; l += NT) {
+      const float2 w = v[l];
+      float sh = 0.f, sl = 0.f;
+      df_mac(w.x, w.y, sj.x, sj.y, sh, sl);
+      if (a.slab) {
+#pragma unroll 4
+        for (int c = 0; c <= j; ++c) {
+          const float2 u = slab[c * a.rows_max + l], r = nrs[c];
+          df_mac(u.x, u.y, r.x, r.y, sh, sl);
+        }
+      } else {
+        const float2* up = a.U + row0 + l;
+        int c = 0;
+        for (; c + 16 <= j + 1; c += 16) {
+          float2 u[16];
+#pragma unroll
+          for (int q = 0; q < 16; ++q) u[q] = __ldcg(up + (int64_t)(c + q) * a.ldu);
+#pragma unroll
+          for (int q = 0; q < 16; ++q) df_mac(u[q].x, u[q].y, nrs[c + q].x, nrs[c + q].y, sh, sl);
+        }
+#pragma unroll 4
+        for (; c <= j; ++c) {
+          const float2 u = __ldcg(up + (int64_t)c * a.ldu), r = nrs[c];
+          df_mac(u.x, u.y, r.x, r.y, sh, sl);
+        }
+      }
+      const float2 u = df_norm(sh, sl);
+      v[l] = u;
+      if (a.slab) slab[(j + 1) * a.rows_max + l] = u;
+      a.U[row0 + l + (int64_t)(j + 1) * a.ldu] = u;
+    }
+    __syncthreads();
+    sketch_out(sx, rank >= G / 2);   // its barrier also orders u~'s rows before the next product
+  }
+}
+
+// CTAs of the fused expansion (0: the separate kernels): a power of two with
+// at least 64 rows each.  At most kSmallRows rows, and S, M and the partial
+// sketches of all CTAs within one CTA's shared memory: read from L2 instead,
+// they cost more than the launches saved (d = 320, 80 columns, 4900 rows: 60
+// us a step against 57).
+int small_expand_ctas(int64_t n, int d, int m, int zeta) {
+  if (n > kSmallRows) return 0;
+  int g = 1;
+  while (g < 16 && n >= (int64_t)g * 128) g *= 2;
+  const int rows = (int)((n + g - 1) / g) + 2;
+  return small_smem(g, d, m, rows, 1, 512, zeta, 0).total <= 200 * 1024 ? g : 0;
+}
+
+bool launch_df_expand_small(const CsrDF& A, float2* U, int64_t ldu, int c0, int m, const SketchTiles& t, int rows_max,
+                            int tiles_max, double zscale, double* S64, float2* S2, float2* M2, int ldm,
+                            double* colscale, double* coef, int ldcoef, int* flag, cudaStream_t st) {
+  if (t.d > 1024 || A.fmt == kSpmvMerge || A.fmt == kSpmvWarp || A.f32) return false;
+  SmallArgs a;
+  a.rowptr = A.rowptr; a.colind = A.colind; a.vals = static_cast<const float2*>(A.vals);
+  a.dvals = static_cast<const float2*>(A.dvals);
+  a.D = A.dvals ? A.D : 0;
+  for (int e = 0; e < a.D; ++e) a.offs.o[e] = A.doff[e];
+  a.ldd = A.ldd; a.n = (int)A.n; a.c0 = c0; a.m = m; a.U = U; a.ldu = ldu; a.tv = t; a.zscale = zscale;
+  a.S64 = S64; a.S2 = S2; a.M2 = M2; a.colscale = colscale; a.coef = coef; a.ldcoef = ldcoef; a.ldm = ldm;
+  a.flag = flag; a.rows_max = rows_max; a.tiles_max = tiles_max;
+  a.slab = 1;
+  auto bytes = [&]() { return small_smem(t.G, t.d, m, rows_max, tiles_max, t.L, t.zeta, a.slab).total; };
+  if (bytes() > 200 * 1024) a.slab = 0;
+  const size_t sm = bytes();
+  if (sm > 200 * 1024) return false;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = t.G;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3(t.G);
+  cfg.blockDim = dim3(512);
+  cfg.dynamicSmemBytes = sm;
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  if (cudaLaunchKernelEx(&cfg, k_df_expand_small, a) == cudaSuccess) return true;
+  (void)cudaGetLastError();     // no room for the cluster on this device: the separate kernels
+  return false;
+}
+
+// ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
 
@@ -2063,6 +2471,9 @@ static cudaError_t configure_df_kernels_once() {
   RKS_SMEM(k_tiles_build<4>); RKS_SMEM(k_tiles_build<8>); RKS_SMEM(k_tiles_build<16>);
   RKS_SMEM(k_df_ls1);
   RKS_SMEM(k_df_ls_coop);
+  RKS_SMEM(k_df_expand_small);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_df_expand_small, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   RKS_SMEM(k_df_rows_gemm<float2>);
   RKS_SMEM(k_df_rows_gemm<float>);
   RKS_SMEM((k_df_restart<float2, 4>)); RKS_SMEM((k_df_restart<float2, 8>)); RKS_SMEM((k_df_restart<float2, 16>));
@@ -2380,12 +2791,14 @@ void launch_df_sketch_vec(const void* x, const SketchTiles& t, double* part, boo
 
 // Row ranges: G CTAs (at most kSketchCtas) own contiguous, even-aligned row
 // ranges of equal length (to within two rows); each range is cut into tiles
-// of at most kTileRows rows.  The partition depends on n only.
-int build_sketch_tiles(int64_t n, int d, int zeta, const uint16_t* otab, SketchTiles* out, cudaStream_t st) {
+// of at most kTileRows rows.  The partition depends on n (and ctas) only.
+int build_sketch_tiles(int64_t n, int d, int zeta, const uint16_t* otab, SketchTiles* out, cudaStream_t st,
+                       int ctas) {
   SketchTiles t;
   t.n = n; t.d = d; t.zeta = zeta;
   const int64_t npair = (n + 1) / 2;
   int64_t G = std::min<int64_t>(kSketchCtas, std::max<int64_t>(1, (n + kTileRows - 1) / kTileRows));
+  if (ctas > 0) G = ctas;
   G = std::max<int64_t>(1, std::min(G, npair));
   std::vector<int> ctile(G + 1);
   std::vector<int64_t> row;
@@ -2397,6 +2810,10 @@ int build_sketch_tiles(int64_t n, int d, int zeta, const uint16_t* otab, SketchT
   ctile[G] = (int)row.size();
   row.push_back(n);
   t.G = (int)G;
+  for (int64_t g = 0; g < G; ++g) {
+    t.tiles_max = std::max(t.tiles_max, ctile[g + 1] - ctile[g]);
+    t.rows_max = std::max<int64_t>(t.rows_max, row[ctile[g + 1]] - row[ctile[g]]);
+  }
   t.ntile = (int)row.size() - 1;
   t.H = 1;
   while (t.H < 8 && (int64_t)d * t.H * 2 <= 512) t.H *= 2;

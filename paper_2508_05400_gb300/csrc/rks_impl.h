@@ -34,6 +34,7 @@ constexpr int kTileRows = 1024;
 struct SketchTiles {
   int64_t n = 0;
   int d = 0, zeta = 0, G = 0, ntile = 0, L = 0, H = 1;   // L: largest list; H: threads per list
+  int tiles_max = 0, rows_max = 0;                       // of a CTA
   int64_t* row = nullptr;
   int* ctile = nullptr;
   uint32_t* meta = nullptr;
@@ -137,7 +138,17 @@ void launch_ks_coef(int pass, int j, int c, int G, const double* part, const dou
                     float2* nrs, float2* sj, cudaStream_t st);
 void launch_ks_finish(int j, int G, const double* part, double thr, double* colscale,
                       const double* rprev, double* coef, int ldcoef, int* flag, cudaStream_t st);
-int build_sketch_tiles(int64_t n, int d, int zeta, const uint16_t* otab, SketchTiles* out, cudaStream_t st);
+// ctas > 0: that many CTAs instead of the default for n
+int build_sketch_tiles(int64_t n, int d, int zeta, const uint16_t* otab, SketchTiles* out, cudaStream_t st,
+                       int ctas = 0);
+// The whole expansion c0 .. m - 1 of a small problem in one launch (CTAs of
+// its tiles: small_expand_ctas, 0 when it is not small); false: not possible
+// for these sizes or storage, nothing launched.
+constexpr int64_t kSmallRows = 16384;
+int small_expand_ctas(int64_t n, int d, int m, int zeta);
+bool launch_df_expand_small(const CsrDF& A, float2* U, int64_t ldu, int c0, int m, const SketchTiles& t, int rows_max,
+                            int tiles_max, double zscale, double* S64, float2* S2, float2* M2, int ldm,
+                            double* colscale, double* coef, int ldcoef, int* flag, cudaStream_t st);
 void free_sketch_tiles(SketchTiles* t);
 size_t sketch_tile_smem(const SketchTiles& t, int c);
 void launch_omega_table(int64_t n, int d, int zeta, uint64_t seed, uint16_t* tab, int* flag, cudaStream_t st);
