@@ -275,21 +275,44 @@ __global__ void __launch_bounds__(256) k_tiles_build(const int64_t* __restrict__
   }
 }
 
-// (s, e) += sign * vals[row] for one bin-list entry; LO = false: the tile
-// holds FP32 values (zero low words), whose low words are left out
-template <bool LO>
-__device__ __forceinline__ void tile_add(uint32_t x, const float2* vals, float& s, float& e) {
-  const float2 v = vals[x & 0x7FFFu];
-  const uint32_t sg = (x & 0x8000u) << 16;
-  if (LO) {
-    df_add(__uint_as_float(__float_as_uint(v.x) ^ sg), __uint_as_float(__float_as_uint(v.y) ^ sg), s, e);
-  } else {
-    float s2, e2;
-    two_sum(s, __uint_as_float(__float_as_uint(v.x) ^ sg), s2, e2);
-    s = s2;
-    e += e2;
-  }
+__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ uint32_t lds32(uint32_t a) {
+  uint32_t x;
+  asm volatile("ld.shared.b32 %0, [%1];" : "=r"(x) : "r"(a));
+  return x;
 }
+__device__ __forceinline__ uint32_t lds16(uint32_t a) {
+  uint16_t x;
+  asm volatile("ld.shared.u16 %0, [%1];" : "=h"(x) : "r"(a));
+  return x;
+}
+__device__ __forceinline__ void lds_val(uint32_t a, uint32_t row, float2& v) {
+  asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a + row * 8u));
+}
+__device__ __forceinline__ void lds_val(uint32_t a, uint32_t row, float& v) {
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a + row * 4u));
+}
+__device__ __forceinline__ float flip(float v, uint32_t x) {   // -v where bit 15 of x is set
+  return __uint_as_float(__float_as_uint(v) ^ ((x << 16) & 0x80000000u));
+}
+
+// (s, e) += sign * v for a bin-list entry x; FP32 values have no low word, so
+// its terms are left out
+__device__ __forceinline__ void tile_add(uint32_t x, float2 v, float& s, float& e) {
+  df_add(flip(v.x, x), flip(v.y, x), s, e);
+}
+__device__ __forceinline__ void tile_add(uint32_t x, float v, float& s, float& e) {
+  float s2, e2;
+  two_sum(s, flip(v, x), s2, e2);
+  s = s2;
+  e += e2;
+}
+__device__ __forceinline__ void zero_val(float2& v) { v = make_float2(0.f, 0.f); }
+__device__ __forceinline__ void zero_val(float& v) { v = 0.f; }
+
+// a stored value (stv) into the tile's value buffer
+__device__ __forceinline__ void tile_put(float2* p, float2 v) { *p = v; }
+__device__ __forceinline__ void tile_put(float* p, float2 v) { *p = v.x; }
 
 // Sketch of one staged tile: acc[row] += sum over the row's bin list of
 // sign * vals[tile row], entries in their stored order.  The tile's slot
@@ -297,31 +320,61 @@ __device__ __forceinline__ void tile_add(uint32_t x, const float2* vals, float& 
 // H adjacent lanes share a position (each takes every H-th entry) when d is
 // small; their sums are combined by a fixed xor tree.  A sketch row has one
 // position per tile, so acc[row] has one writer per tile.
-template <bool LO>
-__device__ __forceinline__ void tile_gather(int d, int H, const float2* vals, const int* offs, const uint32_t* ms,
-                                            const uint16_t* es, float2* acc) {
+//
+// Bound by instruction issue (a 7-point FP32 SpMV with zeta = 8 issues in 73%
+// of the cycles): hence H as a constant (the slot offsets at constant
+// distances), 32-bit shared addresses, a sign by one exclusive or, and the
+// last one to three entries of a list as one masked round (adding an exact
+// zero changes no bit) instead of one by one.  The updates above: 64 -> 59 us
+// and 134 -> 130 us; 23 -> 21 us.  FP32 values are kept as 4 bytes: at random
+// banks a warp's read takes 3 to 4 passes instead of 6.
+template <int H, class TV>
+__device__ __forceinline__ void tile_gather_h(int d, const TV* vals, const int* offs, const uint32_t* ms,
+                                              const uint16_t* es, float2* acc) {
   const int total = d * H;
   const int lane = threadIdx.x & 31;
+  const uint32_t va = smem_addr(vals);
   for (int base = threadIdx.x & ~31; base < total; base += blockDim.x) {
     const int pp = base + lane;
-    const int p = pp / H, h = pp - p * H;
+    const int p = pp / H, h = pp % H;
     float s = 0.f, e = 0.f;
     int b = -1, cnt = 0;
     if (pp < total) {
       const uint32_t mt = ms[p];
       b = (int)(mt & 0xFFFFu);
       cnt = (int)(mt >> 16);
-      int q = h;
-      for (; q + 3 * H < cnt; q += 4 * H) {
-        const uint32_t x0 = es[offs[q] + p], x1 = es[offs[q + H] + p];
-        const uint32_t x2 = es[offs[q + 2 * H] + p], x3 = es[offs[q + 3 * H] + p];
-        tile_add<LO>(x0, vals, s, e);
-        tile_add<LO>(x1, vals, s, e);
-        tile_add<LO>(x2, vals, s, e);
-        tile_add<LO>(x3, vals, s, e);
+      const uint32_t ea = smem_addr(es) + 2u * p;
+      uint32_t oa = smem_addr(offs) + 4u * h;
+      int k = (cnt - h + H - 1) / H;          // entries of this lane
+      for (; k >= 4; k -= 4, oa += 16u * H) {
+        uint32_t x[4];
+        TV v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[u] = lds32(oa + 4u * H * u);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[u] = lds16(ea + 2u * x[u]);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) lds_val(va, x[u] & 0x7FFFu, v[u]);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) tile_add(x[u], v[u], s, e);
       }
-      for (; q < cnt; q += H) tile_add<LO>(es[offs[q] + p], vals, s, e);
+      if (k > 0) {
+        uint32_t x[3];
+        TV v[3];
+#pragma unroll
+        for (int u = 0; u < 3; ++u) x[u] = lds32(u < k ? oa + 4u * H * u : oa);
+#pragma unroll
+        for (int u = 0; u < 3; ++u) x[u] = lds16(ea + 2u * x[u]);
+#pragma unroll
+        for (int u = 0; u < 3; ++u) {
+          lds_val(va, x[u] & 0x7FFFu, v[u]);
+          if (u >= k) zero_val(v[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < 3; ++u) tile_add(x[u], v[u], s, e);
+      }
     }
+#pragma unroll
     for (int o = 1; o < H; o <<= 1) {
       const float s2 = __shfl_xor_sync(0xffffffffu, s, o);
       const float e2 = __shfl_xor_sync(0xffffffffu, e, o);
@@ -336,6 +389,16 @@ __device__ __forceinline__ void tile_gather(int d, int H, const float2* vals, co
       df_add(s, e, as, ae);
       acc[b] = df_norm(as, ae);
     }
+  }
+}
+template <class TV>
+__device__ __forceinline__ void tile_gather(int d, int H, const TV* vals, const int* offs, const uint32_t* ms,
+                                            const uint16_t* es, float2* acc) {
+  switch (H) {
+    case 1: tile_gather_h<1>(d, vals, offs, ms, es, acc); return;
+    case 2: tile_gather_h<2>(d, vals, offs, ms, es, acc); return;
+    case 4: tile_gather_h<4>(d, vals, offs, ms, es, acc); return;
+    default: tile_gather_h<8>(d, vals, offs, ms, es, acc); return;
   }
 }
 
@@ -384,57 +447,103 @@ __device__ __forceinline__ void tile_stage(const SketchTiles& tv, int64_t t, int
   for (int q = q0 + threadIdx.x; q < cnt; q += blockDim.x) es[q] = src[q];
 }
 
-// The bin lists of one tile held in registers between their load and their
-// store into shared memory, so that the loads of the next tile's lists are in
-// flight while this tile's rows are computed.  Valid when every per-thread
-// count fits (tile_regs_fit); the stored bytes are those of tile_stage.
-constexpr int kStageRegs = 2;   // uint4 of entries per thread (zeta <= 8)
-struct TileRegs {
-  uint4 e[kStageRegs];
-  int of[2];
-  uint32_t ms[2];
+// The CTA's tiles: their rows are consecutive and all but the last tile have
+// kTileRows of them, so no tile has to read its bounds first.  rev: taken last
+// to first.
+struct TileRange {
+  int t0, nt;
+  bool rev;
+  int64_t ra;
+  int len;                                        // rows of the CTA
+  __device__ __forceinline__ TileRange(const SketchTiles& tv, bool rev_) : rev(rev_) {
+    t0 = tv.ctile[blockIdx.x];
+    const int t1 = tv.ctile[blockIdx.x + 1];
+    nt = t1 - t0;
+    ra = tv.row[t0];
+    len = (int)(tv.row[t1] - ra);
+  }
+  __device__ __forceinline__ int at(int k) const { return rev ? nt - 1 - k : k; }   // tile of step k, from t0
+  __device__ __forceinline__ int64_t row(int k) const { return ra + at(k) * kTileRows; }
+  __device__ __forceinline__ int rows(int k) const { return min(kTileRows, len - at(k) * kTileRows); }
 };
-__host__ __device__ inline bool tile_regs_fit(const SketchTiles& tv) {
-  return tv.L + 1 <= 2 * 512 && tv.d <= 2 * 512 && kTileRows * tv.zeta / 8 <= kStageRegs * 512;
+
+// The shared buffers of step k (two sets, taken in turn).
+template <class TV>
+struct TileBuf {
+  TV* v;
+  int* of;
+  uint32_t* ms;
+  uint16_t* es;
+  __device__ __forceinline__ TileBuf(uint8_t* sm, const TileSmem& lay, const SketchTiles& tv, int k) {
+    const int buf = k & 1;
+    v = reinterpret_cast<TV*>(reinterpret_cast<float2*>(sm + lay.vb) + buf * kTileRows);
+    of = reinterpret_cast<int*>(sm + lay.offs) + buf * (tv.L + 1);
+    ms = reinterpret_cast<uint32_t*>(sm + lay.ms) + buf * tv.d;
+    es = reinterpret_cast<uint16_t*>(sm + lay.es) + (size_t)buf * kTileRows * tv.zeta;
+  }
+};
+
+__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src));
 }
-__device__ __forceinline__ void tile_regs_load(const SketchTiles& tv, int64_t t, TileRegs& R) {
-  const int L1 = tv.L + 1, d = tv.d;
-  const int64_t r0 = tv.row[t];
-  const int cnt = (int)(tv.row[t + 1] - r0) * tv.zeta;
-  const uint4* src = reinterpret_cast<const uint4*>(tv.ent + r0 * tv.zeta);   // r0 is a multiple of kTileRows
-#pragma unroll
-  for (int u = 0; u < kStageRegs; ++u) {
-    const int q = threadIdx.x + u * 512;
-    R.e[u] = q * 8 < cnt ? __ldg(src + q) : make_uint4(0u, 0u, 0u, 0u);
-  }
-#pragma unroll
-  for (int u = 0; u < 2; ++u) {
-    const int q = threadIdx.x + u * 512;
-    R.of[u] = q < L1 ? tv.off[t * L1 + q] : 0;
-    R.ms[u] = q < d ? __ldg(tv.meta + t * d + q) : 0u;
-  }
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src));
 }
-__device__ __forceinline__ void tile_regs_store(const SketchTiles& tv, int64_t t, const TileRegs& R, int* of,
-                                                uint32_t* ms, uint16_t* es) {
+
+// Starts the copy of the bin lists of step k's tile into its buffers
+// (tile_wait ends it; the bytes are those of tile_stage).  Issued a tile
+// ahead: staged at the tile's start instead, the bounds' load, then those of
+// the lists, were waited for one after the other (FP32 update, n = 4.1e6,
+// d = 96, one basis column: 84 -> 64 us; 26 columns: 150 -> 134 us; pairs,
+// n = 1e6, d = 320, one column: 30 -> 23 us).
+template <class TV>
+__device__ __forceinline__ void tile_fetch(uint8_t* sm, const TileSmem& lay, const SketchTiles& tv,
+                                           const TileRange& tr, int k) {
+  const TileBuf<TV> b(sm, lay, tv, k);
   const int L1 = tv.L + 1, d = tv.d;
-  const int cnt = (int)(tv.row[t + 1] - tv.row[t]) * tv.zeta;
-#pragma unroll
-  for (int u = 0; u < kStageRegs; ++u) {
-    const int q = threadIdx.x + u * 512;
-    if (q * 8 + 8 <= cnt) reinterpret_cast<uint4*>(es)[q] = R.e[u];
-    else if (q * 8 < cnt) {   // the ragged end of the last tile
-      const uint32_t wd[4] = {R.e[u].x, R.e[u].y, R.e[u].z, R.e[u].w};
-#pragma unroll
-      for (int k = 0; k < 8; ++k)
-        if (q * 8 + k < cnt) es[q * 8 + k] = (uint16_t)((wd[k >> 1] >> (16 * (k & 1))) & 0xFFFFu);
-    }
+  const int64_t t = tr.t0 + tr.at(k), e0 = tr.row(k) * tv.zeta;
+  const int cnt = tr.rows(k) * tv.zeta;
+  const int* og = tv.off + t * L1;
+  const uint32_t* mg = tv.meta + t * d;
+  const uint16_t* eg = tv.ent + e0;
+  int q0;
+  if ((e0 & 7) == 0) {
+    for (int q = threadIdx.x; q < cnt >> 3; q += blockDim.x) cp_async16(b.es + 8 * q, eg + 8 * q);
+    q0 = cnt & ~7;
+  } else {                       // tiles start at even rows: 4-byte aligned
+    for (int q = threadIdx.x; q < cnt >> 1; q += blockDim.x) cp_async4(b.es + 2 * q, eg + 2 * q);
+    q0 = cnt & ~1;
   }
-#pragma unroll
-  for (int u = 0; u < 2; ++u) {
-    const int q = threadIdx.x + u * 512;
-    if (q < L1) of[q] = R.of[u];
-    if (q < d) ms[q] = R.ms[u];
+  if ((d & 3) == 0) {
+    for (int q = threadIdx.x; q < d >> 2; q += blockDim.x) cp_async16(b.ms + 4 * q, mg + 4 * q);
+  } else {
+    for (int q = threadIdx.x; q < d; q += blockDim.x) cp_async4(b.ms + q, mg + q);
   }
+  for (int q = threadIdx.x; q < L1; q += blockDim.x) cp_async4(b.of + q, og + q);
+  for (int q = q0 + threadIdx.x; q < cnt; q += blockDim.x) b.es[q] = eg[q];
+}
+__device__ __forceinline__ void tile_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// The end of step k: every value of the tile is in its buffer.  Starts the
+// next tile's lists (their buffers were last read before this barrier) and
+// adds this tile's sums.
+template <class TV>
+__device__ __forceinline__ void tile_finish(uint8_t* sm, const TileSmem& lay, const SketchTiles& tv,
+                                            const TileRange& tr, int k, float2* acc) {
+  tile_wait();
+  __syncthreads();
+  if (k + 1 < tr.nt) tile_fetch<TV>(sm, lay, tv, tr, k + 1);
+  const TileBuf<TV> b(sm, lay, tv, k);
+  tile_gather(tv.d, tv.H, b.v, b.of, b.ms, b.es, acc);
+}
+
+// Asks for p[0 .. cnt) to be brought into L2 (16-byte units; p[cnt] up to the
+// next unit is inside the padded column).
+template <class TU>
+__device__ __forceinline__ void prefetch_rows(const TU* p, int cnt) {
+  const uint64_t a = reinterpret_cast<uint64_t>(p) & ~(uint64_t)15;
+  const uint64_t e = (reinterpret_cast<uint64_t>(p + cnt) + 15) & ~(uint64_t)15;
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a), "r"((uint32_t)(e - a)));
 }
 
 __device__ __forceinline__ void tile_write_part(const float2* acc, int d, double* part) {
@@ -454,21 +563,17 @@ __global__ void __launch_bounds__(512) k_df_spmv_sketch(
     const TU* __restrict__ x, TU* __restrict__ w, const SketchTiles tv, double* __restrict__ part) {
   static_assert(kTileRows == 1024, "two rows per thread of a 512-thread CTA");
   extern __shared__ __align__(16) uint8_t smraw[];
-  const int d = tv.d, L1 = tv.L + 1;
+  const int d = tv.d;
   const TileSmem lay = tile_smem_layout(d, tv.L, 0, tv.zeta);
   float2* acc = reinterpret_cast<float2*>(smraw + lay.acc);
   if (SK)
     for (int r = threadIdx.x; r < d; r += blockDim.x) acc[r] = make_float2(0.f, 0.f);
-  const int t0 = tv.ctile[blockIdx.x], t1 = tv.ctile[blockIdx.x + 1];
-  for (int t = t0; t < t1; ++t) {
-    const int buf = (t - t0) & 1;
-    float2* v = reinterpret_cast<float2*>(smraw + lay.vb) + buf * kTileRows;
-    int* of = reinterpret_cast<int*>(smraw + lay.offs) + buf * L1;
-    uint32_t* ms = reinterpret_cast<uint32_t*>(smraw + lay.ms) + buf * d;
-    uint16_t* es = reinterpret_cast<uint16_t*>(smraw + lay.es) + (size_t)buf * kTileRows * tv.zeta;
-    const int64_t r0 = tv.row[t];
-    const int rows = (int)(tv.row[t + 1] - r0);
-    if (SK) tile_stage(tv, t, r0, rows, of, ms, es);
+  const TileRange tr(tv, false);
+  if (SK && tr.nt > 0) tile_fetch<TU>(smraw, lay, tv, tr, 0);
+  for (int k = 0; k < tr.nt; ++k) {
+    TU* v = TileBuf<TU>(smraw, lay, tv, k).v;
+    const int64_t r0 = tr.row(k);
+    const int rows = tr.rows(k);
     const int la = threadIdx.x, lb = threadIdx.x + 512;
     int pa = 0, ea = 0, pb = 0, eb = 0;
     if (la < rows) { pa = rowptr[r0 + la]; ea = rowptr[r0 + la + 1]; }
@@ -497,12 +602,9 @@ __global__ void __launch_bounds__(512) k_df_spmv_sketch(
         if (cb[u] >= 0) mac_st<TA, TU>(vbv[u], xb[u], sb, tb);
       }
     }
-    if (la < rows) v[la] = stv(w + r0 + la, df_norm(sa, ta));
-    if (lb < rows) v[lb] = stv(w + r0 + lb, df_norm(sb, tb));
-    if (SK) {
-      __syncthreads();
-      tile_gather<sizeof(TU) == 8>(d, tv.H, v, of, ms, es, acc);
-    }
+    if (la < rows) tile_put(v + la, stv(w + r0 + la, df_norm(sa, ta)));
+    if (lb < rows) tile_put(v + lb, stv(w + r0 + lb, df_norm(sb, tb)));
+    if (SK) tile_finish<TU>(smraw, lay, tv, tr, k, acc);
   }
   if (SK) tile_write_part(acc, d, part);
 }
@@ -520,21 +622,17 @@ __global__ void __launch_bounds__(512) k_df_spmv_ell(
     const TU* __restrict__ x, TU* __restrict__ w, const SketchTiles tv, double* __restrict__ part) {
   static_assert(kTileRows == 1024, "two rows per thread of a 512-thread CTA");
   extern __shared__ __align__(16) uint8_t smraw[];
-  const int d = tv.d, L1 = tv.L + 1;
+  const int d = tv.d;
   const TileSmem lay = tile_smem_layout(d, tv.L, 0, tv.zeta);
   float2* acc = reinterpret_cast<float2*>(smraw + lay.acc);
   if (SK)
     for (int r = threadIdx.x; r < d; r += blockDim.x) acc[r] = make_float2(0.f, 0.f);
-  const int t0 = tv.ctile[blockIdx.x], t1 = tv.ctile[blockIdx.x + 1];
-  for (int t = t0; t < t1; ++t) {
-    const int buf = (t - t0) & 1;
-    float2* v = reinterpret_cast<float2*>(smraw + lay.vb) + buf * kTileRows;
-    int* of = reinterpret_cast<int*>(smraw + lay.offs) + buf * L1;
-    uint32_t* ms = reinterpret_cast<uint32_t*>(smraw + lay.ms) + buf * d;
-    uint16_t* es = reinterpret_cast<uint16_t*>(smraw + lay.es) + (size_t)buf * kTileRows * tv.zeta;
-    const int64_t r0 = tv.row[t];
-    const int rows = (int)(tv.row[t + 1] - r0);
-    if (SK) tile_stage(tv, t, r0, rows, of, ms, es);
+  const TileRange tr(tv, false);
+  if (SK && tr.nt > 0) tile_fetch<TU>(smraw, lay, tv, tr, 0);
+  for (int k = 0; k < tr.nt; ++k) {
+    TU* v = TileBuf<TU>(smraw, lay, tv, k).v;
+    const int64_t r0 = tr.row(k);
+    const int rows = tr.rows(k);
     const int la = threadIdx.x, lb = threadIdx.x + 512;
     const bool oka = la < rows, okb = lb < rows;
     const int64_t ia = r0 + la, ib = r0 + lb;
@@ -584,12 +682,9 @@ __global__ void __launch_bounds__(512) k_df_spmv_ell(
         if (cb[u] >= 0) mac_st<TA, TU>(vbv[u], xb[u], sb, tb);
       }
     }
-    if (oka) v[la] = stv(w + ia, df_norm(sa, ta));
-    if (okb) v[lb] = stv(w + ib, df_norm(sb, tb));
-    if (SK) {
-      __syncthreads();
-      tile_gather<sizeof(TU) == 8>(d, tv.H, v, of, ms, es, acc);
-    }
+    if (oka) tile_put(v + la, stv(w + ia, df_norm(sa, ta)));
+    if (okb) tile_put(v + lb, stv(w + ib, df_norm(sb, tb)));
+    if (SK) tile_finish<TU>(smraw, lay, tv, tr, k, acc);
   }
   if (SK) tile_write_part(acc, d, part);
 }
@@ -603,23 +698,19 @@ __global__ void __launch_bounds__(512) k_df_spmv_warp(const int32_t* __restrict_
                                                       const TU* __restrict__ x, TU* __restrict__ w,
                                                       const SketchTiles tv, double* __restrict__ part) {
   extern __shared__ __align__(16) uint8_t smraw[];
-  const int d = tv.d, L1 = tv.L + 1;
+  const int d = tv.d;
   const TileSmem lay = tile_smem_layout(d, tv.L, 0, tv.zeta);
   float2* acc = reinterpret_cast<float2*>(smraw + lay.acc);
   if (SK)
     for (int r = threadIdx.x; r < d; r += blockDim.x) acc[r] = make_float2(0.f, 0.f);
   // groups of LPR lanes per row (LPR = 32: a warp per row)
   const int grp = threadIdx.x / LPR, lane = threadIdx.x % LPR, ngrp = blockDim.x / LPR;
-  const int t0 = tv.ctile[blockIdx.x], t1 = tv.ctile[blockIdx.x + 1];
-  for (int t = t0; t < t1; ++t) {
-    const int buf = (t - t0) & 1;
-    float2* v = reinterpret_cast<float2*>(smraw + lay.vb) + buf * kTileRows;
-    int* of = reinterpret_cast<int*>(smraw + lay.offs) + buf * L1;
-    uint32_t* ms = reinterpret_cast<uint32_t*>(smraw + lay.ms) + buf * d;
-    uint16_t* es = reinterpret_cast<uint16_t*>(smraw + lay.es) + (size_t)buf * kTileRows * tv.zeta;
-    const int64_t r0 = tv.row[t];
-    const int rows = (int)(tv.row[t + 1] - r0);
-    if (SK) tile_stage(tv, t, r0, rows, of, ms, es);
+  const TileRange tr(tv, false);
+  if (SK && tr.nt > 0) tile_fetch<TU>(smraw, lay, tv, tr, 0);
+  for (int k = 0; k < tr.nt; ++k) {
+    TU* v = TileBuf<TU>(smraw, lay, tv, k).v;
+    const int64_t r0 = tr.row(k);
+    const int rows = tr.rows(k);
     const int nit = (rows + ngrp - 1) / ngrp;        // the same trip count for every lane
     for (int it = 0; it < nit; ++it) {
       const int l = it * ngrp + grp;
@@ -640,12 +731,9 @@ __global__ void __launch_bounds__(512) k_df_spmv_warp(const int32_t* __restrict_
         sh = ss;
         sl = sl + t2 + e;
       }
-      if (l < rows && lane == 0) v[l] = stv(w + r0 + l, df_norm(sh, sl));
+      if (l < rows && lane == 0) tile_put(v + l, stv(w + r0 + l, df_norm(sh, sl)));
     }
-    if (SK) {
-      __syncthreads();
-      tile_gather<sizeof(TU) == 8>(d, tv.H, v, of, ms, es, acc);
-    }
+    if (SK) tile_finish<TU>(smraw, lay, tv, tr, k, acc);
   }
   if (SK) tile_write_part(acc, d, part);
 }
@@ -880,29 +968,17 @@ __global__ void __launch_bounds__(512, 2) k_df_spmv_dia(const DiaOffs offs, int 
                                                      double* __restrict__ part) {
   static_assert(kTileRows == 1024, "two rows per thread of a 512-thread CTA");
   extern __shared__ __align__(16) uint8_t smraw[];
-  const int d = tv.d, L1 = tv.L + 1;
+  const int d = tv.d;
   const TileSmem lay = tile_smem_layout(d, tv.L, 0, tv.zeta);
   float2* acc = reinterpret_cast<float2*>(smraw + lay.acc);
   if (SK)
     for (int r = threadIdx.x; r < d; r += blockDim.x) acc[r] = make_float2(0.f, 0.f);
-  const int t0 = tv.ctile[blockIdx.x], t1 = tv.ctile[blockIdx.x + 1];
-  const bool regs = SK && tile_regs_fit(tv);
-  TileRegs R;
-  if (regs && t0 < t1) tile_regs_load(tv, t0, R);
-  for (int t = t0; t < t1; ++t) {
-    const int buf = (t - t0) & 1;
-    float2* v = reinterpret_cast<float2*>(smraw + lay.vb) + buf * kTileRows;
-    int* of = reinterpret_cast<int*>(smraw + lay.offs) + buf * L1;
-    uint32_t* ms = reinterpret_cast<uint32_t*>(smraw + lay.ms) + buf * d;
-    uint16_t* es = reinterpret_cast<uint16_t*>(smraw + lay.es) + (size_t)buf * kTileRows * tv.zeta;
-    const int64_t r0 = tv.row[t];
-    const int rows = (int)(tv.row[t + 1] - r0);
-    if (regs) {            // this tile's lists were loaded during the previous tile
-      tile_regs_store(tv, t, R, of, ms, es);
-      if (t + 1 < t1) tile_regs_load(tv, t + 1, R);
-    } else if (SK) {
-      tile_stage(tv, t, r0, rows, of, ms, es);
-    }
+  const TileRange tr(tv, false);
+  if (SK && tr.nt > 0) tile_fetch<TU>(smraw, lay, tv, tr, 0);
+  for (int k = 0; k < tr.nt; ++k) {
+    TU* v = TileBuf<TU>(smraw, lay, tv, k).v;
+    const int64_t r0 = tr.row(k);
+    const int rows = tr.rows(k);
     const int la = threadIdx.x, lb = threadIdx.x + 512;
     const bool oka = la < rows, okb = lb < rows;
     const int64_t ia = r0 + la, ib = r0 + lb;
@@ -964,12 +1040,11 @@ __global__ void __launch_bounds__(512, 2) k_df_spmv_dia(const DiaOffs offs, int 
         }
       }
     }
-    if (oka) v[la] = stv(w + ia, df_norm(sa, ta));
-    if (okb) v[lb] = stv(w + ib, df_norm(sb, tb));
-    if (SK) {
-      __syncthreads();
-      tile_gather<sizeof(TU) == 8>(d, tv.H, v, of, ms, es, acc);
-    }
+    if (oka) tile_put(v + la, stv(w + ia, df_norm(sa, ta)));
+    if (okb) tile_put(v + lb, stv(w + ib, df_norm(sb, tb)));
+    if (SK && k + 1 < tr.nt && (int)threadIdx.x < D)   // the next tile's diagonals on their way to L2
+      prefetch_rows(dv + tr.row(k + 1) + threadIdx.x * ldd, tr.rows(k + 1));
+    if (SK) tile_finish<TU>(smraw, lay, tv, tr, k, acc);
   }
   if (SK) tile_write_part(acc, d, part);
 }
@@ -1030,7 +1105,7 @@ __global__ void __launch_bounds__(512, MINB) k_df_update_sketch(
     const SketchTiles tv, double* __restrict__ part) {
   constexpr bool SK = MODE == 1;
   extern __shared__ __align__(16) uint8_t smraw[];
-  const int d = tv.d, L1 = tv.L + 1;
+  const int d = tv.d;
   const TileSmem lay = tile_smem_layout(d, tv.L, c, tv.zeta);
   float2* acc = reinterpret_cast<float2*>(smraw + lay.acc);
   float2* rsh = reinterpret_cast<float2*>(smraw + lay.rsh);
@@ -1040,21 +1115,15 @@ __global__ void __launch_bounds__(512, MINB) k_df_update_sketch(
   double ss = 0.0;
   __syncthreads();
   const float2 sc = sj[0];
-  const int t0 = tv.ctile[blockIdx.x], t1 = tv.ctile[blockIdx.x + 1];
   // The second half of the grid takes its tiles last to first: the two CTAs
   // an SM holds (blocks b and b + G/2) then meet their short last tile at
   // different times, and the SM keeps more loads in flight.
-  const bool rev = blockIdx.x >= gridDim.x / 2;
-  for (int tt = t0; tt < t1; ++tt) {
-    const int t = rev ? t1 - 1 - (tt - t0) : tt;
-    const int buf = (tt - t0) & 1;
-    float2* v = reinterpret_cast<float2*>(smraw + lay.vb) + buf * kTileRows;
-    int* of = reinterpret_cast<int*>(smraw + lay.offs) + buf * L1;
-    uint32_t* ms = reinterpret_cast<uint32_t*>(smraw + lay.ms) + buf * d;
-    uint16_t* es = reinterpret_cast<uint16_t*>(smraw + lay.es) + (size_t)buf * kTileRows * tv.zeta;
-    const int64_t r0 = tv.row[t];
-    const int rows = (int)(tv.row[t + 1] - r0);
-    if (SK) tile_stage(tv, t, r0, rows, of, ms, es);
+  const TileRange tr(tv, blockIdx.x >= gridDim.x / 2);
+  if (SK && tr.nt > 0) tile_fetch<TU>(smraw, lay, tv, tr, 0);
+  for (int k = 0; k < tr.nt; ++k) {
+    TU* v = TileBuf<TU>(smraw, lay, tv, k).v;
+    const int64_t r0 = tr.row(k);
+    const int rows = tr.rows(k);
     for (int l = 2 * threadIdx.x; l < rows; l += 2 * blockDim.x) {
       const int64_t i = r0 + l;
       float s0 = 0.f, t0a = 0.f, s1 = 0.f, t1a = 0.f;
@@ -1085,18 +1154,19 @@ __global__ void __launch_bounds__(512, MINB) k_df_update_sketch(
         mac_st<TU, float2>(bb, r, s1, t1a);
       }
       const float2 v0 = stv(U + i + (int64_t)c * ldu, df_norm(s0, t0a));
-      v[l] = v0;
+      tile_put(v + l, v0);
       if (MODE == 2) { const double x = df_to_double(v0); ss = fma(x, x, ss); }
       if (l + 1 < rows) {
         const float2 v1 = stv(U + i + 1 + (int64_t)c * ldu, df_norm(s1, t1a));
-        v[l + 1] = v1;
+        tile_put(v + l + 1, v1);
         if (MODE == 2) { const double x = df_to_double(v1); ss = fma(x, x, ss); }
       }
     }
-    if (SK) {
-      __syncthreads();
-      tile_gather<sizeof(TU) == 8>(d, tv.H, v, of, ms, es, acc);
-    }
+    // the next tile's first batch of columns on its way to L2 while this
+    // tile's sums are formed
+    if (SK && k + 1 < tr.nt && (int)threadIdx.x <= min(c, UNR))
+      prefetch_rows(U + tr.row(k + 1) + (int64_t)(threadIdx.x == 0 ? c : threadIdx.x - 1) * ldu, tr.rows(k + 1));
+    if (SK) tile_finish<TU>(smraw, lay, tv, tr, k, acc);
   }
   if (SK) tile_write_part(acc, d, part);
   if (MODE == 2) {
@@ -1641,23 +1711,18 @@ template <class TU>
 __global__ void __launch_bounds__(512) k_df_sketch_vec(const TU* __restrict__ x, const SketchTiles tv,
                                                        double* __restrict__ part) {
   extern __shared__ __align__(16) uint8_t smraw[];
-  const int d = tv.d, L1 = tv.L + 1;
+  const int d = tv.d;
   const TileSmem lay = tile_smem_layout(d, tv.L, 0, tv.zeta);
   float2* acc = reinterpret_cast<float2*>(smraw + lay.acc);
   for (int r = threadIdx.x; r < d; r += blockDim.x) acc[r] = make_float2(0.f, 0.f);
-  const int t0 = tv.ctile[blockIdx.x], t1 = tv.ctile[blockIdx.x + 1];
-  for (int t = t0; t < t1; ++t) {
-    const int buf = (t - t0) & 1;
-    float2* v = reinterpret_cast<float2*>(smraw + lay.vb) + buf * kTileRows;
-    int* of = reinterpret_cast<int*>(smraw + lay.offs) + buf * L1;
-    uint32_t* ms = reinterpret_cast<uint32_t*>(smraw + lay.ms) + buf * d;
-    uint16_t* es = reinterpret_cast<uint16_t*>(smraw + lay.es) + (size_t)buf * kTileRows * tv.zeta;
-    const int64_t r0 = tv.row[t];
-    const int rows = (int)(tv.row[t + 1] - r0);
-    tile_stage(tv, t, r0, rows, of, ms, es);
-    for (int l = threadIdx.x; l < rows; l += blockDim.x) v[l] = ldv(x + r0 + l);
-    __syncthreads();
-    tile_gather<sizeof(TU) == 8>(d, tv.H, v, of, ms, es, acc);
+  const TileRange tr(tv, false);
+  if (tr.nt > 0) tile_fetch<TU>(smraw, lay, tv, tr, 0);
+  for (int k = 0; k < tr.nt; ++k) {
+    TU* v = TileBuf<TU>(smraw, lay, tv, k).v;
+    const int64_t r0 = tr.row(k);
+    const int rows = tr.rows(k);
+    for (int l = threadIdx.x; l < rows; l += blockDim.x) v[l] = x[r0 + l];
+    tile_finish<TU>(smraw, lay, tv, tr, k, acc);
   }
   tile_write_part(acc, d, part);
 }
@@ -1716,7 +1781,7 @@ __global__ void __launch_bounds__(512, 2) k_df_sketch_cols(const TS* __restrict_
         if (lb < rows) b = xn[lb];
       }
       __syncthreads();
-      tile_gather<true>(d, tv.H, v, of, ms, es, acc + (size_t)q * d);
+      tile_gather(d, tv.H, v, of, ms, es, acc + (size_t)q * d);
     }
   }
   __syncthreads();
@@ -2188,7 +2253,7 @@ __global__ void __launch_bounds__(512) k_df_expand_small(const SmallArgs a) {
     for (int q = 0; q < t1 - t0; ++q) {
       const int t = rev ? t1 - t0 - 1 - q : q;
       __syncthreads();
-      tile_gather<true>(d, tv.H, v + t * kTileRows, of + t * L1, ms + t * d, es + (size_t)t * kTileRows * tv.zeta, acc);
+      tile_gather(d, tv.H, v + t * kTileRows, of + t * L1, ms + t * d, es + (size_t)t * kTileRows * tv.zeta, acc);
     }
     __syncthreads();
     for (int r = tid; r < d; r += NT) {
