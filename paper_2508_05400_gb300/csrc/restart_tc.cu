@@ -8,17 +8,14 @@
 // below 2^-32 |u| |q|); every bf16 x bf16 product is exact and the sums are
 // FP32 in tensor memory, so the result has FP32-class accuracy.
 //
-// One CTA (256 threads) owns tiles of 128 rows; per tile the K dimension
-// (the nin input columns, padded to kKc) streams through two shared-memory
-// stages of 32 columns: all threads load and split a stage (FP32 loads,
-// coalesced along the rows, issued one stage ahead into registers) into the
-// canonical K-major no-swizzle layout,
-// thread 0 issues 2 x 6 MMAs of 128 x N x 16 on it and commits them to the
-// stage's mbarrier, which the next load of that stage waits for.  The
-// epilogue reads the 128 x N FP32 accumulator with tcgen05.ld (warps 0-3 and
-// 4-7 take alternate 16-column groups of their lane quarter) and writes the
-// outputs; every read of a tile's rows precedes its writes, so the product
-// may be formed in place.  All waits are bounded (RKS_FLAG_TIMEOUT).
+// A CTA owns tiles of 128 rows; per tile the K dimension (the nin input
+// columns, padded) streams through shared-memory stages of one K-step of 16
+// columns: FP32 loads, coalesced along the rows, three K-steps ahead in
+// registers, split into a K-major no-swizzle layout; 6 MMAs of 128 x N x 16
+// per stage.  The epilogue reads the 128 x N FP32 accumulator with tcgen05.ld
+// and writes the outputs; every read of a tile's rows precedes its writes, so
+// the product may be formed in place.  All waits are bounded
+// (RKS_FLAG_TIMEOUT).
 
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -36,10 +33,12 @@ namespace rks {
 namespace {
 
 constexpr int kM = 128;           // rows per tile (MMA M)
-constexpr int kKc = 32;           // input columns per stage (two MMA K-steps)
-constexpr int kThreads = 256;
-constexpr int kStageSplit = kM * kKc * 2;   // bytes of one split of one stage
-constexpr int kStage = 3 * kStageSplit;
+constexpr int kKc = 32;           // Kp is padded to a multiple of this
+constexpr int kThreads = 256;     // splitters of the FP32 product; one more warp issues the MMAs
+constexpr int kF32All = kThreads + 32;
+constexpr int kF32Stages = 3;
+constexpr int kF32Split = kM * 16 * 2;      // bytes of one split of one stage (a K-step of 16 columns)
+constexpr int kF32Stage = 3 * kF32Split;
 constexpr int kTmemCols = 64;
 
 // Byte offset of element (r, k) of a K-major, no-swizzle tile with `rows`
@@ -57,6 +56,13 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
 // descriptor version 1 (bits 46-48), no swizzle.
 __device__ __forceinline__ uint64_t sdesc(uint32_t addr) {
   return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)(128 >> 4) << 16) | ((uint64_t)(256 >> 4) << 32) |
+         (1ull << 46);
+}
+
+// Shared-memory matrix descriptor of a K-major, no-swizzle operand whose
+// rows lie 16 bytes apart: SBO (next 8 rows) 128 bytes, LBO (next 8 columns) lbo.
+__device__ __forceinline__ uint64_t sdesc_rows(uint32_t addr, uint32_t lbo) {
+  return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo >> 4) << 16) | ((uint64_t)(128 >> 4) << 32) |
          (1ull << 46);
 }
 
@@ -82,6 +88,10 @@ __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::be
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
+__device__ __forceinline__ void mbar_arrive(uint32_t mbar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(mbar) : "memory");
+}
+
 __device__ __forceinline__ bool mbar_try(uint32_t mbar, uint32_t parity) {
   uint32_t done;
   asm volatile(
@@ -105,18 +115,6 @@ __device__ __noinline__ bool mbar_wait_slow(uint32_t mbar, uint32_t parity, int*
 // Bounded wait for the completion of the mbarrier phase with this parity.
 __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, int* flag) {
   return mbar_try(mbar, parity) || mbar_wait_slow(mbar, parity, flag);
-}
-
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
-  uint32_t r[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
 }
 
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
@@ -144,7 +142,21 @@ __host__ __device__ constexpr int pair_b(int p) { return p == 1 || p == 4 ? 1 : 
 // out[i, o] = sum_l in[i, l] Q'[l, o] for i < n, o < nout; then, when mvsrc
 // is given, mvdst[i] = mvsrc[i].  bimg: the three bf16 splits of Q' (Kp x N,
 // zero padded) in the canonical layout, split j at byte j * Kp * N * 2.
-__global__ void __launch_bounds__(kThreads, 3) k_tc_restart_f32(int64_t n, const float* in, float* out, int64_t ldu,
+//
+// Warps 0..7 load and split (a thread one row and 8 of a K-step's 16 columns,
+// three K-steps ahead, in three sets of registers taken in turn: a set copied
+// to another would wait for its loads; one 16-byte store per split) and run
+// the epilogue; warp 8 issues the MMAs.  Per stage: full (every splitter arrives)
+// and empty (the MMA commit arrives), per tile: done and tfree.  A thread
+// whose bounded wait gave up skips its later waits and otherwise goes on, so
+// that every barrier keeps its count.
+//
+// 4 096 000 x 150 -> 51 columns: 1750 us with CTA barriers around every stage
+// and one CTA per SM; 1529 us with the MMAs issued by a warp of their own and
+// loads three steps ahead; 944 us (3.5 TB/s) with the CTAs an SM has room for
+// (two here).  The MMAs of a tile are 60 of 128 x 64 x 16, a seventh of the
+// tensor pipe; bound by the split's shared-memory traffic and loads in flight.
+__global__ void __launch_bounds__(kF32All, 3) k_tc_restart_f32(int64_t n, const float* in, float* out, int64_t ldu,
                                                                 int nin, int Kp, int N, int nout,
                                                                 const uint4* __restrict__ bimg, const float* mvsrc,
                                                                 float* mvdst, int* flag) {
@@ -153,17 +165,21 @@ __global__ void __launch_bounds__(kThreads, 3) k_tc_restart_f32(int64_t n, const
   const int bbytes = 3 * Kp * N * 2;
   uint8_t* sB = smem;
   uint8_t* sA = smem + ((bbytes + 1023) & ~1023);
-  uint64_t* mbar = reinterpret_cast<uint64_t*>(sA + 2 * kStage);
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + 3);
+  uint64_t* mbar = reinterpret_cast<uint64_t*>(sA + kF32Stages * kF32Stage);   // full[], empty[], done, tfree
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + 2 * kF32Stages + 2);
+  const uint32_t full0 = smem_u32(mbar), empty0 = smem_u32(mbar + kF32Stages);
+  const uint32_t done_b = smem_u32(mbar + 2 * kF32Stages), tfree_b = smem_u32(mbar + 2 * kF32Stages + 1);
 
-  for (int t = tid; t < bbytes / 16; t += kThreads) reinterpret_cast<uint4*>(sB)[t] = bimg[t];
+  for (int t = tid; t < bbytes / 16; t += kF32All) reinterpret_cast<uint4*>(sB)[t] = bimg[t];
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
                  "r"(kTmemCols));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   if (tid == 0) {
-    for (int s = 0; s < 3; ++s) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(mbar + s)));
+    for (int s = 0; s < 2 * kF32Stages + 2; ++s)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(mbar + s)),
+                   "r"(s < kF32Stages || s == 2 * kF32Stages + 1 ? kThreads : 1));
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   fence_async_smem();
@@ -171,126 +187,138 @@ __global__ void __launch_bounds__(kThreads, 3) k_tc_restart_f32(int64_t n, const
   __syncthreads();
   fence_after();
   const uint32_t tmem = *tslot;
-  const uint32_t idesc = idesc_bf16(N);
-  const uint32_t sA32 = smem_u32(sA), sB32 = smem_u32(sB);
-  const int nk = Kp / kKc;
+  const int nk = Kp / 16;
   const int64_t ntiles = (n + kM - 1) / kM;
-  int g = 0;                 // stages filled so far (all tiles)
-  uint32_t dpar = 0;         // parity of the accumulator-done barrier
   bool ok = true;
-  const int r = tid & (kM - 1), kh = tid >> 7;   // loader: row, half of the stage's 32 columns
 
-  // the 16 values (one row, half a stage) that this thread loads for stage kc of a tile
-  auto load16 = [&](int64_t tile, int kc, float* v) {
-    const int64_t i = tile * kM + r;
-    const int l0 = kc * kKc + kh * 16;
-#pragma unroll
-    for (int u = 0; u < 16; ++u) {
-      const int l = l0 + u;
-      v[u] = (tile < ntiles && i < n && l < nin) ? in[i + (int64_t)l * ldu] : 0.f;
-    }
-  };
-  // loads run two stages ahead of the split (three register stages): one
-  // stage of work is shorter than the DRAM latency
-  auto next_step = [&](int64_t& t, int& k) {
-    if (++k == nk) { k = 0; t += gridDim.x; }
-  };
-  float v[16], vn[16], vnn[16];
-  int64_t pt = blockIdx.x;
-  int pk = 0;
-  load16(pt, pk, v);
-  next_step(pt, pk);
-  load16(pt, pk, vn);
-  for (int64_t tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
-    for (int kc = 0; kc < nk && ok; ++kc, ++g) {
-      const int s = g & 1;
-      next_step(pt, pk);
-      load16(pt, pk, vnn);
-      if (g >= 2) ok = mbar_wait(smem_u32(mbar + s), (uint32_t)(((g - 2) >> 1) & 1), flag);
-      ok = __syncthreads_and(ok);
-      if (!ok) break;
-      uint8_t* st = sA + s * kStage;
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        uint32_t w[3][4];
-#pragma unroll
-        for (int u = 0; u < 8; u += 2) {
-          uint32_t p[3][2];
-#pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            const float x = v[h * 8 + u + e];
-            const __nv_bfloat16 a = __float2bfloat16_rn(x);
-            const float r1 = x - __bfloat162float(a);
-            const __nv_bfloat16 b = __float2bfloat16_rn(r1);
-            const __nv_bfloat16 c = __float2bfloat16_rn(r1 - __bfloat162float(b));
-            p[0][e] = bf16_bits(a);
-            p[1][e] = bf16_bits(b);
-            p[2][e] = bf16_bits(c);
-          }
-#pragma unroll
-          for (int q = 0; q < 3; ++q) w[q][u >> 1] = p[q][0] | (p[q][1] << 16);
-        }
-        const uint32_t off = canon_off(r, kh * 16 + h * 8, kM);
-#pragma unroll
-        for (int q = 0; q < 3; ++q)
-          *reinterpret_cast<uint4*>(st + q * kStageSplit + off) = make_uint4(w[q][0], w[q][1], w[q][2], w[q][3]);
-      }
-      fence_async_smem();
-      __syncthreads();
-      if (tid == 0) {
+  if (warp == kThreads / 32) {
+    // ---- MMA issuer
+    if (lane == 0) {
+      const uint32_t idesc = idesc_bf16(N);
+      const uint32_t sA32 = smem_u32(sA), sB32 = smem_u32(sB);
+      int s = 0, tcount = 0;
+      uint32_t ph = 0;
+      for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++tcount) {
+        if (tcount > 0 && ok) ok = mbar_wait(tfree_b, (uint32_t)((tcount - 1) & 1), flag);   // accumulator read
         fence_after();
+        for (int ks = 0; ks < nk; ++ks) {
+          if (ok) ok = mbar_wait(full0 + 8u * s, ph, flag);
+          fence_after();
+          if (ok) {
 #pragma unroll
-        for (int kk = 0; kk < 2; ++kk) {
-          const int ks = kc * 2 + kk;   // K-step of 16 within the padded K
+            for (int pr = 0; pr < 6; ++pr) {
+              const uint64_t a = sdesc_rows(sA32 + s * kF32Stage + pair_a(pr) * kF32Split, 2048);
+              const uint64_t b = sdesc(sB32 + pair_b(pr) * Kp * N * 2 + ks * N * 32);
+              mma_bf16(tmem, a, b, idesc, (ks | pr) ? 1u : 0u);
+            }
+          }
+          mma_commit(empty0 + 8u * s);
+          if (ks == nk - 1) mma_commit(done_b);
+          if (++s == kF32Stages) { s = 0; ph ^= 1u; }
+        }
+      }
+      // every issued MMA has completed before the accumulator is freed: the
+      // last commit made to each stage's barrier
+      const int64_t g = (int64_t)tcount * nk;
+      for (int q = 0; q < kF32Stages; ++q) {
+        const int64_t c = (g - q + kF32Stages - 1) / kF32Stages;
+        if (g > q && c > 0) (void)mbar_wait(empty0 + 8u * q, (uint32_t)((c - 1) & 1), flag);
+      }
+    }
+    __syncwarp();
+  } else {
+    const int r = tid & (kM - 1), c8 = (tid >> 7) * 8;
+    int s = 0, ks = 0, filled = 0;
+    uint32_t ph = 1, dpar = 0;             // parity of empty[s]: the first round passes
+    int64_t tile = blockIdx.x;
+    // the 8 values (one row) of K-step pk of tile pt; then on to the next K-step
+    int64_t pt = tile;
+    int pk = 0;
+    auto load8 = [&](float* v) {
+      if (pt < ntiles) {
+        const int64_t i = pt * kM + r;
+        const int c = pk * 16 + c8;
+        const float* p = in + (i < n ? i : n - 1) + (int64_t)c * ldu;
+        if (c + 8 <= nin) {
 #pragma unroll
-          for (int pr = 0; pr < 6; ++pr) {
-            const uint64_t a = sdesc(sA32 + s * kStage + pair_a(pr) * kStageSplit + kk * kM * 32);
-            const uint64_t b = sdesc(sB32 + pair_b(pr) * Kp * N * 2 + ks * N * 32);
-            mma_bf16(tmem, a, b, idesc, (kc | kk | pr) ? 1u : 0u);
+          for (int u = 0; u < 8; ++u) v[u] = p[u * ldu];
+        } else {
+#pragma unroll
+          for (int u = 0; u < 8; ++u) v[u] = c + u < nin ? p[u * ldu] : 0.f;
+        }
+      }
+      if (++pk == nk) { pk = 0; pt += gridDim.x; }
+    };
+    // one K-step: its values to shared memory, then the loads of three
+    // K-steps later into the same registers
+    auto step = [&](float* v) {
+      uint32_t w[3][4];
+#pragma unroll
+      for (int u = 0; u < 8; u += 2) {
+        uint32_t p[3][2];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const float x = v[u + e];
+          const __nv_bfloat16 a = __float2bfloat16_rn(x);
+          const float r1 = x - __bfloat162float(a);
+          const __nv_bfloat16 b = __float2bfloat16_rn(r1);
+          const __nv_bfloat16 c = __float2bfloat16_rn(r1 - __bfloat162float(b));
+          p[0][e] = bf16_bits(a);
+          p[1][e] = bf16_bits(b);
+          p[2][e] = bf16_bits(c);
+        }
+#pragma unroll
+        for (int q = 0; q < 3; ++q) w[q][u >> 1] = p[q][0] | (p[q][1] << 16);
+      }
+      load8(v);
+      if (filled < kF32Stages) ++filled;
+      else if (ok) ok = mbar_wait(empty0 + 8u * s, ph, flag);
+      uint8_t* st = sA + s * kF32Stage + (c8 >> 3) * 2048 + r * 16;
+#pragma unroll
+      for (int q = 0; q < 3; ++q)
+        *reinterpret_cast<uint4*>(st + q * kF32Split) = make_uint4(w[q][0], w[q][1], w[q][2], w[q][3]);
+      fence_async_smem();
+      mbar_arrive(full0 + 8u * s);
+      if (++s == kF32Stages) { s = 0; ph ^= 1u; }
+      if (++ks < nk) return;
+      // epilogue
+      if (ok) ok = mbar_wait(done_b, dpar, flag);
+      dpar ^= 1u;
+      __syncwarp();
+      fence_after();
+      const int q4 = warp & 3;
+      const int64_t ir = tile * kM + q4 * 32 + lane;
+      float mv = 0.f;
+      if (mvsrc && warp < 4 && ir < n) mv = mvsrc[ir];
+      for (int cg = warp >> 2; cg < N / 8; cg += 2) {
+        float acc[8];
+        tmem_ld8(tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(cg * 8), acc);
+        if (ir < n) {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const int o = cg * 8 + j;
+            if (o < nout) out[ir + (int64_t)o * ldu] = acc[j];
           }
         }
-        mma_commit(smem_u32(mbar + s));
-        if (kc == nk - 1) mma_commit(smem_u32(mbar + 2));
       }
-#pragma unroll
-      for (int u = 0; u < 16; ++u) {
-        v[u] = vn[u];
-        vn[u] = vnn[u];
-      }
+      if (mvsrc && warp < 4 && ir < n) mvdst[ir] = mv;
+      fence_before();
+      mbar_arrive(tfree_b);
+      ks = 0;
+      tile += gridDim.x;
+    };
+    float v0[8], v1[8], v2[8];
+    load8(v0);
+    load8(v1);
+    load8(v2);
+    while (true) {
+      if (tile >= ntiles) break;
+      step(v0);
+      if (tile >= ntiles) break;
+      step(v1);
+      if (tile >= ntiles) break;
+      step(v2);
     }
-    if (!ok) break;
-    // epilogue
-    ok = mbar_wait(smem_u32(mbar + 2), dpar, flag);
-    dpar ^= 1u;
-    ok = __syncthreads_and(ok);
-    if (!ok) break;
-    fence_after();
-    const int q4 = warp & 3;
-    const int64_t ir = tile * kM + q4 * 32 + lane;
-    float mv = 0.f;
-    if (mvsrc && warp < 4 && ir < n) mv = mvsrc[ir];
-    for (int cg = warp >> 2; cg < N / 16; cg += 2) {
-      float acc[16];
-      tmem_ld16(tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(cg * 16), acc);
-      if (ir < n) {
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const int o = cg * 16 + j;
-          if (o < nout) out[ir + (int64_t)o * ldu] = acc[j];
-        }
-      }
-    }
-    if (mvsrc && warp < 4 && ir < n) mvdst[ir] = mv;
-    fence_before();
-    __syncthreads();   // accumulator read before the next tile's first MMA
-  }
-  // Every issued MMA has completed unless a wait gave up; then thread 0 waits
-  // (bounded again) for the last commit of each barrier before the tensor
-  // memory is released.
-  if (!ok && tid == 0) {
-    const int c0 = (g + 1) / 2, c1 = g / 2;      // commits made to the two stage barriers
-    if (c0 > 0) (void)mbar_wait(smem_u32(mbar + 0), (uint32_t)((c0 - 1) & 1), flag);
-    if (c1 > 0) (void)mbar_wait(smem_u32(mbar + 1), (uint32_t)((c1 - 1) & 1), flag);
   }
   fence_before();
   __syncthreads();
@@ -338,13 +366,6 @@ constexpr int kDfGroups = 8;
 constexpr int kDfStepSplit = kM * 16 * 2;                 // one digit slice of one K-step
 constexpr int kDfStage = kDfDigits * kDfStepSplit;        // 28 KB
 
-// Shared-memory matrix descriptor of a K-major, no-swizzle operand whose
-// rows lie 16 bytes apart: SBO (next 8 rows) 128 bytes, LBO (next 8 columns) lbo.
-__device__ __forceinline__ uint64_t sdesc_rows(uint32_t addr, uint32_t lbo) {
-  return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo >> 4) << 16) | ((uint64_t)(128 >> 4) << 32) |
-         (1ull << 46);
-}
-
 // What the split needs of a type.  Row exponents are kept biased and clamped
 // to [4, 257], so that the row factor 2^(131 - emax) is a float; rows below or
 // above lie outside what an FP32 pair resolves.
@@ -388,10 +409,6 @@ struct Split<double> {
     y = d >= 47 << 20 ? yi * __int_as_float(((xb & 0x7F800000) - (46 << 23)) | sg) : 0.f;
   }
 };
-
-__device__ __forceinline__ void mbar_arrive(uint32_t mbar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(mbar) : "memory");
-}
 
 constexpr int kDfAllThreads = kDfThreads + 32;
 
@@ -724,7 +741,7 @@ bool tc_restart_supported(int nin, int nout) { return nin >= 1 && nin <= 256 && 
 
 size_t tc_restart_smem(int nin, int nout) {
   const int Kp = (nin + kKc - 1) / kKc * kKc, N = (nout + 15) / 16 * 16;
-  return (size_t)((3 * Kp * N * 2 + 1023) & ~1023) + 2 * kStage + 64;
+  return (size_t)((3 * Kp * N * 2 + 1023) & ~1023) + kF32Stages * kF32Stage + 128;
 }
 
 // Host image of the three bf16 splits of Q (nin x nout, column-major FP64).
@@ -849,16 +866,14 @@ void launch_tc_restart_f32(int64_t n, const float* in, float* out, int64_t ldu, 
   const int Kp = (nin + kKc - 1) / kKc * kKc, N = (nout + 15) / 16 * 16;
   const int64_t ntiles = (n + kM - 1) / kM;
   const size_t sm = tc_restart_smem(nin, nout);
-  int per_sm = 1, sms = 152, dev = 0;
+  int sms = 152, dev = 0;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tc_restart_f32, kThreads, sm) != cudaSuccess ||
-      per_sm < 1)
-    per_sm = 1;
-  per_sm = std::min(per_sm, 512 / kTmemCols);   // tensor memory columns per SM
+  // CTAs an SM holds: three by registers, the rest by shared memory (the
+  // occupancy query counts one for a kernel that allocates tensor memory)
+  const int per_sm = (int)std::min<size_t>(3, std::max<size_t>(1, (size_t)228 * 1024 / (sm + 1024)));
   const int g = (int)std::min<int64_t>(ntiles, (int64_t)sms * per_sm);
-  k_tc_restart_f32<<<g, kThreads, sm, st>>>(n, in, out, ldu, nin, Kp, N, nout,
-                                                                      static_cast<const uint4*>(bimg), mvsrc, mvdst,
-                                                                      flag);
+  k_tc_restart_f32<<<g, kF32All, sm, st>>>(n, in, out, ldu, nin, Kp, N, nout, static_cast<const uint4*>(bimg), mvsrc,
+                                           mvdst, flag);
 }
 
 }  // namespace rks
