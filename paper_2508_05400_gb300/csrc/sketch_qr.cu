@@ -40,14 +40,139 @@
 
 namespace {
 
-// Q[i, j] = (x.hi + x.lo)[i, j] * scale[j] in FP64
-__global__ void k_df2d_scaled(int64_t n, const float2* __restrict__ x, int64_t ldx, const double* __restrict__ scale,
-                              double* __restrict__ y, int64_t ldy) {
+// Q[i, j] = (x.hi + x.lo)[i, j] * scale[j] in FP64, four rows a thread with
+// their loads in flight together
+__global__ void __launch_bounds__(256) k_df2d_scaled(int64_t n, const float2* __restrict__ x, int64_t ldx,
+                                                     const double* __restrict__ scale, double* __restrict__ y,
+                                                     int64_t ldy) {
   const int j = blockIdx.y;
   const double sc = scale[j];
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const float2 v = x[i + (int64_t)j * ldx];
-    y[i + (int64_t)j * ldy] = rks::df_to_double(v) * sc;
+  x += (int64_t)j * ldx;
+  y += (int64_t)j * ldy;
+  for (int64_t i0 = blockIdx.x * (int64_t)1024 + threadIdx.x; i0 < n; i0 += (int64_t)gridDim.x * 1024) {
+    float2 v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (i0 + 256 * q < n) v[q] = x[i0 + 256 * q];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (i0 + 256 * q < n) y[i0 + 256 * q] = rks::df_to_double(v[q]) * sc;
+  }
+}
+
+constexpr int kRgsThreads = 256;
+
+// Device state of the randomized Gram-Schmidt (column-major arrays).
+struct RgsState {
+  int s, d;
+  double zscale;
+  const double* Z;     // d x s: sums of Omega k_j, unscaled
+  double* sum;         // d: sums of the sketch of the column just updated, unscaled
+  double* P;           // d x kPanelCols: the panel's sketches after the earlier panels' projection
+  double* S;           // d x s: the sketches of the orthonormal columns
+  double* R;           // s x s
+  double* cs;          // s: 1 / beta_j, the scale of a stored column
+  float2* nrs;         // coefficients of the next update
+  int* flag;           // 1: a column vanished or is not finite
+};
+
+// a[c] = S[:, c0 + c]^T z for c < nc, then z -= S[:, c0 ..] a, a warp per
+// column and a thread per row; z and a in shared memory.
+__device__ void rgs_project(const RgsState& g, int c0, int nc, double* z, double* a) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int c = warp; c < nc; c += kRgsThreads / 32) {
+    const double* sc = g.S + (size_t)(c0 + c) * g.d;
+    double v = 0.0;
+    for (int i = lane; i < g.d; i += 32) v += sc[i] * z[i];
+    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) a[c] = v;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < g.d; i += kRgsThreads) {
+    double v = z[i];
+#pragma unroll 4
+    for (int c = 0; c < nc; ++c) v -= g.S[i + (size_t)(c0 + c) * g.d] * a[c];
+    z[i] = v;
+  }
+  __syncthreads();
+}
+
+// Column k of a panel against the p0 earlier columns, twice: its coefficients
+// for the panel update (zero for k >= nb), its part of R and its sketch after
+// it.  One CTA per column; bound by FP64 at two lanes a clock: 31 us on average
+// over the ten panels of 80 columns, d = 320.
+__global__ void __launch_bounds__(kRgsThreads) k_rgs_panel(RgsState g, int p0, int nb) {
+  extern __shared__ double rgs_sm[];
+  double* z = rgs_sm;
+  double* a = rgs_sm + g.d;
+  constexpr int B = rks::kPanelCols;
+  const int k = blockIdx.x;
+  if (k >= nb) {
+    for (int c = threadIdx.x; c < p0; c += kRgsThreads) g.nrs[(size_t)c * B + k] = make_float2(0.f, 0.f);
+    return;
+  }
+  for (int i = threadIdx.x; i < g.d; i += kRgsThreads) z[i] = g.Z[i + (size_t)(p0 + k) * g.d] * g.zscale;
+  __syncthreads();
+  for (int pass = 0; pass < 2 && p0 > 0; ++pass) {
+    rgs_project(g, 0, p0, z, a);
+    for (int c = threadIdx.x; c < p0; c += kRgsThreads) {
+      double* r = g.R + c + (size_t)(p0 + k) * g.s;
+      const double v = pass ? *r + a[c] : a[c];
+      *r = v;
+      if (pass) g.nrs[(size_t)c * B + k] = rks::df_from_double(-v * g.cs[c]);
+    }
+    __syncthreads();
+  }
+  for (int i = threadIdx.x; i < g.d; i += kRgsThreads) g.P[i + (size_t)k * g.d] = z[i];
+}
+
+// Column p0 + done of a panel has been updated: beta, its sketch, its scale.
+// Then (next >= 0) column p0 + next against the panel's columns before it,
+// twice: the coefficients of its update.  One CTA, 11 us at d = 320, in place
+// of a copy to the host, its loops and a copy back; with the panels' share the
+// 80-column RGS at n = 1e6 went from 8.8 to 8.0 ms.
+__global__ void __launch_bounds__(kRgsThreads) k_rgs_col(RgsState g, int p0, int done, int next) {
+  extern __shared__ double rgs_sm[];
+  double* z = rgs_sm;
+  double* a = rgs_sm + g.d;
+  __shared__ double red[kRgsThreads / 32 + 1];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int j = p0 + done;
+  double bb = 0.0;
+  for (int i = threadIdx.x; i < g.d; i += kRgsThreads) {
+    const double v = g.sum[i] * g.zscale;
+    bb += v * v;
+  }
+  for (int o = 16; o; o >>= 1) bb += __shfl_xor_sync(0xffffffffu, bb, o);
+  if (lane == 0) red[warp] = bb;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (int q = 0; q < kRgsThreads / 32; ++q) t += red[q];
+    const double beta = sqrt(t);
+    if (!(beta > 0.0) || !isfinite(beta)) *g.flag = 1;
+    red[kRgsThreads / 32] = beta;
+    g.R[j + (size_t)j * g.s] = beta;
+    g.cs[j] = 1.0 / beta;
+  }
+  __syncthreads();
+  const double beta = red[kRgsThreads / 32];
+  for (int i = threadIdx.x; i < g.d; i += kRgsThreads) {
+    g.S[i + (size_t)j * g.d] = g.sum[i] * g.zscale / beta;
+    if (next >= 0) z[i] = g.P[i + (size_t)next * g.d];
+  }
+  if (next < 0) return;
+  __syncthreads();
+  for (int pass = 0; pass < 2; ++pass) {
+    rgs_project(g, p0, next, z, a);
+    if ((int)threadIdx.x < next) {
+      const int c = threadIdx.x;
+      double* r = g.R + p0 + c + (size_t)(p0 + next) * g.s;
+      const double v = pass ? *r + a[c] : a[c];
+      *r = v;
+      if (pass) g.nrs[c] = rks::df_from_double(-v * g.cs[p0 + c]);
+    }
+    __syncthreads();
   }
 }
 
@@ -72,11 +197,12 @@ struct QrWork {
   float2* nrs = nullptr;      // update coefficients (s x 8 of a panel, or 2 s)
   float2* sj = nullptr;       // scale of the updated column
   double* scale = nullptr;    // s column scales for the output
+  double* dense = nullptr;    // small matrices of the randomized Gram-Schmidt
   int* flag = nullptr;
   std::vector<double> host;   // sums read back
   ~QrWork() {
     cudaFree(U); cudaFree(otab); cudaFree(part); cudaFree(sums); cudaFree(Q2); cudaFree(nrs); cudaFree(sj);
-    cudaFree(scale); cudaFree(flag);
+    cudaFree(scale); cudaFree(dense); cudaFree(flag);
     if (have_tiles) rks::free_sketch_tiles(&tiles);
   }
 };
@@ -123,15 +249,6 @@ int setup(QrWork& w, int64_t n, int s, int d, int zeta, uint64_t seed, cudaStrea
 }
 
 float2* col(QrWork& w, int j) { return w.U + (size_t)j * w.ldu; }
-
-// host <- the folded sums of the last kernel's per-CTA partials (rows < cnt)
-int fold_to_host(QrWork& w, int cnt) {
-  rks::launch_df_fold(w.part, cnt, w.tiles.G, w.sums, w.st);
-  QK(cudaGetLastError());
-  QK(cudaMemcpyAsync(w.host.data(), w.sums, (size_t)cnt * sizeof(double), cudaMemcpyDeviceToHost, w.st));
-  QK(cudaStreamSynchronize(w.st));
-  return RKS_OK;
-}
 
 // U[:, c0 + o] = sum_l U[:, a0 + l] F[l, o] for o < s (F s x s, host FP64),
 // out of place, in blocks of at most 64 outputs
@@ -213,96 +330,54 @@ int whiten(QrWork& w, const double* K, int64_t ldk, std::vector<double>& R1, std
 // columns updates the whole panel (they were read once per column, 26 GB at
 // n = 1e6, s = 80); inside the panel a column at a time, its sketch measured
 // after its update.  Every projection is made twice (r = S^T z,
-// r += S^T (z - S r): S is sketch-orthonormal); eight columns side by side
-// give the host loops independent sums.
+// r += S^T (z - S r): S is sketch-orthonormal).  The small steps are kernels
+// (k_rgs_panel, k_rgs_col), so that the host waits once, at the end.
 int rgs(QrWork& w, const double* K, int64_t ldk, std::vector<double>& R, std::vector<double>& S) {
   constexpr int B = rks::kPanelCols;
   const int s = w.s, d = w.d;
-  R.assign((size_t)s * s, 0.0);
-  S.assign((size_t)d * s, 0.0);
-  std::vector<double> Z, z(d), r(B), cs(s, 0.0), P((size_t)d * B), C((size_t)s * B);
-  std::vector<float2> nrs((size_t)s * B);
+  const size_t need = (size_t)d * (1 + B + s) + (size_t)s * s;
+  QK(cudaMalloc(&w.dense, need * sizeof(double)));
+  RgsState g;
+  g.s = s; g.d = d; g.zscale = w.zscale;
+  g.Z = w.sums; g.cs = w.scale; g.nrs = w.nrs; g.flag = w.flag;
+  g.sum = w.dense; g.P = g.sum + d; g.S = g.P + (size_t)d * B; g.R = g.S + (size_t)d * s;
+  const size_t sm = (size_t)(d + s) * sizeof(double);
+  if (sm > 48 * 1024 &&
+      cudaFuncSetAttribute(k_rgs_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess)
+    return RKS_ECUDA;
+  if (sm > 48 * 1024 &&
+      cudaFuncSetAttribute(k_rgs_col, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess)
+    return RKS_ECUDA;
   const float2 one = make_float2(1.f, 0.f);
   QK(cudaMemcpyAsync(w.sj, &one, sizeof(float2), cudaMemcpyHostToDevice, w.st));
+  QK(cudaMemsetAsync(g.R, 0, (size_t)s * s * sizeof(double), w.st));
   // z_j = Omega k_j does not depend on the process: all of them at once
-  int rc = sketch_input(w, K, ldk, Z);
-  if (rc) return rc;
+  for (int j = 0; j < s; j += w.chunk) {
+    const int m = std::min(w.chunk, s - j);
+    rks::launch_sketch_cols_f64(K + (size_t)j * ldk, ldk, m, col(w, j), w.ldu, w.tiles, w.part, w.st);
+    rks::launch_df_fold(w.part, d, w.tiles.G, w.sums + (size_t)j * d, w.st, m);
+  }
   for (int p0 = 0; p0 < s; p0 += B) {
     const int nb = std::min(B, s - p0);
-    std::fill(P.begin(), P.end(), 0.0);
-    for (int k = 0; k < nb; ++k)
-      for (int i = 0; i < d; ++i) P[(size_t)i * B + k] = Z[i + (size_t)(p0 + k) * d];
-    if (p0 > 0) {
-      std::fill(C.begin(), C.end(), 0.0);
-      for (int pass = 0; pass < 2; ++pass) {
-        std::vector<double> D((size_t)p0 * B, 0.0);
-        for (int c = 0; c < p0; ++c) {
-          const double* sc = &S[(size_t)c * d];
-          double a[B] = {};
-          for (int i = 0; i < d; ++i)
-            for (int k = 0; k < B; ++k) a[k] += sc[i] * P[(size_t)i * B + k];
-          for (int k = 0; k < B; ++k) D[(size_t)c * B + k] = a[k];
-        }
-        for (int c = 0; c < p0; ++c) {
-          const double* sc = &S[(size_t)c * d];
-          const double* dc = &D[(size_t)c * B];
-          for (int i = 0; i < d; ++i)
-            for (int k = 0; k < B; ++k) P[(size_t)i * B + k] -= sc[i] * dc[k];
-          for (int k = 0; k < B; ++k) C[(size_t)c * B + k] += dc[k];
-        }
-      }
-      for (int c = 0; c < p0; ++c)
-        for (int k = 0; k < B; ++k) {
-          if (k < nb) R[c + (size_t)(p0 + k) * s] = C[(size_t)c * B + k];
-          nrs[(size_t)c * B + k] = to_df(-C[(size_t)c * B + k] * cs[c]);
-        }
-      QK(cudaMemcpyAsync(w.nrs, nrs.data(), (size_t)p0 * B * sizeof(float2), cudaMemcpyHostToDevice, w.st));
-      rks::launch_df_panel(w.n, w.U, w.ldu, p0, p0, nb, w.nrs, w.st);
-    }
+    k_rgs_panel<<<B, kRgsThreads, sm, w.st>>>(g, p0, nb);
+    if (p0 > 0) rks::launch_df_panel(w.n, w.U, w.ldu, p0, p0, nb, w.nrs, w.st);
     for (int jj = 0; jj < nb; ++jj) {
-      const int j = p0 + jj;
-      // against the panel's columns, twice
-      for (int i = 0; i < d; ++i) z[i] = P[(size_t)i * B + jj];
-      std::fill(r.begin(), r.end(), 0.0);
-      for (int pass = 0; pass < 2; ++pass) {
-        double a[B] = {};
-        for (int c = 0; c < jj; ++c) {
-          const double* sc = &S[(size_t)(p0 + c) * d];
-          double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-          int i = 0;
-          for (; i + 4 <= d; i += 4) {
-            a0 += sc[i] * z[i];
-            a1 += sc[i + 1] * z[i + 1];
-            a2 += sc[i + 2] * z[i + 2];
-            a3 += sc[i + 3] * z[i + 3];
-          }
-          for (; i < d; ++i) a0 += sc[i] * z[i];
-          a[c] = (a0 + a1) + (a2 + a3);
-        }
-        for (int c = 0; c < jj; ++c) {
-          const double* sc = &S[(size_t)(p0 + c) * d];
-          for (int i = 0; i < d; ++i) z[i] -= sc[i] * a[c];
-          r[c] += a[c];
-        }
-      }
       // q~ = k_j - sum_c (q~_c / beta_c) r_c, fused with its partial sketches
-      for (int c = 0; c < jj; ++c) nrs[c] = to_df(-r[c] * cs[p0 + c]);
-      if (jj > 0) QK(cudaMemcpyAsync(w.nrs, nrs.data(), (size_t)jj * sizeof(float2), cudaMemcpyHostToDevice, w.st));
+      if (jj > 0) k_rgs_col<<<1, kRgsThreads, sm, w.st>>>(g, p0, jj - 1, jj);
       rks::launch_df_update_sketch(col(w, p0), w.ldu, jj, w.nrs, w.sj, w.tiles, w.part, false, w.st);
-      rc = fold_to_host(w, d);
-      if (rc) return rc;
-      double bb = 0.0;
-      for (int i = 0; i < d; ++i) { const double v = w.host[i] * w.zscale; bb += v * v; }
-      const double beta = std::sqrt(bb);
-      if (!(beta > 0.0) || !std::isfinite(beta)) return RKS_EBREAKDOWN;
-      for (int i = 0; i < d; ++i) S[i + (size_t)j * d] = w.host[i] * w.zscale / beta;
-      for (int c = 0; c < jj; ++c) R[p0 + c + (size_t)j * s] = r[c];
-      R[j + (size_t)j * s] = beta;
-      cs[j] = 1.0 / beta;
+      rks::launch_df_fold(w.part, d, w.tiles.G, g.sum, w.st);
     }
+    k_rgs_col<<<1, kRgsThreads, sm, w.st>>>(g, p0, nb - 1, -1);
   }
-  QK(cudaMemcpyAsync(w.scale, cs.data(), (size_t)s * sizeof(double), cudaMemcpyHostToDevice, w.st));
-  return RKS_OK;
+  QK(cudaGetLastError());
+  int bad = 0;
+  R.resize((size_t)s * s);
+  S.resize((size_t)d * s);
+  QK(cudaMemcpyAsync(&bad, w.flag, sizeof(int), cudaMemcpyDeviceToHost, w.st));
+  QK(cudaMemcpyAsync(R.data(), g.R, R.size() * sizeof(double), cudaMemcpyDeviceToHost, w.st));
+  QK(cudaMemcpyAsync(S.data(), g.S, S.size() * sizeof(double), cudaMemcpyDeviceToHost, w.st));
+  QK(cudaStreamSynchronize(w.st));
+  return bad ? RKS_EBREAKDOWN : RKS_OK;
 }
 
 // Randomized Householder QR: Householder QR of Theta K ((s + d) x s, Theta =
@@ -501,7 +576,7 @@ extern "C" int rks_sketch_qr(int64_t n, int s, const double* K, int64_t ldk, int
       if (rc) return rc;
     }
   }
-  dim3 grid((unsigned)std::min<int64_t>((n + 255) / 256, 1024), (unsigned)s);
+  dim3 grid((unsigned)std::min<int64_t>((n + 1023) / 1024, 1024), (unsigned)s);
   k_df2d_scaled<<<grid, 256, 0, st>>>(n, col(w, out0), w.ldu, w.scale, Q, ldq);
   QK(cudaGetLastError());
   QK(cudaStreamSynchronize(st));
