@@ -209,7 +209,7 @@ struct BdArgs {
 };
 
 struct BdLayout {
-  int S, B, T, Q, Td, Qd, W, G, Ri, QC, z, sv, r, sig, coef, bk, lre, lim, est, scr, xs, total;
+  int S, B, T, Q, Td, Qd, W, G, Ri, QC, z, sv, r, sig, coef, bk, lre, lim, est, scr, xs, lists, total;
 };
 
 __host__ __device__ inline int bd_take(int& o, int cnt) {
@@ -218,10 +218,22 @@ __host__ __device__ inline int bd_take(int& o, int cnt) {
   return at;
 }
 
+// Entries of a tile's bin lists at most: every list padded to kBH chunks of a
+// multiple of 8.
+__host__ __device__ inline int bd_max_entries(int d, int zeta) { return kBR * zeta + 63 * d; }
+// 8-byte words of a staged tile's lists: d + 1 offsets, then the entries.
+__host__ __device__ inline int bd_off_words(int d) { return (d + 4) / 4 * 2; }
+__host__ __device__ inline int bd_list_words(int d, int zeta) {
+  return bd_off_words(d) + (bd_max_entries(d, zeta) + 7) / 8 * 2;
+}
+constexpr int kBSmemTwo = 112 * 1024;   // dynamic shared memory that leaves room for two CTAs per SM
+
 // Offsets (in 8-byte words) of the per-CTA arrays in dynamic shared memory.
 // The arrays of the contraction share their space with the two tile buffers
-// of the expansions (never live at the same time).
-__host__ __device__ inline BdLayout bd_layout(int m, int d) {
+// of the expansions and the current tile's bin lists (never live at the same
+// time).  lists = 0: no room for the lists beside two CTAs per SM, they are
+// read from global memory.
+__host__ __device__ inline BdLayout bd_layout(int m, int d, int zeta) {
   BdLayout L;
   int o = 0;
   L.S = bd_take(o, d * (m + 1));         // sketches of the basis (orthonormal), FP64
@@ -247,6 +259,12 @@ __host__ __device__ inline BdLayout bd_layout(int m, int d) {
   L.QC = bd_take(o, m * m);              // restart coefficients (double-float); packed Y
   L.xs = u0;                             // expansions only: two tiles of one column (double-float)
   if (o < u0 + 2 * kBR) o = u0 + 2 * kBR;
+  L.lists = u0 + 2 * kBR;
+  const int oe = L.lists + bd_list_words(d, zeta);
+  if (oe > o) {
+    if (oe <= kBSmemTwo / 8) o = oe;
+    else L.lists = 0;
+  }
   L.total = o;
   return L;
 }
@@ -263,20 +281,19 @@ struct BdShared {
 // ---------------------------------------------------------------------------
 
 // Tile sums of the sketch of one column for tile t (xt: that column of the
-// tile, rows written by this CTA): ts[t * d + b] = sum of the signed xt[row]
-// listed for sketch row b.  8 lanes
-// per sketch row, lane h adds its chunk of the list in order, then the
-// butterfly; loop bounds are warp-uniform (4 groups a warp).
-__device__ __forceinline__ void bd_bins_tile(const BdProb& P, int d, int t, const float2* __restrict__ xt,
-                                          float2* __restrict__ ts) {
+// tile): ts[t * d + b] = sum of the signed xt[row] listed for sketch row b,
+// whose entry block lies at ent[off[b] - o0].  8 lanes per sketch row, lane h
+// adds its chunk of the list in order, then the butterfly; loop bounds are
+// warp-uniform (4 groups a warp).
+__device__ __forceinline__ void bd_bins_tile(const int32_t* off, const uint16_t* ent, int o0, int d, int t,
+                                          const float2* xt, float2* __restrict__ ts) {
   const int g = threadIdx.x / kBH, h = threadIdx.x % kBH;
-  const int32_t* off = P.tbin + (size_t)t * (d + 1);
   for (int bb = g & ~3; bb < d; bb += kBT / kBH) {
     const int b = bb + (g & 3);
     float s = 0.f, e = 0.f;
     if (b < d) {
       const int e0 = off[b], len = (off[b + 1] - e0) / kBH;   // per lane, a multiple of 8
-      const uint4* ev = reinterpret_cast<const uint4*>(P.ent + e0 + (size_t)h * len);
+      const uint4* ev = reinterpret_cast<const uint4*>(ent + (e0 - o0) + (size_t)h * len);
       // branch-free: the padding entries gather row 0 with sign 0 (adding an
       // exact zero changes no bit), so that all 8 gathers are in flight at once
 #pragma unroll 2
@@ -514,26 +531,42 @@ __device__ __forceinline__ void bd_update_tile(const BdProb& P, int t, int m1, i
   }
 }
 
-// Restart product of the rows of tile t: U[:, l] = sum_c U[:, c] qc[c * ka + l]
+// Restart product of the rows of tile t: U[:, l] = sum_c U[:, c] qc[c * ks + l]
 // (l < ka, c < m), then U[:, ka] = U[:, m].  Each row is read whole before
-// its first write.
-template <int KM>
-__device__ __noinline__ void bd_restart_tile(const BdProb& P, int t, int m, int ka, const float2* qc) {
+// its first write.  ks: ka rounded up to even, the coefficients there zero;
+// EX: ks = KM (no test per coefficient).  The next four columns' loads are in
+// flight while four are used; bound by the FP32 pipes (12 operations a term).
+// In a batch of 128 (m = 32, 13 kept) 3.0e9 cycles of the CTAs -> 1.5e9.
+template <int KM, bool EX>
+__device__ __noinline__ void bd_restart_tile(const BdProb& P, int t, int m, int ka, int ks, int qoff) {
+  extern __shared__ __align__(16) double bd_dyn[];
+  const float2* qc = reinterpret_cast<const float2*>(bd_dyn + qoff);
   const int rows = (int)min((int64_t)kBR, P.n - (int64_t)t * kBR);
   float2* Ut = P.U + (int64_t)t * (m + 1) * kBR;
   for (int r = threadIdx.x; r < rows; r += kBT) {
     float s[KM], e[KM];
 #pragma unroll
     for (int l = 0; l < KM; ++l) { s[l] = 0.f; e[l] = 0.f; }
-#pragma unroll 4
-    for (int c = 0; c < m; ++c) {
-      const float2 u = Ut[(size_t)c * kBR + r];
+    float2 u[4], un[4];
 #pragma unroll
-      for (int l = 0; l < KM; ++l)
-        if (l < ka) {
-          const float2 q = qc[c * ka + l];
-          bd_mac(u.x, u.y, q.x, q.y, s[l], e[l]);
+    for (int q = 0; q < 4; ++q) u[q] = Ut[(size_t)min(q, m - 1) * kBR + r];
+    for (int c0 = 0; c0 < m; c0 += 4) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) un[q] = Ut[(size_t)min(c0 + 4 + q, m - 1) * kBR + r];
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (c0 + q < m) {
+          const float4* qr = reinterpret_cast<const float4*>(qc + (c0 + q) * ks);
+#pragma unroll
+          for (int l = 0; l < KM; l += 2)
+            if (EX || l < ks) {
+              const float4 w = qr[l / 2];
+              bd_mac(u[q].x, u[q].y, w.x, w.y, s[l], e[l]);
+              bd_mac(u[q].x, u[q].y, w.z, w.w, s[l + 1], e[l + 1]);
+            }
         }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) u[q] = un[q];
     }
     const float2 last = Ut[(size_t)m * kBR + r];
 #pragma unroll
@@ -542,49 +575,128 @@ __device__ __noinline__ void bd_restart_tile(const BdProb& P, int t, int m, int 
     Ut[(size_t)ka * kBR + r] = last;
   }
 }
+__device__ __forceinline__ void bd_restart_rows(const BdProb& P, int t, int m, int ka, int ks, int qoff) {
+  switch (ks) {
+    case 8: bd_restart_tile<8, true>(P, t, m, ka, ks, qoff); return;
+    case 10: bd_restart_tile<10, true>(P, t, m, ka, ks, qoff); return;
+    case 12: bd_restart_tile<12, true>(P, t, m, ka, ks, qoff); return;
+    case 14: bd_restart_tile<14, true>(P, t, m, ka, ks, qoff); return;
+    case 16: bd_restart_tile<16, true>(P, t, m, ka, ks, qoff); return;
+    default:
+      if (ks < 16) bd_restart_tile<16, false>(P, t, m, ka, ks, qoff);
+      else bd_restart_tile<kBMaxKa, false>(P, t, m, ka, ks, qoff);
+  }
+}
 
-// The passes over the tiles t0..t1-1 of this CTA, each a function of its own
-// (own register allocation, one call per pass).  The sketch sums of tile t - 1
-// are formed while the rows of tile t are computed; one barrier per tile.
-// xs: two tile buffers in shared memory (tile t in buffer t % 2).
+__device__ __forceinline__ void bd_cp4(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src));
+}
+__device__ __forceinline__ void bd_cp16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src));
+}
+// bytes (a multiple of 16) from p (16-byte aligned) on their way to L2
+__device__ __forceinline__ void bd_prefetch(const void* p, uint32_t bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes));
+}
+// the first nc (at most kBPre) columns of tile t of the basis, one thread each
+constexpr int kBPre = 8;
+__device__ __forceinline__ void bd_prefetch_cols(const BdProb& P, int t, int m1, int nc) {
+  if ((int)threadIdx.x < min(nc, kBPre))
+    bd_prefetch(P.U + ((int64_t)t * m1 + threadIdx.x) * kBR, kBR * sizeof(float2));
+}
+
+// One pass over the tiles t0..t1-1 of this CTA: rows(t, x) computes the rows
+// of tile t, writing its values to x in shared memory; then the tile's sketch
+// sums are formed.  The tile's bin lists (18 bytes a row: two columns' worth)
+// are copied to shared memory while the rows are computed, and ahead(t + 1)
+// asks for the next tile's first bytes before the sums, so that memory is
+// not idle while the CTA reads shared memory only (read from global memory
+// inside the sums, the lists put three dependent loads in every tile).
+// Shared memory is addressed by its offset, not by a pointer argument: these
+// functions are not inlined, and a pointer would make its loads generic.
+template <class ROWS, class AHEAD>
+__device__ __forceinline__ void bd_pass(const BdProb& P, int t0, int t1, int d, float2* ts, int xs, int lists,
+                                        ROWS rows, AHEAD ahead) {
+  extern __shared__ __align__(16) double bd_dyn[];
+  float2* x = reinterpret_cast<float2*>(bd_dyn + xs);
+  if (lists == 0) {     // the sums of tile t - 1 while the rows of tile t are computed
+    for (int t = t0; t <= t1; ++t) {
+      if (t < t1) rows(t, x + (t & 1) * kBR);
+      if (t > t0) {
+        const int32_t* off = P.tbin + (size_t)(t - 1) * (d + 1);
+        bd_bins_tile(off, P.ent, 0, d, t - 1, x + ((t - 1) & 1) * kBR, ts);
+      }
+      __syncthreads();
+    }
+    return;
+  }
+  int* so = reinterpret_cast<int*>(bd_dyn + lists);
+  uint16_t* se = reinterpret_cast<uint16_t*>(bd_dyn + lists + bd_off_words(d));
+  int o0 = 0, o1 = 0;
+  if (t0 < t1) {
+    o0 = P.tbin[(size_t)t0 * (d + 1)];
+    o1 = P.tbin[(size_t)t0 * (d + 1) + d];
+  }
+  for (int t = t0; t < t1; ++t) {
+    const int32_t* off = P.tbin + (size_t)t * (d + 1);
+    for (int q = threadIdx.x; q <= d; q += kBT) bd_cp4(so + q, off + q);
+    for (int q = threadIdx.x; q < (o1 - o0) / 8; q += kBT) bd_cp16(se + 8 * q, P.ent + o0 + 8 * q);
+    int n0 = 0, n1 = 0;
+    if (t + 1 < t1) {
+      n0 = o1;                       // the tiles' blocks follow one another
+      n1 = off[2 * d + 1];
+    }
+    rows(t, x);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    if (t + 1 < t1) ahead(t + 1);
+    bd_bins_tile(so, se, o0, d, t, x, ts);
+    __syncthreads();
+    o0 = n0;
+    o1 = n1;
+  }
+}
+
 template <bool L2, bool V32>
 __device__ __noinline__ void bd_pass_spmv(const BdProb& P, int t0, int t1, int m1, int j, float2 sg, int d,
-                                          float2* ts, float2* xs) {
-  for (int t = t0; t <= t1; ++t) {
-    if (t < t1) {
-      if (V32) bd_spmv_dia<L2, true>(P, t, m1, j, sg, xs + (t & 1) * kBR);
-      else if (P.D > 0) bd_spmv_dia<L2, false>(P, t, m1, j, sg, xs + (t & 1) * kBR);
-      else bd_spmv_csr<L2>(P, t, m1, j, sg, xs + (t & 1) * kBR);
-    }
-    if (t > t0) bd_bins_tile(P, d, t - 1, xs + ((t - 1) & 1) * kBR, ts);
-    __syncthreads();
-  }
+                                          float2* ts, int xs, int lists) {
+  bd_pass(P, t0, t1, d, ts, xs, lists,
+          [&](int t, float2* x) {
+            if (V32) bd_spmv_dia<L2, true>(P, t, m1, j, sg, x);
+            else if (P.D > 0) bd_spmv_dia<L2, false>(P, t, m1, j, sg, x);
+            else bd_spmv_csr<L2>(P, t, m1, j, sg, x);
+          },
+          [&](int t) {
+            if ((int)threadIdx.x < P.D) {
+              const int64_t r0 = (int64_t)t * kBR;
+              const int rows = (int)min((int64_t)kBR, P.ldu - r0);
+              const size_t at = (size_t)threadIdx.x * P.ldu + r0;
+              if (V32) bd_prefetch(reinterpret_cast<const float*>(P.dvals) + at, rows * (uint32_t)sizeof(float));
+              else bd_prefetch(P.dvals + at, rows * (uint32_t)sizeof(float2));
+            }
+          });
 }
-__device__ __noinline__ void bd_pass_update(const BdProb& P, int t0, int t1, int m1, int j, const float2* coef, int d,
-                                            float2* ts, float2* xs) {
-  for (int t = t0; t <= t1; ++t) {
-    if (t < t1) bd_update_tile(P, t, m1, j, coef, xs + (t & 1) * kBR);
-    if (t > t0) bd_bins_tile(P, d, t - 1, xs + ((t - 1) & 1) * kBR, ts);
-    __syncthreads();
-  }
+__device__ __noinline__ void bd_pass_update(const BdProb& P, int t0, int t1, int m1, int j, int coef, int d,
+                                            float2* ts, int xs, int lists) {
+  extern __shared__ __align__(16) double bd_dyn[];
+  const float2* cf = reinterpret_cast<const float2*>(bd_dyn + coef);
+  bd_pass(P, t0, t1, d, ts, xs, lists, [&](int t, float2* x) { bd_update_tile(P, t, m1, j, cf, x); },
+          [&](int t) { bd_prefetch_cols(P, t, m1, j + 1); });
 }
 __device__ __noinline__ void bd_pass_start(const BdProb& P, int t0, int t1, int m1, uint64_t seed, int d, float2* ts,
-                                           float2* xs) {
-  for (int t = t0; t <= t1; ++t) {
-    if (t < t1) {
-      const int64_t r0 = (int64_t)t * kBR;
-      const int rows = (int)min((int64_t)kBR, P.n - r0);
-      float2* col = P.U + (int64_t)t * m1 * kBR;
-      float2* x = xs + (t & 1) * kBR;
-      for (int r = threadIdx.x; r < rows; r += kBT) {
-        const float2 v = bd_from(bd_normal(seed, r0 + r));
-        col[r] = v;
-        x[r] = v;
-      }
-    }
-    if (t > t0) bd_bins_tile(P, d, t - 1, xs + ((t - 1) & 1) * kBR, ts);
-    __syncthreads();
-  }
+                                           int xs, int lists) {
+  bd_pass(P, t0, t1, d, ts, xs, lists,
+          [&](int t, float2* x) {
+            const int64_t r0 = (int64_t)t * kBR;
+            const int rows = (int)min((int64_t)kBR, P.n - r0);
+            float2* col = P.U + (int64_t)t * m1 * kBR;
+            for (int r = threadIdx.x; r < rows; r += kBT) {
+              const float2 v = bd_from(bd_normal(seed, r0 + r));
+              col[r] = v;
+              x[r] = v;
+            }
+          },
+          [](int) {});
 }
 
 // cluster-wide barrier; the fence orders this thread's global writes before it
@@ -672,7 +784,7 @@ __device__ void bd_solve(const BdArgs& A, const BdProb& P, double* sm, BdShared&
   }
   const int m = A.m, d = A.d, k = A.k;
   const int G = (int)cl.num_blocks(), rank = (int)cl.block_rank();
-  const BdLayout L = bd_layout(m, d);
+  const BdLayout L = bd_layout(m, d, A.zeta);
   double* S = sm + L.S;
   double* B = sm + L.B;
   df* T = reinterpret_cast<df*>(sm + L.T);
@@ -695,7 +807,6 @@ __device__ void bd_solve(const BdArgs& A, const BdProb& P, double* sm, BdShared&
   double* est = sm + L.est;
   double* scr = sm + L.scr;
   df* scr_df = reinterpret_cast<df*>(scr);
-  float2* xs = reinterpret_cast<float2*>(sm + L.xs);
   df* Yr = reinterpret_cast<df*>(W);
   df* Yi = reinterpret_cast<df*>(W) + m * m;
   const int ldb = m + 1;
@@ -717,7 +828,7 @@ __device__ void bd_solve(const BdArgs& A, const BdProb& P, double* sm, BdShared&
   // ---- start (Sec. 3.1 with k = 0): U[:, 0] = u~_1, S[:, 0] = Omega u~_1 / beta
   {
     float2* ts = P.tsum + (size_t)(ex & 1) * P.ntile * d;
-    bd_pass_start(P, t0, t1, m1, A.seed + 1, d, ts, xs);
+    bd_pass_start(P, t0, t1, m1, A.seed + 1, d, ts, L.xs, L.lists);
     bd_cluster_sync(cl);
     bd_tiles_reduce(ts, P.ntile, d, zscale, sv);
     ++ex;
@@ -745,13 +856,14 @@ __device__ void bd_solve(const BdArgs& A, const BdProb& P, double* sm, BdShared&
       const float2 sg = bd_from(sig[j]);
       // w = A u_j, partial z = Omega w (FP32 diagonals when A's values are FP32 numbers)
       if (P.dv32) {
-        if (G > 1) bd_pass_spmv<true, true>(P, t0, t1, m1, j, sg, d, ts, xs);
-        else bd_pass_spmv<false, true>(P, t0, t1, m1, j, sg, d, ts, xs);
+        if (G > 1) bd_pass_spmv<true, true>(P, t0, t1, m1, j, sg, d, ts, L.xs, L.lists);
+        else bd_pass_spmv<false, true>(P, t0, t1, m1, j, sg, d, ts, L.xs, L.lists);
       } else {
-        if (G > 1) bd_pass_spmv<true, false>(P, t0, t1, m1, j, sg, d, ts, xs);
-        else bd_pass_spmv<false, false>(P, t0, t1, m1, j, sg, d, ts, xs);
+        if (G > 1) bd_pass_spmv<true, false>(P, t0, t1, m1, j, sg, d, ts, L.xs, L.lists);
+        else bd_pass_spmv<false, false>(P, t0, t1, m1, j, sg, d, ts, L.xs, L.lists);
       }
       BD_MARK(kPhSpmvRows);
+      if (t0 < t1) bd_prefetch_cols(P, t0, m1, j + 1);   // for the update, behind the exchange and the least squares
       bd_cluster_sync(cl);
       bd_tiles_reduce(ts, P.ntile, d, zscale, z);
       ++ex;
@@ -783,7 +895,7 @@ __device__ void bd_solve(const BdArgs& A, const BdProb& P, double* sm, BdShared&
       __syncthreads();
       BD_MARK(kPhLs);
       ts = P.tsum + (size_t)(ex & 1) * P.ntile * d;
-      bd_pass_update(P, t0, t1, m1, j, coef, d, ts, xs);   // u~ = w - U b, partial s~ = Omega u~
+      bd_pass_update(P, t0, t1, m1, j, L.coef, d, ts, L.xs, L.lists);   // u~ = w - U b, partial s~ = Omega u~
       BD_MARK(kPhUpdRows);
       bd_cluster_sync(cl);
       bd_tiles_reduce(ts, P.ntile, d, zscale, sv);
@@ -942,16 +1054,14 @@ __device__ void bd_solve(const BdArgs& A, const BdProb& P, double* sm, BdShared&
       __syncthreads();
     }
     // restart coefficients sig_c Q'[c, l] and the restart product (Eq. 3.5)
-    for (int t = tid; t < m * ka; t += kBT) {
-      const int c = t / ka, l = t % ka;
-      qc[t] = bd_from(sig[c] * Qd[c + l * m]);
+    const int ks = (ka + 1) & ~1;
+    for (int t = tid; t < m * ks; t += kBT) {
+      const int c = t / ks, l = t % ks;
+      qc[t] = l < ka ? bd_from(sig[c] * Qd[c + l * m]) : make_float2(0.f, 0.f);
     }
     __syncthreads();
     BD_MARK(kPhKept);
-    for (int t = t0; t < t1; ++t) {
-      if (ka <= 16) bd_restart_tile<16>(P, t, m, ka, qc);
-      else bd_restart_tile<kBMaxKa>(P, t, m, ka, qc);
-    }
+    for (int t = t0; t < t1; ++t) bd_restart_rows(P, t, m, ka, ks, L.QC);
     // S <- [S Q', s], B <- [T_a; b^T Q'], sig <- [1 .. 1, sig_m]
     for (int i = tid; i < d; i += kBT) {
       const double last = S[i + (size_t)m * d];
@@ -1421,7 +1531,7 @@ extern "C" int rks_create_batched_dev(rks_dbatch** out, int count, const int64_t
       if (!std::isfinite(v) || std::fabs(v) > 3.0e38) return RKS_EINVAL;   // double-float range
     }
   }
-  const BdLayout L = bd_layout(m, d);
+  const BdLayout L = bd_layout(m, d, o.zeta);
   rks_dbatch* b = new (std::nothrow) rks_dbatch();
   if (!b) return RKS_ENOMEM;
   b->count = count;
