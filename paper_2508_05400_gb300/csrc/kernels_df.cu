@@ -961,7 +961,10 @@ struct DiaOffs {
 // diagonal e at row i, x at i + off_e), the products in increasing column
 // order (the CSR kernel's order, the same bits); two rows per thread, the
 // tiles and the sketch gather of k_df_spmv_ell.
-template <class TU, class TA, bool SK, int DMAX>
+// ND > 0: exactly ND diagonals, so that an interior tile's loads need neither
+// a test nor a zero (rows past a ragged tile's end are read, not stored).
+// DIATIME
+template <class TU, class TA, bool SK, int DMAX, int ND = 0>
 __global__ void __launch_bounds__(512, 2) k_df_spmv_dia(const DiaOffs offs, int D, const TA* __restrict__ dv,
                                                      int64_t ldd, int64_t n, const TU* __restrict__ x,
                                                      TU* __restrict__ w, const SketchTiles tv,
@@ -989,29 +992,32 @@ __global__ void __launch_bounds__(512, 2) k_df_spmv_dia(const DiaOffs offs, int 
     float sa = 0.f, ta = 0.f, sb = 0.f, tb = 0.f;
     // an interior tile (every x[i + off] of its rows inside 0 .. n-1, the
     // usual case) needs no bounds test: 32-bit offsets from the row pointers
-    // (D <= 8 and FP32 values; the other kernels keep one path within their
-    // registers)
-    const bool interior = DMAX == 8 && sizeof(TA) == 4 && r0 + offs.lo >= 0 && r0 + kTileRows + offs.hi <= n;
+    // (FP32 values or an exact number of diagonals; the other kernels keep one
+    // path within their registers)
+    const bool interior = (ND > 0 || (DMAX == 8 && sizeof(TA) == 4)) && r0 + offs.lo >= 0 &&
+                          r0 + kTileRows + (offs.hi > 0 ? offs.hi : 0) <= n;
     if (interior) {
-      const TA* dva = dv + ia;
+      const TA* pv = dv + ia;
       const TU* xpa = x + ia;
+      constexpr int DE = ND > 0 ? ND : DMAX;
 #pragma unroll
-      for (int e0 = 0; e0 < DMAX; e0 += RU) {
+      for (int e0 = 0; e0 < DE; e0 += RU) {
         float2 va[RU], vb[RU], xa[RU], xb[RU];
 #pragma unroll
         for (int u = 0; u < RU; ++u) {
           const int e = e0 + u;
-          const bool on = e < D;
-          const TA* pv = dva + e * ldd;
+          if (e >= DE) continue;
+          const bool on = ND > 0 || e < D, la_on = ND > 0 || (on && oka), lb_on = ND > 0 || (on && okb);
           const TU* px = xpa + offs.o[e];
-          va[u] = (on && oka) ? ldv(pv) : make_float2(0.f, 0.f);
-          vb[u] = (on && okb) ? ldv(pv + 512) : make_float2(0.f, 0.f);
-          xa[u] = (on && oka) ? ldv(px) : make_float2(0.f, 0.f);
-          xb[u] = (on && okb) ? ldv(px + 512) : make_float2(0.f, 0.f);
+          va[u] = la_on ? ldv(pv) : make_float2(0.f, 0.f);
+          vb[u] = lb_on ? ldv(pv + 512) : make_float2(0.f, 0.f);
+          xa[u] = la_on ? ldv(px) : make_float2(0.f, 0.f);
+          xb[u] = lb_on ? ldv(px + 512) : make_float2(0.f, 0.f);
+          pv += ldd;
         }
 #pragma unroll
         for (int u = 0; u < RU; ++u) {
-          if (e0 + u < D) {
+          if (e0 + u < DE && (ND > 0 || e0 + u < D)) {
             mac_st<TA, TU>(va[u], xa[u], sa, ta);
             mac_st<TA, TU>(vb[u], xb[u], sb, tb);
           }
@@ -2525,6 +2531,11 @@ static cudaError_t configure_df_kernels_once() {
   RKS_SMEM((k_df_spmv_dia<float2, float2, true, 16>)); RKS_SMEM((k_df_spmv_dia<float, float, true, 16>));
   RKS_SMEM((k_df_spmv_dia<float2, float2, false, 8>)); RKS_SMEM((k_df_spmv_dia<float2, float2, false, 16>));
   RKS_SMEM((k_df_spmv_dia<float2, float, true, 8>)); RKS_SMEM((k_df_spmv_dia<float2, float, false, 8>));
+  RKS_SMEM((k_df_spmv_dia<float2, float2, true, 8, 5>)); RKS_SMEM((k_df_spmv_dia<float2, float2, true, 8, 7>));
+  RKS_SMEM((k_df_spmv_dia<float2, float2, false, 8, 5>)); RKS_SMEM((k_df_spmv_dia<float2, float2, false, 8, 7>));
+  RKS_SMEM((k_df_spmv_dia<float2, float, true, 8, 5>)); RKS_SMEM((k_df_spmv_dia<float2, float, true, 8, 7>));
+  RKS_SMEM((k_df_spmv_dia<float2, float, false, 8, 5>)); RKS_SMEM((k_df_spmv_dia<float2, float, false, 8, 7>));
+  RKS_SMEM((k_df_spmv_dia<float, float, true, 8, 5>)); RKS_SMEM((k_df_spmv_dia<float, float, true, 8, 7>));
   RKS_SMEM((k_df_spmv_ell<float2, float2, false, 0>)); RKS_SMEM((k_df_spmv_ell<float2, float2, true, 6>));
   RKS_SMEM((k_df_spmv_ell<float, float, true, 6>)); RKS_SMEM((k_df_spmv_ell<float2, float2, false, 6>));
   constexpr int U8 = kDfUpdUnroll, MB = kDfUpdMinBlocks;
@@ -2589,17 +2600,22 @@ static void launch_dia(const CsrDF& A, const void* x, void* w, const SketchTiles
   const TU* dv = static_cast<const TU*>(A.dvals);
   if (A.D > 8) {
     k_df_spmv_dia<TU, TU, SK, 16><<<t.G, 512, sm, st>>>(o, A.D, dv, A.ldd, A.n, xx, ww, t, part);
-  } else if constexpr (std::is_same<TU, float2>::value) {
+    return;
+  }
+  // exact kernels for the 5- and 7-point stencils
+  if constexpr (std::is_same<TU, float2>::value) {
     // double-float vectors: the FP32 copy of the diagonals when every value
     // of A is an FP32 number (the pairs' low words are zero: the same bits)
-    if (A.dvals_f32)
-      k_df_spmv_dia<float2, float, SK, 8><<<t.G, 512, sm, st>>>(o, A.D, static_cast<const float*>(A.dvals_f32),
-                                                                A.ldd, A.n, xx, ww, t, part);
-    else
-      k_df_spmv_dia<float2, float2, SK, 8><<<t.G, 512, sm, st>>>(o, A.D, dv, A.ldd, A.n, xx, ww, t, part);
-  } else {
-    k_df_spmv_dia<TU, TU, SK, 8><<<t.G, 512, sm, st>>>(o, A.D, dv, A.ldd, A.n, xx, ww, t, part);
+    if (A.dvals_f32) {
+      auto k = A.D == 5 ? k_df_spmv_dia<float2, float, SK, 8, 5>
+                        : A.D == 7 ? k_df_spmv_dia<float2, float, SK, 8, 7> : k_df_spmv_dia<float2, float, SK, 8>;
+      k<<<t.G, 512, sm, st>>>(o, A.D, static_cast<const float*>(A.dvals_f32), A.ldd, A.n, xx, ww, t, part);
+      return;
+    }
   }
+  auto k = A.D == 5 ? k_df_spmv_dia<TU, TU, SK, 8, 5>
+                    : A.D == 7 ? k_df_spmv_dia<TU, TU, SK, 8, 7> : k_df_spmv_dia<TU, TU, SK, 8>;
+  k<<<t.G, 512, sm, st>>>(o, A.D, dv, A.ldd, A.n, xx, ww, t, part);
 }
 
 // The merge-path partition of A (the first row of every CTA's range), once per
