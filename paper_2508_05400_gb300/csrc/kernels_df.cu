@@ -276,14 +276,15 @@ __global__ void __launch_bounds__(256) k_tiles_build(const int64_t* __restrict__
 }
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+template <int OFF>
 __device__ __forceinline__ uint32_t lds32(uint32_t a) {
   uint32_t x;
-  asm volatile("ld.shared.b32 %0, [%1];" : "=r"(x) : "r"(a));
+  asm volatile("ld.shared.b32 %0, [%1+%2];" : "=r"(x) : "r"(a), "n"(OFF));
   return x;
 }
-__device__ __forceinline__ uint32_t lds16(uint32_t a) {
-  uint16_t x;
-  asm volatile("ld.shared.u16 %0, [%1];" : "=h"(x) : "r"(a));
+__device__ __forceinline__ uint32_t lds16(uint32_t a) {   // sign-extended: bit 15 in bit 31
+  uint32_t x;
+  asm volatile("ld.shared.s16 %0, [%1];" : "=r"(x) : "r"(a));
   return x;
 }
 __device__ __forceinline__ void lds_val(uint32_t a, uint32_t row, float2& v) {
@@ -292,8 +293,8 @@ __device__ __forceinline__ void lds_val(uint32_t a, uint32_t row, float2& v) {
 __device__ __forceinline__ void lds_val(uint32_t a, uint32_t row, float& v) {
   asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a + row * 4u));
 }
-__device__ __forceinline__ float flip(float v, uint32_t x) {   // -v where bit 15 of x is set
-  return __uint_as_float(__float_as_uint(v) ^ ((x << 16) & 0x80000000u));
+__device__ __forceinline__ float flip(float v, uint32_t x) {   // -v for a negative entry
+  return __uint_as_float(__float_as_uint(v) ^ (x & 0x80000000u));
 }
 
 // (s, e) += sign * v for a bin-list entry x; FP32 values have no low word, so
@@ -321,13 +322,15 @@ __device__ __forceinline__ void tile_put(float* p, float2 v) { *p = v.x; }
 // small; their sums are combined by a fixed xor tree.  A sketch row has one
 // position per tile, so acc[row] has one writer per tile.
 //
-// Bound by instruction issue (a 7-point FP32 SpMV with zeta = 8 issues in 73%
-// of the cycles): hence H as a constant (the slot offsets at constant
+// Bound by instruction issue (a 7-point FP32 SpMV with zeta = 8 issues in 70%
+// of the cycles, more than half of them here): hence H as a constant (the slot offsets at constant
 // distances), 32-bit shared addresses, a sign by one exclusive or, and the
 // last one to three entries of a list as one masked round (adding an exact
-// zero changes no bit) instead of one by one.  The updates above: 64 -> 59 us
-// and 134 -> 130 us; 23 -> 21 us.  FP32 values are kept as 4 bytes: at random
-// banks a warp's read takes 3 to 4 passes instead of 6.
+// zero changes no bit) instead of one by one.  FP32 values are kept as 4 bytes:
+// at random banks a warp's read takes 3 to 4 passes instead of 6.  With the
+// lists fetched by the CTA's last warps only, at n = 4.1e6, d = 96: the update
+// of 2 to 27 columns 119 -> 93 us on average, the SpMV 73 -> 64 us; pairs,
+// n = 1e6, d = 320, 1 to 80 columns: update 70 -> 62 us.
 template <int H, class TV>
 __device__ __forceinline__ void tile_gather_h(int d, const TV* vals, const int* offs, const uint32_t* ms,
                                               const uint16_t* es, float2* acc) {
@@ -349,8 +352,10 @@ __device__ __forceinline__ void tile_gather_h(int d, const TV* vals, const int* 
       for (; k >= 4; k -= 4, oa += 16u * H) {
         uint32_t x[4];
         TV v[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) x[u] = lds32(oa + 4u * H * u);
+        x[0] = lds32<0>(oa);
+        x[1] = lds32<4 * H>(oa);
+        x[2] = lds32<8 * H>(oa);
+        x[3] = lds32<12 * H>(oa);
 #pragma unroll
         for (int u = 0; u < 4; ++u) x[u] = lds16(ea + 2u * x[u]);
 #pragma unroll
@@ -362,7 +367,7 @@ __device__ __forceinline__ void tile_gather_h(int d, const TV* vals, const int* 
         uint32_t x[3];
         TV v[3];
 #pragma unroll
-        for (int u = 0; u < 3; ++u) x[u] = lds32(u < k ? oa + 4u * H * u : oa);
+        for (int u = 0; u < 3; ++u) x[u] = lds32<0>(u < k ? oa + 4u * H * u : oa);
 #pragma unroll
         for (int u = 0; u < 3; ++u) x[u] = lds16(ea + 2u * x[u]);
 #pragma unroll
@@ -490,8 +495,10 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src));
 }
 
-// Starts the copy of the bin lists of step k's tile into its buffers
-// (tile_wait ends it; the bytes are those of tile_stage).  Issued a tile
+constexpr int kFetchThreads = 128;
+// Starts the copy of the bin lists of step k's tile into its buffers, by the
+// CTA's last warps (for most d they have no sketch row of their own in the
+// gather), and ends with tile_wait; the bytes are those of tile_stage.  Issued a tile
 // ahead: staged at the tile's start instead, the bounds' load, then those of
 // the lists, were waited for one after the other (FP32 update, n = 4.1e6,
 // d = 96, one basis column: 84 -> 64 us; 26 columns: 150 -> 134 us; pairs,
@@ -499,6 +506,8 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
 template <class TV>
 __device__ __forceinline__ void tile_fetch(uint8_t* sm, const TileSmem& lay, const SketchTiles& tv,
                                            const TileRange& tr, int k) {
+  const int f = (int)threadIdx.x - ((int)blockDim.x - kFetchThreads);
+  if (f < 0) return;
   const TileBuf<TV> b(sm, lay, tv, k);
   const int L1 = tv.L + 1, d = tv.d;
   const int64_t t = tr.t0 + tr.at(k), e0 = tr.row(k) * tv.zeta;
@@ -508,19 +517,20 @@ __device__ __forceinline__ void tile_fetch(uint8_t* sm, const TileSmem& lay, con
   const uint16_t* eg = tv.ent + e0;
   int q0;
   if ((e0 & 7) == 0) {
-    for (int q = threadIdx.x; q < cnt >> 3; q += blockDim.x) cp_async16(b.es + 8 * q, eg + 8 * q);
+#pragma unroll 4
+    for (int q = f; q < cnt >> 3; q += kFetchThreads) cp_async16(b.es + 8 * q, eg + 8 * q);
     q0 = cnt & ~7;
   } else {                       // tiles start at even rows: 4-byte aligned
-    for (int q = threadIdx.x; q < cnt >> 1; q += blockDim.x) cp_async4(b.es + 2 * q, eg + 2 * q);
+    for (int q = f; q < cnt >> 1; q += kFetchThreads) cp_async4(b.es + 2 * q, eg + 2 * q);
     q0 = cnt & ~1;
   }
   if ((d & 3) == 0) {
-    for (int q = threadIdx.x; q < d >> 2; q += blockDim.x) cp_async16(b.ms + 4 * q, mg + 4 * q);
+    for (int q = f; q < d >> 2; q += kFetchThreads) cp_async16(b.ms + 4 * q, mg + 4 * q);
   } else {
-    for (int q = threadIdx.x; q < d; q += blockDim.x) cp_async4(b.ms + q, mg + q);
+    for (int q = f; q < d; q += kFetchThreads) cp_async4(b.ms + q, mg + q);
   }
-  for (int q = threadIdx.x; q < L1; q += blockDim.x) cp_async4(b.of + q, og + q);
-  for (int q = q0 + threadIdx.x; q < cnt; q += blockDim.x) b.es[q] = eg[q];
+  for (int q = f; q < L1; q += kFetchThreads) cp_async4(b.of + q, og + q);
+  for (int q = q0 + f; q < cnt; q += kFetchThreads) b.es[q] = eg[q];
 }
 __device__ __forceinline__ void tile_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
