@@ -40,6 +40,30 @@
 
 namespace rks {
 
+// Programmatic launch: a kernel launched by launch_pdl may start before the one
+// in front of it in the stream has ended; pdl_wait returns when that one has
+// ended and its writes are visible (at once in a kernel launched normally).
+// pdl_next lets the next such kernel start; its CTAs come in as this kernel's
+// leave.  Before pdl_wait only constant data is read (the bin lists), and
+// prefetches to L2 are made.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_next() { asm volatile("griddepcontrol.launch_dependents;"); }
+
+template <class... P, class... A>
+static void launch_pdl(void (*k)(P...), int g, int b, size_t sm, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  cfg.gridDim = dim3((unsigned)g);
+  cfg.blockDim = dim3((unsigned)b);
+  cfg.dynamicSmemBytes = sm;
+  cfg.stream = st;
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  (void)cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);   // an error stays in cudaGetLastError, as with <<<>>>
+}
+
 // ---------------------------------------------------------------------------
 // double-float helpers
 // ---------------------------------------------------------------------------
@@ -580,6 +604,8 @@ __global__ void __launch_bounds__(512) k_df_spmv_sketch(
     for (int r = threadIdx.x; r < d; r += blockDim.x) acc[r] = make_float2(0.f, 0.f);
   const TileRange tr(tv, false);
   if (SK && tr.nt > 0) tile_fetch<TU>(smraw, lay, tv, tr, 0);
+  pdl_next();
+  pdl_wait();
   for (int k = 0; k < tr.nt; ++k) {
     TU* v = TileBuf<TU>(smraw, lay, tv, k).v;
     const int64_t r0 = tr.row(k);
@@ -639,6 +665,8 @@ __global__ void __launch_bounds__(512) k_df_spmv_ell(
     for (int r = threadIdx.x; r < d; r += blockDim.x) acc[r] = make_float2(0.f, 0.f);
   const TileRange tr(tv, false);
   if (SK && tr.nt > 0) tile_fetch<TU>(smraw, lay, tv, tr, 0);
+  pdl_next();
+  pdl_wait();
   for (int k = 0; k < tr.nt; ++k) {
     TU* v = TileBuf<TU>(smraw, lay, tv, k).v;
     const int64_t r0 = tr.row(k);
@@ -717,6 +745,8 @@ __global__ void __launch_bounds__(512) k_df_spmv_warp(const int32_t* __restrict_
   const int grp = threadIdx.x / LPR, lane = threadIdx.x % LPR, ngrp = blockDim.x / LPR;
   const TileRange tr(tv, false);
   if (SK && tr.nt > 0) tile_fetch<TU>(smraw, lay, tv, tr, 0);
+  pdl_next();
+  pdl_wait();
   for (int k = 0; k < tr.nt; ++k) {
     TU* v = TileBuf<TU>(smraw, lay, tv, k).v;
     const int64_t r0 = tr.row(k);
@@ -988,6 +1018,8 @@ __global__ void __launch_bounds__(512, 2) k_df_spmv_dia(const DiaOffs offs, int 
     for (int r = threadIdx.x; r < d; r += blockDim.x) acc[r] = make_float2(0.f, 0.f);
   const TileRange tr(tv, false);
   if (SK && tr.nt > 0) tile_fetch<TU>(smraw, lay, tv, tr, 0);
+  pdl_next();
+  pdl_wait();
   for (int k = 0; k < tr.nt; ++k) {
     TU* v = TileBuf<TU>(smraw, lay, tv, k).v;
     const int64_t r0 = tr.row(k);
@@ -1108,6 +1140,12 @@ __device__ __forceinline__ void ld2(const float* p, float2& a, float2& b) {
   b = make_float2(v.y, 0.f);
 }
 
+// Bytes of the basis that a CTA of the update asks for ahead of the least
+// squares in front of it (304 CTAs: 49 MB, 7 us of HBM, within L2 beside w').
+// With the launches' overlap: first restart of the 1000 x 1000 problem 11.6 ->
+// 11.2 ms, of a power-law matrix 3.42 -> 3.29 ms, 160^3 mixed 12.1 -> 11.8 ms.
+constexpr int kPdlPrefetch = 160 * 1024;
+
 // u~ = sj * w' + sum_{col < c} U[:, col] * nrs[col]  (nrs = -b .* scale, DF)
 // written to U[:, c]; part[cta] = the CTA's Omega-sums of u~ as stored.
 // A thread takes two consecutive rows (tile starts are even and ld is a
@@ -1125,17 +1163,26 @@ __global__ void __launch_bounds__(512, MINB) k_df_update_sketch(
   const TileSmem lay = tile_smem_layout(d, tv.L, c, tv.zeta);
   float2* acc = reinterpret_cast<float2*>(smraw + lay.acc);
   float2* rsh = reinterpret_cast<float2*>(smraw + lay.rsh);
-  for (int col = threadIdx.x; col < c; col += blockDim.x) rsh[col] = nrs[col];
   if (SK)
     for (int r = threadIdx.x; r < d; r += blockDim.x) acc[r] = make_float2(0.f, 0.f);
   double ss = 0.0;
-  __syncthreads();
-  const float2 sc = sj[0];
   // The second half of the grid takes its tiles last to first: the two CTAs
   // an SM holds (blocks b and b + G/2) then meet their short last tile at
   // different times, and the SM keeps more loads in flight.
   const TileRange tr(tv, blockIdx.x >= gridDim.x / 2);
   if (SK && tr.nt > 0) tile_fetch<TU>(smraw, lay, tv, tr, 0);
+  // the first columns of the CTA's first tiles on their way to L2 while the
+  // least squares in front of this kernel is still running
+  pdl_next();
+  if (SK && c > 0) {
+    const int k = threadIdx.x / c, col = threadIdx.x - k * c;
+    if (k < tr.nt && (int)threadIdx.x < kPdlPrefetch / (int)(kTileRows * sizeof(TU)))
+      prefetch_rows(U + tr.row(k) + (int64_t)col * ldu, tr.rows(k));
+  }
+  pdl_wait();
+  for (int col = threadIdx.x; col < c; col += blockDim.x) rsh[col] = nrs[col];
+  __syncthreads();
+  const float2 sc = sj[0];
   for (int k = 0; k < tr.nt; ++k) {
     TU* v = TileBuf<TU>(smraw, lay, tv, k).v;
     const int64_t r0 = tr.row(k);
@@ -1528,6 +1575,7 @@ __global__ void __launch_bounds__(256) k_df_ls_coop(
   double* sst = zst + d;
   __shared__ double red[33];
   const int tid = threadIdx.x, nt = blockDim.x, warp = tid >> 5, lane = tid & 31, nw = nt >> 5;
+  pdl_next();                           // the update's CTAs may come in and fetch what does not depend on this
   const int gw = blockIdx.x * nw + warp, tw = gridDim.x * nw;   // global warp index, warps in grid
   const int c = j + 1;
   // stall (a test hook) waits for one CTA more than the grid holds, so every
@@ -1733,6 +1781,8 @@ __global__ void __launch_bounds__(512) k_df_sketch_vec(const TU* __restrict__ x,
   for (int r = threadIdx.x; r < d; r += blockDim.x) acc[r] = make_float2(0.f, 0.f);
   const TileRange tr(tv, false);
   if (tr.nt > 0) tile_fetch<TU>(smraw, lay, tv, tr, 0);
+  pdl_next();
+  pdl_wait();
   for (int k = 0; k < tr.nt; ++k) {
     TU* v = TileBuf<TU>(smraw, lay, tv, k).v;
     const int64_t r0 = tr.row(k);
@@ -2609,7 +2659,7 @@ static void launch_dia(const CsrDF& A, const void* x, void* w, const SketchTiles
   TU* ww = static_cast<TU*>(w);
   const TU* dv = static_cast<const TU*>(A.dvals);
   if (A.D > 8) {
-    k_df_spmv_dia<TU, TU, SK, 16><<<t.G, 512, sm, st>>>(o, A.D, dv, A.ldd, A.n, xx, ww, t, part);
+    launch_pdl(k_df_spmv_dia<TU, TU, SK, 16>, t.G, 512, sm, st, o, A.D, dv, A.ldd, A.n, xx, ww, t, part);
     return;
   }
   // exact kernels for the 5- and 7-point stencils
@@ -2619,13 +2669,13 @@ static void launch_dia(const CsrDF& A, const void* x, void* w, const SketchTiles
     if (A.dvals_f32) {
       auto k = A.D == 5 ? k_df_spmv_dia<float2, float, SK, 8, 5>
                         : A.D == 7 ? k_df_spmv_dia<float2, float, SK, 8, 7> : k_df_spmv_dia<float2, float, SK, 8>;
-      k<<<t.G, 512, sm, st>>>(o, A.D, static_cast<const float*>(A.dvals_f32), A.ldd, A.n, xx, ww, t, part);
+      launch_pdl(k, t.G, 512, sm, st, o, A.D, static_cast<const float*>(A.dvals_f32), A.ldd, A.n, xx, ww, t, part);
       return;
     }
   }
   auto k = A.D == 5 ? k_df_spmv_dia<TU, TU, SK, 8, 5>
                     : A.D == 7 ? k_df_spmv_dia<TU, TU, SK, 8, 7> : k_df_spmv_dia<TU, TU, SK, 8>;
-  k<<<t.G, 512, sm, st>>>(o, A.D, dv, A.ldd, A.n, xx, ww, t, part);
+  launch_pdl(k, t.G, 512, sm, st, o, A.D, dv, A.ldd, A.n, xx, ww, t, part);
 }
 
 // The merge-path partition of A (the first row of every CTA's range), once per
@@ -2665,11 +2715,11 @@ void launch_df_spmv_sketch(const CsrDF& A, const void* x, void* w, const SketchT
     const bool wide = A.nnz >= 64 * A.n;   // mean row length >= 64: a warp per row, else 8 lanes
     if (A.f32) {
       auto k = wide ? k_df_spmv_warp<float, float, true, 32> : k_df_spmv_warp<float, float, true, 8>;
-      k<<<t.G, 512, sm, st>>>(A.rowptr, A.colind, static_cast<const float*>(A.vals), static_cast<const float*>(x),
+      launch_pdl(k, t.G, 512, sm, st, A.rowptr, A.colind, static_cast<const float*>(A.vals), static_cast<const float*>(x),
                               static_cast<float*>(w), t, part);
     } else {
       auto k = wide ? k_df_spmv_warp<float2, float2, true, 32> : k_df_spmv_warp<float2, float2, true, 8>;
-      k<<<t.G, 512, sm, st>>>(A.rowptr, A.colind, static_cast<const float2*>(A.vals), static_cast<const float2*>(x),
+      launch_pdl(k, t.G, 512, sm, st, A.rowptr, A.colind, static_cast<const float2*>(A.vals), static_cast<const float2*>(x),
                               static_cast<float2*>(w), t, part);
     }
     return;
@@ -2683,22 +2733,22 @@ void launch_df_spmv_sketch(const CsrDF& A, const void* x, void* w, const SketchT
     const bool narrow = A.W <= 6;
     if (A.f32) {
       auto k = narrow ? k_df_spmv_ell<float, float, true, 6> : k_df_spmv_ell<float, float, true, 0>;
-      k<<<t.G, 512, sm, st>>>(A.ecol, static_cast<const float*>(A.evals), A.W, static_cast<const float*>(x),
+      launch_pdl(k, t.G, 512, sm, st, A.ecol, static_cast<const float*>(A.evals), A.W, static_cast<const float*>(x),
                               static_cast<float*>(w), t, part);
     } else {
       auto k = narrow ? k_df_spmv_ell<float2, float2, true, 6> : k_df_spmv_ell<float2, float2, true, 0>;
-      k<<<t.G, 512, sm, st>>>(A.ecol, static_cast<const float2*>(A.evals), A.W, static_cast<const float2*>(x),
+      launch_pdl(k, t.G, 512, sm, st, A.ecol, static_cast<const float2*>(A.evals), A.W, static_cast<const float2*>(x),
                               static_cast<float2*>(w), t, part);
     }
     return;
   }
   if (A.f32)
-    k_df_spmv_sketch<float, float, true><<<t.G, 512, sm, st>>>(
-        A.rowptr, A.colind, static_cast<const float*>(A.vals), static_cast<const float*>(x), static_cast<float*>(w),
+    launch_pdl(
+        k_df_spmv_sketch<float, float, true>, t.G, 512, sm, st, A.rowptr, A.colind, static_cast<const float*>(A.vals), static_cast<const float*>(x), static_cast<float*>(w),
         t, part);
   else
-    k_df_spmv_sketch<float2, float2, true><<<t.G, 512, sm, st>>>(
-        A.rowptr, A.colind, static_cast<const float2*>(A.vals), static_cast<const float2*>(x),
+    launch_pdl(
+        k_df_spmv_sketch<float2, float2, true>, t.G, 512, sm, st, A.rowptr, A.colind, static_cast<const float2*>(A.vals), static_cast<const float2*>(x),
         static_cast<float2*>(w), t, part);
 }
 
@@ -2796,10 +2846,11 @@ void launch_df_update_sketch(void* U, int64_t ldu, int c, const float2* nrs, con
   // FP32 basis: twice the columns per batch, so that a thread has as many
   // bytes of loads in flight as with pairs (same order of the sums)
   if (f32)
-    k_df_update_sketch<float, 2 * U8, MB, 1><<<t.G, 512, sm, st>>>(static_cast<float*>(U), ldu, c, nrs, sj, t,
-                                                                   part);
+    launch_pdl(k_df_update_sketch<float, 2 * U8, MB, 1>, t.G, 512, sm, st, static_cast<float*>(U), ldu, c, nrs, sj, t,
+               part);
   else
-    k_df_update_sketch<float2, U8, MB, 1><<<t.G, 512, sm, st>>>(static_cast<float2*>(U), ldu, c, nrs, sj, t, part);
+    launch_pdl(k_df_update_sketch<float2, U8, MB, 1>, t.G, 512, sm, st, static_cast<float2*>(U), ldu, c, nrs, sj, t,
+               part);
 }
 
 int launch_df_small(int j, int d, double zscale, int finish, int ls, double* s_raw, double* z_raw, double* S64,
@@ -2876,8 +2927,8 @@ void launch_df_axpy_cols(int64_t n, float2* U, int64_t ldu, int src, int c0, int
 
 void launch_df_sketch_vec(const void* x, const SketchTiles& t, double* part, bool f32, cudaStream_t st) {
   const size_t sm = tile_smem_bytes(t.d, t.L, 0, t.zeta);
-  if (f32) k_df_sketch_vec<float><<<t.G, 512, sm, st>>>(static_cast<const float*>(x), t, part);
-  else k_df_sketch_vec<float2><<<t.G, 512, sm, st>>>(static_cast<const float2*>(x), t, part);
+  if (f32) launch_pdl(k_df_sketch_vec<float>, t.G, 512, sm, st, static_cast<const float*>(x), t, part);
+  else launch_pdl(k_df_sketch_vec<float2>, t.G, 512, sm, st, static_cast<const float2*>(x), t, part);
 }
 
 // Row ranges: G CTAs (at most kSketchCtas) own contiguous, even-aligned row
