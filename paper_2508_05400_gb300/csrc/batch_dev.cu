@@ -58,6 +58,7 @@
 #include <vector>
 
 #include "../../include/rks.h"
+#include "convert.cuh"
 #include "dense_dev.cuh"
 #include "rks_impl.h"
 
@@ -125,7 +126,7 @@ __host__ __device__ __forceinline__ float2 bd_from(double x) {
   const float h = (float)x;
   return make_float2(h, (float)(x - (double)h));
 }
-__device__ __forceinline__ double bd_to(float2 v) { return (double)v.x + (double)v.y; }
+__device__ __forceinline__ double bd_to(float2 v) { return rks::df_to_double(v); }
 
 // butterfly over the kBH lanes of a group (fixed order)
 __device__ __forceinline__ void bd_group_sum(float& s, float& t) {
@@ -739,12 +740,20 @@ __device__ __noinline__ void bd_resid_tile(const BdProb& P, int64_t r0, int rows
       ar += a * __ldcg(xr + cc);
       if (pair) ai += a * __ldcg(xi + cc);
     }
-    const double x0 = __ldcg(xr + i), x1 = pair ? __ldcg(xi + i) : 0.0;
-    const double re = ar - lr * x0 + li * x1, im = ai - li * x0 - lr * x1;
-    v[0] += re * re + im * im;
-    v[1] += x0 * x0 + x1 * x1;
-    v[2] += x0 * ar + x1 * ai;
-    v[3] += x0 * ai - x1 * ar;
+    const double x0 = __ldcg(xr + i);
+    if (pair) {
+      const double x1 = __ldcg(xi + i);
+      const double re = ar - lr * x0 + li * x1, im = ai - li * x0 - lr * x1;
+      v[0] += re * re + im * im;
+      v[1] += x0 * x0 + x1 * x1;
+      v[2] += x0 * ar + x1 * ai;
+      v[3] += x0 * ai - x1 * ar;
+    } else {                 // a real eigenvalue: half the FP64 operations
+      const double re = ar - lr * x0;
+      v[0] += re * re;
+      v[1] += x0 * x0;
+      v[2] += x0 * ar;
+    }
   }
   bd_block_sum4(v, red);
   if (threadIdx.x < 4) out4[threadIdx.x] = v[threadIdx.x];
