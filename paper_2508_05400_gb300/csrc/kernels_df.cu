@@ -36,33 +36,10 @@
 #include <vector>
 
 #include "convert.cuh"
+#include "pdl.cuh"
 #include "rks_impl.h"
 
 namespace rks {
-
-// Programmatic launch: a kernel launched by launch_pdl may start before the one
-// in front of it in the stream has ended; pdl_wait returns when that one has
-// ended and its writes are visible (at once in a kernel launched normally).
-// pdl_next lets the next such kernel start; its CTAs come in as this kernel's
-// leave.  Before pdl_wait only constant data is read (the bin lists), and
-// prefetches to L2 are made.
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_next() { asm volatile("griddepcontrol.launch_dependents;"); }
-
-template <class... P, class... A>
-static void launch_pdl(void (*k)(P...), int g, int b, size_t sm, cudaStream_t st, A... args) {
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute at[1];
-  cfg.gridDim = dim3((unsigned)g);
-  cfg.blockDim = dim3((unsigned)b);
-  cfg.dynamicSmemBytes = sm;
-  cfg.stream = st;
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  (void)cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);   // an error stays in cudaGetLastError, as with <<<>>>
-}
 
 // ---------------------------------------------------------------------------
 // double-float helpers
@@ -299,6 +276,8 @@ __global__ void __launch_bounds__(256) k_tiles_build(const int64_t* __restrict__
   }
 }
 
+// (s, e) += sign * vals[row] for one bin-list entry: the loads (32-bit shared
+// addresses) and the addition
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 template <int OFF>
 __device__ __forceinline__ uint32_t lds32(uint32_t a) {
@@ -606,6 +585,7 @@ __global__ void __launch_bounds__(512) k_df_spmv_sketch(
   if (SK && tr.nt > 0) tile_fetch<TU>(smraw, lay, tv, tr, 0);
   pdl_next();
   pdl_wait();
+  x = pdl_fresh(x);
   for (int k = 0; k < tr.nt; ++k) {
     TU* v = TileBuf<TU>(smraw, lay, tv, k).v;
     const int64_t r0 = tr.row(k);
@@ -667,6 +647,7 @@ __global__ void __launch_bounds__(512) k_df_spmv_ell(
   if (SK && tr.nt > 0) tile_fetch<TU>(smraw, lay, tv, tr, 0);
   pdl_next();
   pdl_wait();
+  x = pdl_fresh(x);
   for (int k = 0; k < tr.nt; ++k) {
     TU* v = TileBuf<TU>(smraw, lay, tv, k).v;
     const int64_t r0 = tr.row(k);
@@ -747,6 +728,7 @@ __global__ void __launch_bounds__(512) k_df_spmv_warp(const int32_t* __restrict_
   if (SK && tr.nt > 0) tile_fetch<TU>(smraw, lay, tv, tr, 0);
   pdl_next();
   pdl_wait();
+  x = pdl_fresh(x);
   for (int k = 0; k < tr.nt; ++k) {
     TU* v = TileBuf<TU>(smraw, lay, tv, k).v;
     const int64_t r0 = tr.row(k);
@@ -1020,6 +1002,7 @@ __global__ void __launch_bounds__(512, 2) k_df_spmv_dia(const DiaOffs offs, int 
   if (SK && tr.nt > 0) tile_fetch<TU>(smraw, lay, tv, tr, 0);
   pdl_next();
   pdl_wait();
+  x = pdl_fresh(x);
   for (int k = 0; k < tr.nt; ++k) {
     TU* v = TileBuf<TU>(smraw, lay, tv, k).v;
     const int64_t r0 = tr.row(k);
@@ -1180,6 +1163,8 @@ __global__ void __launch_bounds__(512, MINB) k_df_update_sketch(
       prefetch_rows(U + tr.row(k) + (int64_t)col * ldu, tr.rows(k));
   }
   pdl_wait();
+  nrs = pdl_fresh(nrs);
+  sj = pdl_fresh(sj);
   for (int col = threadIdx.x; col < c; col += blockDim.x) rsh[col] = nrs[col];
   __syncthreads();
   const float2 sc = sj[0];
@@ -1783,6 +1768,7 @@ __global__ void __launch_bounds__(512) k_df_sketch_vec(const TU* __restrict__ x,
   if (tr.nt > 0) tile_fetch<TU>(smraw, lay, tv, tr, 0);
   pdl_next();
   pdl_wait();
+  x = pdl_fresh(x);
   for (int k = 0; k < tr.nt; ++k) {
     TU* v = TileBuf<TU>(smraw, lay, tv, k).v;
     const int64_t r0 = tr.row(k);
@@ -2959,13 +2945,16 @@ int build_sketch_tiles(int64_t n, int d, int zeta, const uint16_t* otab, SketchT
   t.ntile = (int)row.size() - 1;
   t.H = 1;
   while (t.H < 8 && (int64_t)d * t.H * 2 <= 512) t.H *= 2;
+  // two device blocks (row bounds, CTA bounds and the longest list; positions,
+  // slot offsets and entries): an allocation costs about as much as the
+  // kernels that fill them
+  const size_t nrow = row.size(), nct = ctile.size();
+  row.resize(nrow + (nct + 2) / 2, 0);                 // ctile and a zero behind the rows, in one copy
+  std::copy(ctile.begin(), ctile.end(), reinterpret_cast<int*>(row.data() + nrow));
   cudaError_t e = cudaMalloc(&t.row, row.size() * sizeof(int64_t));
-  if (e == cudaSuccess) e = cudaMalloc(&t.ctile, ctile.size() * sizeof(int));
+  t.ctile = reinterpret_cast<int*>(t.row + nrow);
+  int* lmax = t.ctile + nct;
   if (e == cudaSuccess) e = cudaMemcpy(t.row, row.data(), row.size() * sizeof(int64_t), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(t.ctile, ctile.data(), ctile.size() * sizeof(int), cudaMemcpyHostToDevice);
-  int* lmax = nullptr;
-  if (e == cudaSuccess) e = cudaMalloc(&lmax, sizeof(int));
-  if (e == cudaSuccess) e = cudaMemsetAsync(lmax, 0, sizeof(int), st);
   const int slots = omega_slots(zeta);
   const size_t smc = (size_t)d * sizeof(int);
   if (e == cudaSuccess) {
@@ -2977,11 +2966,14 @@ int build_sketch_tiles(int64_t n, int d, int zeta, const uint16_t* otab, SketchT
   int L = 0;
   if (e == cudaSuccess) e = cudaMemcpyAsync(&L, lmax, sizeof(int), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  cudaFree(lmax);
   t.L = L;
-  if (e == cudaSuccess) e = cudaMalloc(&t.meta, (size_t)t.ntile * d * sizeof(uint32_t));
-  if (e == cudaSuccess) e = cudaMalloc(&t.off, (size_t)t.ntile * (L + 1) * sizeof(int));
-  if (e == cudaSuccess) e = cudaMalloc(&t.ent, (size_t)n * zeta * sizeof(uint16_t));
+  auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
+  const size_t bm = al((size_t)t.ntile * d * sizeof(uint32_t)), bo = al((size_t)t.ntile * (L + 1) * sizeof(int));
+  if (e == cudaSuccess) e = cudaMalloc(&t.meta, bm + bo + (size_t)n * zeta * sizeof(uint16_t));
+  if (e == cudaSuccess) {
+    t.off = reinterpret_cast<int*>(reinterpret_cast<char*>(t.meta) + bm);
+    t.ent = reinterpret_cast<uint16_t*>(reinterpret_cast<char*>(t.meta) + bm + bo);
+  }
   const size_t smb = ((size_t)4 * d + L + 1) * sizeof(int);
   if (e == cudaSuccess) {
     if (slots == 4) k_tiles_build<4><<<t.ntile, 256, smb, st>>>(t.row, d, zeta, L, otab, t.meta, t.off, t.ent);
@@ -2995,7 +2987,8 @@ int build_sketch_tiles(int64_t n, int d, int zeta, const uint16_t* otab, SketchT
 }
 
 void free_sketch_tiles(SketchTiles* t) {
-  cudaFree(t->row); cudaFree(t->ctile); cudaFree(t->meta); cudaFree(t->off); cudaFree(t->ent);
+  cudaFree(t->row);
+  cudaFree(t->meta);
   *t = SketchTiles();
 }
 

@@ -36,6 +36,7 @@
 #include "../../include/rks.h"
 #include "convert.cuh"
 #include "dense.h"
+#include "pdl.cuh"
 #include "rks_impl.h"
 
 namespace {
@@ -130,7 +131,8 @@ __global__ void __launch_bounds__(kRgsThreads) k_rgs_panel(RgsState g, int p0, i
 // Then (next >= 0) column p0 + next against the panel's columns before it,
 // twice: the coefficients of its update.  One CTA, 11 us at d = 320, in place
 // of a copy to the host, its loops and a copy back; with the panels' share the
-// 80-column RGS at n = 1e6 went from 8.8 to 8.0 ms.
+// 80-column RGS at n = 1e6 went from 8.8 to 8.0 ms, and from 7.4 to 7.0 ms with
+// the division per row gone and the launch overlapped with the fold.
 __global__ void __launch_bounds__(kRgsThreads) k_rgs_col(RgsState g, int p0, int done, int next) {
   extern __shared__ double rgs_sm[];
   double* z = rgs_sm;
@@ -138,6 +140,10 @@ __global__ void __launch_bounds__(kRgsThreads) k_rgs_col(RgsState g, int p0, int
   __shared__ double red[kRgsThreads / 32 + 1];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int j = p0 + done;
+  rks::pdl_next();
+  if (next >= 0)                       // written before the update in front of the fold
+    for (int i = threadIdx.x; i < g.d; i += kRgsThreads) z[i] = g.P[i + (size_t)next * g.d];
+  rks::pdl_wait();
   double bb = 0.0;
   for (int i = threadIdx.x; i < g.d; i += kRgsThreads) {
     const double v = g.sum[i] * g.zscale;
@@ -151,15 +157,13 @@ __global__ void __launch_bounds__(kRgsThreads) k_rgs_col(RgsState g, int p0, int
     for (int q = 0; q < kRgsThreads / 32; ++q) t += red[q];
     const double beta = sqrt(t);
     if (!(beta > 0.0) || !isfinite(beta)) *g.flag = 1;
-    red[kRgsThreads / 32] = beta;
     g.R[j + (size_t)j * g.s] = beta;
-    g.cs[j] = 1.0 / beta;
+    g.cs[j] = red[kRgsThreads / 32] = 1.0 / beta;
   }
   __syncthreads();
-  const double beta = red[kRgsThreads / 32];
+  const double inv = red[kRgsThreads / 32];
   for (int i = threadIdx.x; i < g.d; i += kRgsThreads) {
-    g.S[i + (size_t)j * g.d] = g.sum[i] * g.zscale / beta;
-    if (next >= 0) z[i] = g.P[i + (size_t)next * g.d];
+    g.S[i + (size_t)j * g.d] = g.sum[i] * g.zscale * inv;   // a division per row is nine FP64 operations
   }
   if (next < 0) return;
   __syncthreads();
@@ -198,11 +202,11 @@ struct QrWork {
   float2* sj = nullptr;       // scale of the updated column
   double* scale = nullptr;    // s column scales for the output
   double* dense = nullptr;    // small matrices of the randomized Gram-Schmidt
+  char* small = nullptr;      // the block that holds sums, Q2, nrs, sj, scale, dense and flag
   int* flag = nullptr;
   std::vector<double> host;   // sums read back
   ~QrWork() {
-    cudaFree(U); cudaFree(otab); cudaFree(part); cudaFree(sums); cudaFree(Q2); cudaFree(nrs); cudaFree(sj);
-    cudaFree(scale); cudaFree(dense); cudaFree(flag);
+    cudaFree(U); cudaFree(otab); cudaFree(part); cudaFree(small);
     if (have_tiles) rks::free_sketch_tiles(&tiles);
   }
 };
@@ -219,15 +223,27 @@ int setup(QrWork& w, int64_t n, int s, int d, int zeta, uint64_t seed, cudaStrea
   w.zscale = 1.0 / std::sqrt((double)zeta);
   w.ldu = (n + 31) / 32 * 32;
   const size_t nsum = std::max((size_t)d * s, (size_t)rks::gram_pairs(s));
+  // one block for the small arrays (and two for the tiles): seven allocations
+  // fewer took randomized Cholesky QR of 50 021 x 24 from 832 to 740 us
+  const size_t small[7] = {nsum * sizeof(double), (size_t)s * s * sizeof(float2),
+                           (size_t)rks::kPanelCols * s * sizeof(float2), sizeof(float2), (size_t)s * sizeof(double),
+                           ((size_t)d * (1 + rks::kPanelCols + s) + (size_t)s * s) * sizeof(double), sizeof(int)};
+  size_t at[7], total = 0;
+  for (int q = 0; q < 7; ++q) {
+    at[q] = total;
+    total += (small[q] + 255) & ~(size_t)255;
+  }
   if (cudaMalloc(&w.U, (size_t)w.ldu * ncol * sizeof(float2)) != cudaSuccess ||
       cudaMalloc(&w.otab, (size_t)nsk * rks::omega_slots(zeta) * sizeof(uint16_t)) != cudaSuccess ||
-      cudaMalloc(&w.sums, nsum * sizeof(double)) != cudaSuccess ||
-      cudaMalloc(&w.Q2, (size_t)s * s * sizeof(float2)) != cudaSuccess ||
-      cudaMalloc(&w.nrs, (size_t)rks::kPanelCols * s * sizeof(float2)) != cudaSuccess ||
-      cudaMalloc(&w.sj, sizeof(float2)) != cudaSuccess ||
-      cudaMalloc(&w.scale, (size_t)s * sizeof(double)) != cudaSuccess ||
-      cudaMalloc(&w.flag, sizeof(int)) != cudaSuccess)
+      cudaMalloc(&w.small, total) != cudaSuccess)
     return RKS_ENOMEM;
+  w.sums = reinterpret_cast<double*>(w.small + at[0]);
+  w.Q2 = reinterpret_cast<float2*>(w.small + at[1]);
+  w.nrs = reinterpret_cast<float2*>(w.small + at[2]);
+  w.sj = reinterpret_cast<float2*>(w.small + at[3]);
+  w.scale = reinterpret_cast<double*>(w.small + at[4]);
+  w.dense = reinterpret_cast<double*>(w.small + at[5]);
+  w.flag = reinterpret_cast<int*>(w.small + at[6]);
   w.host.assign(nsum, 0.0);
   QK(cudaMemsetAsync(w.flag, 0, sizeof(int), st));
   rks::launch_omega_table(nsk, d, zeta, seed, w.otab, w.flag, st);
@@ -335,8 +351,6 @@ int whiten(QrWork& w, const double* K, int64_t ldk, std::vector<double>& R1, std
 int rgs(QrWork& w, const double* K, int64_t ldk, std::vector<double>& R, std::vector<double>& S) {
   constexpr int B = rks::kPanelCols;
   const int s = w.s, d = w.d;
-  const size_t need = (size_t)d * (1 + B + s) + (size_t)s * s;
-  QK(cudaMalloc(&w.dense, need * sizeof(double)));
   RgsState g;
   g.s = s; g.d = d; g.zscale = w.zscale;
   g.Z = w.sums; g.cs = w.scale; g.nrs = w.nrs; g.flag = w.flag;
@@ -363,11 +377,11 @@ int rgs(QrWork& w, const double* K, int64_t ldk, std::vector<double>& R, std::ve
     if (p0 > 0) rks::launch_df_panel(w.n, w.U, w.ldu, p0, p0, nb, w.nrs, w.st);
     for (int jj = 0; jj < nb; ++jj) {
       // q~ = k_j - sum_c (q~_c / beta_c) r_c, fused with its partial sketches
-      if (jj > 0) k_rgs_col<<<1, kRgsThreads, sm, w.st>>>(g, p0, jj - 1, jj);
+      if (jj > 0) rks::launch_pdl(k_rgs_col, 1, kRgsThreads, sm, w.st, g, p0, jj - 1, jj);
       rks::launch_df_update_sketch(col(w, p0), w.ldu, jj, w.nrs, w.sj, w.tiles, w.part, false, w.st);
       rks::launch_df_fold(w.part, d, w.tiles.G, g.sum, w.st);
     }
-    k_rgs_col<<<1, kRgsThreads, sm, w.st>>>(g, p0, nb - 1, -1);
+    rks::launch_pdl(k_rgs_col, 1, kRgsThreads, sm, w.st, g, p0, nb - 1, -1);
   }
   QK(cudaGetLastError());
   int bad = 0;
