@@ -984,8 +984,9 @@ struct DiaOffs {
 // order (the CSR kernel's order, the same bits); two rows per thread, the
 // tiles and the sketch gather of k_df_spmv_ell.
 // ND > 0: exactly ND diagonals, so that an interior tile's loads need neither
-// a test nor a zero (rows past a ragged tile's end are read, not stored).
-// DIATIME
+// a test nor a zero (rows past a ragged tile's end are read, not stored): pairs,
+// 5 diagonals, n = 1e6, d = 320: 29.4 -> 24.2 us; FP32, 7 diagonals,
+// n = 4.1e6, d = 96: 73 -> 71 us (64 us with the gather's last form).
 template <class TU, class TA, bool SK, int DMAX, int ND = 0>
 __global__ void __launch_bounds__(512, 2) k_df_spmv_dia(const DiaOffs offs, int D, const TA* __restrict__ dv,
                                                      int64_t ldd, int64_t n, const TU* __restrict__ x,
