@@ -117,8 +117,12 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, int* f
   return mbar_try(mbar, parity) || mbar_wait_slow(mbar, parity, flag);
 }
 
+// Aligned instructions: all 32 lanes execute them together.  The lanes come
+// here from bounded waits of their own and from stores guarded by the row, so
+// they are brought together first.
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
   uint32_t r[8];
+  __syncwarp();
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
                : "r"(taddr));
@@ -284,7 +288,6 @@ __global__ void __launch_bounds__(kF32All, 3) k_tc_restart_f32(int64_t n, const 
       // epilogue
       if (ok) ok = mbar_wait(done_b, dpar, flag);
       dpar ^= 1u;
-      __syncwarp();
       fence_after();
       const int q4 = warp & 3;
       const int64_t ir = tile * kM + q4 * 32 + lane;
@@ -712,6 +715,7 @@ __global__ void __launch_bounds__(kDfAllThreads, MINB) k_tc_restart_df(int64_t n
       if (mvsrc && warp < 4 && ir < n) mvdst[ir] = mv;
       fence_before();
       mbar_arrive(tfree_b);
+      __syncwarp();
       asm volatile("bar.sync 1, %0;" ::"n"(kDfThreads) : "memory");   // the next tile's row exponents
     }
   }
