@@ -201,6 +201,16 @@ void* thread_block() {
   return p;
 }
 
+// Whether a value of out (n x nout) lies in another row of U (n x nin, the
+// same leading dimension).
+bool rows_cross(const double* U, int nin, const double* out, int nout, int64_t n, int64_t ldu) {
+  const intptr_t u = (intptr_t)U, v = (intptr_t)out, col = (intptr_t)(ldu * sizeof(double));
+  const intptr_t row = (intptr_t)(n * sizeof(double));
+  if (v >= u + (nin - 1) * col + row || u >= v + (nout - 1) * col + row) return false;
+  const intptr_t at = ((v - u) % col + col) % col;   // of out's first row within a column of U
+  return at != 0 && !(at >= row && at + row <= col);
+}
+
 int launch_err() {
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
@@ -1859,12 +1869,24 @@ int rks_basis_product_df(int64_t n, const double* U, int64_t ldu, int nin, const
   void* dblob = thread_block();
   if (!flag || !dblob) return RKS_ENOMEM;
   *flag = 0;
+  // the kernel writes a tile's rows while other tiles are still to be read: a
+  // result that shares memory with other rows of U goes by a copy
+  double* to = out;
+  if (rows_cross(U, nin, out, nout, n, ldu) &&
+      cudaMalloc(&to, ((size_t)ldu * (nout - 1) + n) * sizeof(double)) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return RKS_ENOMEM;
+  }
   cudaError_t e = cudaMemcpyAsync(dblob, blob.data(), blob.size(), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) {
-    rks::launch_tc_product_f64(n, U, out, ldu, nin, nout, dblob, flag, st);
+    rks::launch_tc_product_f64(n, U, to, ldu, nin, nout, dblob, flag, st);
     e = cudaGetLastError();
   }
+  for (int o = 0; to != out && o < nout && e == cudaSuccess; ++o)
+    e = cudaMemcpyAsync(out + (size_t)o * ldu, to + (size_t)o * ldu, (size_t)n * sizeof(double),
+                        cudaMemcpyDeviceToDevice, st);
   const cudaError_t es = cudaStreamSynchronize(st);
+  if (to != out) cudaFree(to);
   if (e != cudaSuccess || es != cudaSuccess) return RKS_ECUDA;
   return (*flag & rks::RKS_FLAG_TIMEOUT) ? RKS_ETIMEOUT : RKS_OK;
 }
