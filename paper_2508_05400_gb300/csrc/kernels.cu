@@ -123,22 +123,29 @@ __global__ void k_sketch_vec(int64_t n, const double* __restrict__ x, double sca
 
 // The same sums in fixed point.  What bounds the FP64 form is the shared-
 // memory FP64 atomic (a compare-and-swap loop) and the sequential hash; here
-// a tile's values become 59-bit integers relative to a shared power of two,
-// cut into three 20-bit limbs that are added with native 32-bit integer
-// atomics (a tile has at most 2048 rows and a row meets a bin at most once,
-// so a limb sum stays below 2^31), and all zeta draws of a row are hashed at
-// once, repeats redrawn afterwards.  The limbs go to 64-bit integers per
-// tile; FP64 appears only when a CTA hands its bins over (at its end, or when
-// a later tile outgrows the power of two).  An addend is off by at most
-// 2^-58 of the largest |x| of its CTA, less than one rounding of the FP64
-// sums.  A tile that holds an infinity or a NaN adds its values in FP64.
-// Measured, n = 4 096 000, d = 600, zeta = 8: 239 us with FP64 bins, 165 us
-// here (three shared atomics per entry are now the bound; HBM would take
-// 5 us); the whole rks_sketch_apply call 456 -> 186 us, and 210 -> 27 us at
-// n = 20 000 (no allocation, no copy of the sums to the host and back).
+// a tile's values become integers in units of 2^-78 of a shared power of two,
+// cut into 20-bit limbs that are added with native 32-bit integer atomics (a
+// tile has at most 2048 rows and a row meets a bin at most once, so a limb sum
+// stays below 2^31), and all zeta draws of a row are hashed at once, repeats
+// redrawn afterwards.  The limbs go to 80-bit sums per tile; FP64 appears only
+// when a CTA hands its bins over (at its end, or when a tile's largest value
+// leaves the power of two).
+//
+// No addend loses a bit: a value takes the limbs its 53 bits reach, three
+// within 2^-4 of the tile's largest, four within 2^-24, and one that is
+// smaller still, or is no number, goes to FP64 bins beside the integers.  (With
+// three limbs for everything a bin without large entries lost the low bits
+// of its small ones.)
+// Measured, n = 4 096 000, d = 600, zeta = 8, the whole rks_sketch_apply call
+// (the shared atomics are the bound; HBM would take 5 us): 453 us with FP64
+// bins, allocations and a copy of the sums to the host and back; 204 us here
+// (186 us with three limbs and rounded values); 207 -> 27 us at n = 20 000.
+// With exponents at random over the whole range, where the FP64 bins take all:
+// 423 -> 383 us.
+constexpr int kFixSpan = 8;       // binades a tile's largest value may lie below the power of two
 constexpr int kFixThreads = 512;
 constexpr int kFixTile = 2048;
-constexpr int kFixMaxD = 3072;    // bins: 28 bytes each, two CTAs per SM
+constexpr int kFixMaxD = 3072;    // 40 bytes a bin
 
 // One distinct-row draw set: rows[t] and signs (bit t of the result) of
 // column i; false if the draw cap was reached.
@@ -191,46 +198,49 @@ __global__ void __launch_bounds__(kFixThreads) k_sketch_vec_fix(int64_t n, int t
                                                                 double* __restrict__ out, int* flag) {
   constexpr int RPT = kFixTile / kFixThreads;
   extern __shared__ __align__(8) unsigned char fixmem[];
-  long long* hi = reinterpret_cast<long long*>(fixmem);   // d: sums in units of 2^40
-  long long* lo = hi + d;                                  // d: remainders
-  int* limb = reinterpret_cast<int*>(lo + d);              // 3 x d
+  long long* hi = reinterpret_cast<long long*>(fixmem);   // d: sums in units of 2^60
+  long long* lo = hi + d;                                  // d: remainders in -2^59 .. 2^59
+  double* fb = reinterpret_cast<double*>(lo + d);          // d: FP64 sums of what the limbs do not take
+  int* limb = reinterpret_cast<int*>(fb + d);              // 4 x d, lowest first
   __shared__ int wmax[kFixThreads / 32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int b = tid; b < d; b += kFixThreads) {
     hi[b] = 0;
     lo[b] = 0;
-    limb[b] = 0;
-    limb[b + d] = 0;
-    limb[b + 2 * d] = 0;
+    fb[b] = 0.0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) limb[b + q * d] = 0;
   }
-  auto hand_over = [&](int es) {   // bins to out, in FP64
-    for (int b = tid; b < d; b += kFixThreads) {
-      const double v = (double)hi[b] * 1099511627776.0 + (double)lo[b];
-      if (v != 0.0) atomicAdd(&out[b], scalbn(v, es - 1081) * scale);
-    }
+  // a bin's integer sum in FP64; its owner thread alone reads and writes it
+  auto sum_of = [&](int b, int es) {
+    return scalbn((double)hi[b] * 1152921504606846976.0 + (double)lo[b], es - 1101);
   };
   const int64_t ntile = (n + tile - 1) / tile;
   const int64_t t0 = blockIdx.x * ntile / gridDim.x, t1 = (blockIdx.x + 1) * ntile / gridDim.x;
-  int es = -1;                     // |x| < 2^(es - 1022); -1: no tile yet
+  int es = -1;                     // |x| < 2^(es - 1022) for the integers; -1: none yet
   for (int64_t t = t0; t < t1; ++t) {
     const int64_t r0 = t * tile;
     const int rows = (int)(n - r0 < tile ? n - r0 : tile);
     unsigned long long xb[RPT];
-    int em = 0;
+    int em = 0;                    // largest exponent of the tile's numbers, 0: all are zero
 #pragma unroll
     for (int k = 0; k < RPT; ++k) {
       const int l = tid + k * kFixThreads;
       xb[k] = l < rows ? (unsigned long long)__double_as_longlong(x[r0 + l]) : 0ull;
-      em = max(em, (int)((xb[k] >> 52) & 0x7FF));
+      const int E = (int)((xb[k] >> 52) & 0x7FF);
+      if ((xb[k] << 1) != 0 && E != 0x7FF) em = max(em, max(E, 1));
     }
     em = __reduce_max_sync(0xffffffffu, em);
     if (lane == 0) wmax[warp] = em;
     __syncthreads();
-    em = max(1, __reduce_max_sync(0xffffffffu, wmax[lane & (kFixThreads / 32 - 1)]));
-    const bool special = em == 0x7FF;
-    if (!special && em > es) {     // the bins' owners read only what they wrote
-      if (es >= 0) hand_over(es);
-      for (int b = tid; b < d; b += kFixThreads) { hi[b] = 0; lo[b] = 0; }
+    em = __reduce_max_sync(0xffffffffu, wmax[lane & (kFixThreads / 32 - 1)]);
+    if (em > es || (em > 0 && em < es - kFixSpan)) {
+      for (int b = tid; b < d; b += kFixThreads) {
+        const double v = es >= 0 ? sum_of(b, es) : 0.0;
+        if (v != 0.0) atomicAdd(&out[b], v * scale);
+        hi[b] = 0;
+        lo[b] = 0;
+      }
       es = em + 2;
     }
 #pragma unroll
@@ -240,19 +250,25 @@ __global__ void __launch_bounds__(kFixThreads) k_sketch_vec_fix(int64_t n, int t
       int rw[MAXZ];
       unsigned neg;
       if (!omega_rows<MAXZ>(seed, (uint64_t)(r0 + l), d, zeta, rw, neg)) { atomicOr(flag, RKS_FLAG_HASH); continue; }
-      if (special) {
-        const double v = __longlong_as_double((long long)xb[k]) * scale;
-#pragma unroll
-        for (int u = 0; u < MAXZ; ++u)
-          if (u < zeta) atomicAdd(&out[rw[u]], (neg >> u) & 1u ? -v : v);
-        continue;
-      }
       int E = (int)((xb[k] >> 52) & 0x7FF);
       unsigned long long m = xb[k] & 0xFFFFFFFFFFFFFull;
       if (E) m |= 1ull << 52; else E = 1;
-      const int sh = E - es + 6;
-      if (sh >= 0) m <<= sh;
-      else m = sh >= -54 ? (m + (1ull << (-sh - 1))) >> -sh : 0ull;
+      const int sh = E - es + 6;   // at most 6
+      if (E == 0x7FF || sh < -20) {
+        const double v = __longlong_as_double((long long)xb[k]);
+        if (v != 0.0)
+#pragma unroll
+          for (int u = 0; u < MAXZ; ++u)
+            if (u < zeta) atomicAdd(&fb[rw[u]], (neg >> u) & 1u ? -v : v);
+        continue;
+      }
+      int lf = 0;
+      if (sh >= 0) {
+        m <<= sh;
+      } else {
+        lf = (int)((m & ((1ull << -sh) - 1)) << (20 + sh));
+        m >>= -sh;
+      }
       const int l0 = (int)(m & 0xFFFFF), l1 = (int)((m >> 20) & 0xFFFFF), l2 = (int)(m >> 40);
       neg ^= (xb[k] >> 63) ? ~0u : 0u;
 #pragma unroll
@@ -260,24 +276,28 @@ __global__ void __launch_bounds__(kFixThreads) k_sketch_vec_fix(int64_t n, int t
         if (u < zeta) {
           const int sg = -(int)((neg >> u) & 1u);
           int* q = limb + rw[u];
-          atomicAdd(q, (l0 ^ sg) - sg);
-          atomicAdd(q + d, (l1 ^ sg) - sg);
-          atomicAdd(q + 2 * d, (l2 ^ sg) - sg);
+          if (lf) atomicAdd(q, (lf ^ sg) - sg);
+          atomicAdd(q + d, (l0 ^ sg) - sg);
+          atomicAdd(q + 2 * d, (l1 ^ sg) - sg);
+          atomicAdd(q + 3 * d, (l2 ^ sg) - sg);
         }
     }
     __syncthreads();
     for (int b = tid; b < d; b += kFixThreads) {
-      long long s = lo[b] + ((long long)limb[b + d] << 20) + limb[b];
-      const long long c = s >> 40;
-      hi[b] += limb[b + 2 * d] + c;
-      lo[b] = s - (c << 40);
-      limb[b] = 0;
-      limb[b + d] = 0;
-      limb[b + 2 * d] = 0;
+      const int mid = limb[b + 2 * d];
+      const long long s = lo[b] + limb[b] + ((long long)limb[b + d] << 20) + ((long long)(mid & 0xFFFFF) << 40);
+      const long long c = (s + (1ll << 59)) >> 60;
+      hi[b] += limb[b + 3 * d] + (mid >> 20) + c;
+      lo[b] = s - (c << 60);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) limb[b + q * d] = 0;
     }
     __syncthreads();
   }
-  if (es >= 0) hand_over(es);
+  for (int b = tid; b < d; b += kFixThreads) {
+    const double v = (es >= 0 ? sum_of(b, es) : 0.0) + fb[b];
+    if (v != 0.0) atomicAdd(&out[b], v * scale);
+  }
 }
 
 // w = A (x * xscale[0]); out_raw += Omega-sums of w.
@@ -664,8 +684,10 @@ void launch_sketch_vec(int64_t n, const double* x, double scale, int d, int zeta
     // tiles of 2048 rows (a flush of d bins each) once every SM has one,
     // smaller ones before, so that short vectors still use many SMs
     const int tile = n >= (int64_t)152 * kFixTile ? kFixTile : (n >= (int64_t)76 * kFixTile ? kFixTile / 2 : kFixThreads);
-    const int g = (int)((n + tile - 1) / tile < 152 * 3 ? (n + tile - 1) / tile : 152 * 3);
-    const size_t sm = (size_t)d * 28;
+    // two CTAs per SM: a third adds contention for the bins (226 us instead of
+    // 204 at n = 4 096 000, d = 600; 471 instead of 383 where FP64 bins take all)
+    const int g = (int)((n + tile - 1) / tile < 152 * 2 ? (n + tile - 1) / tile : 152 * 2);
+    const size_t sm = (size_t)d * 40;
     if (zeta <= 4) k_sketch_vec_fix<4><<<g, kFixThreads, sm, st>>>(n, tile, x, scale, d, zeta, seed, out, flag);
     else if (zeta <= 8) k_sketch_vec_fix<8><<<g, kFixThreads, sm, st>>>(n, tile, x, scale, d, zeta, seed, out, flag);
     else k_sketch_vec_fix<16><<<g, kFixThreads, sm, st>>>(n, tile, x, scale, d, zeta, seed, out, flag);
