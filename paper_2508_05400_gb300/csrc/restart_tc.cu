@@ -402,14 +402,21 @@ struct Split<double> {
   static __device__ __forceinline__ Key key(Key k, Probe v, float) { return max(k, v & 0x7FFFFFFF); }
   static __device__ __forceinline__ int key_exp(Key k) { return max(k >> 20, 1); }
   static __device__ __forceinline__ int scale(int emax) { return emax - 1021; }
-  static __device__ __forceinline__ int row(int emax) { return (131 - emax) * (1 << 20); }
-  static __device__ __forceinline__ void scaled(double v, float, int rowk, float& x, float& y) {
+  // k moves a high word to the row's scale; from x0 and y0 on, the moved word
+  // gives x and y.  A zero or subnormal value (no leading one to move) lies
+  // below x0 in every row: it counts as zero.
+  struct Row { int k, x0, y0; };
+  static __device__ __forceinline__ Row row(int emax) {
+    const int k = (131 - emax) * (1 << 20), x0 = max(k, 0) + (1 << 20);
+    return {k, x0, max(x0, 47 << 20)};
+  }
+  static __device__ __forceinline__ void scaled(double v, float, const Row& r, float& x, float& y) {
     const int hi = __double2hiint(v), lo = __double2loint(v);
-    const int d = (hi & 0x7FFFFFFF) + rowk;                 // biased exponent of x, 20 bits of mantissa
+    const int d = (hi & 0x7FFFFFFF) + r.k;                  // biased exponent of x, 20 bits of mantissa
     const int xb = __funnelshift_l(lo, d, 3), sg = hi & 0x80000000;
     const float yi = __int_as_float((((lo & 0x1FFFFFFF) + 32) >> 6) + 0x4B000000) - 8388608.0f;
-    x = d >= 1 << 20 ? __int_as_float(xb | sg) : 0.f;
-    y = d >= 47 << 20 ? yi * __int_as_float(((xb & 0x7F800000) - (46 << 23)) | sg) : 0.f;
+    x = d >= r.x0 ? __int_as_float(xb | sg) : 0.f;
+    y = d >= r.y0 ? yi * __int_as_float(((xb & 0x7F800000) - (46 << 23)) | sg) : 0.f;
   }
 };
 
