@@ -641,7 +641,8 @@ __global__ void __launch_bounds__(kDfAllThreads, MINB) k_tc_restart_df(int64_t n
       fence_after();
       const int q4 = warp & 3;
       const int64_t ir = tile * kM + q4 * 32 + lane;
-      const int er = S::scale(max((int)re[q4 * 32 + lane], (int)re[kM + q4 * 32 + lane])) - 12;
+      const int em = max((int)re[q4 * 32 + lane], (int)re[kM + q4 * 32 + lane]);
+      const int er = S::scale(em) - 12;
       T mv{};
       if (mvsrc && warp < 4 && ir < n) mv = mvsrc[ir];
       for (int cg = warp >> 2; cg < N / 8; cg += kDfThreads / 128) {
@@ -710,8 +711,10 @@ __global__ void __launch_bounds__(kDfAllThreads, MINB) k_tc_restart_df(int64_t n
                 const int sc = er + head->fexp[o] - 42;
                 const double d = __ll2double_rn(acc[jj]);
                 const int hi = __double2hiint(d), e = ((hi >> 20) & 0x7FF) + sc;
-                // scaling by an exponent add where the result is a normal number
-                out[ir + (int64_t)o * ldu] = (hi & 0x7FF00000) == 0 ? d
+                // scaling by an exponent add where the result is a normal number;
+                // a row with an infinity or a NaN has no digits to add up
+                out[ir + (int64_t)o * ldu] = em == 0x7FF             ? __hiloint2double(0x7FF80000, 0)
+                                             : (hi & 0x7FF00000) == 0 ? d
                                              : e > 0 && e < 0x7FF   ? __hiloint2double(hi + (sc << 20), __double2loint(d))
                                                                     : scalbn(d, sc);
               }
