@@ -43,8 +43,8 @@ __device__ __forceinline__ float2 df_from_double(double x) {
   }
   const int m = ((xh & 0xFFFFF) << 3) | (int)((unsigned)xl >> 29), low = xl & 0x1FFFFFFF;
   const int up = low > 0x10000000 || (low == 0x10000000 && (m & 1)) ? 1 : 0;
-  const int sg = xh & 0x80000000;
-  const float l = __int2float_rn(low - (up << 29)) * __int_as_float(((E - 948) << 23) | sg);
+  const int sg = xh & 0x80000000, rest = low - (up << 29);
+  const float l = __int2float_rn(sg ? -rest : rest) * __int_as_float((E - 948) << 23);   // +0 where hi is all of x
   return make_float2(__int_as_float(((((E - 896) << 23) | m) + up) | sg), l);
 }
 
