@@ -123,7 +123,8 @@ __global__ void __launch_bounds__(256) k_conv3x3(const float* __restrict__ z, in
   float* ws = sm + 2 * kCvStage * kCvPlane;     // (cin * 9) x 4 groups x OUTS
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int og = tid >> 6, xg = tid & 7, ty = (tid >> 3) & 7;
-  const int x0 = blockIdx.x * kCvW, y0 = blockIdx.y * kCvH;
+  const int tiles_x = (W + kCvW - 1) / kCvW;    // tiles in grid.x: a grid of 65 536 tile rows is legal
+  const int x0 = blockIdx.x % tiles_x * kCvW, y0 = blockIdx.x / tiles_x * kCvH;
   const int o0 = (blockIdx.z * 4 + og) * OUTS;
   const size_t hw = (size_t)H * W;
   auto stage = [&](int c0, float* dst) {        // a warp a channel
@@ -713,9 +714,9 @@ void conv(rks_ws* s, int l, int lv, const float* z, bool back, int relu, const f
     k_conv3x3_one<<<grid, 256, (size_t)(cin * kHalo2 + cin * 9) * sizeof(float), s->st>>>(z, cin, H, W, w, bias, out);
     return;
   }
-  dim3 grid((W + kCvW - 1) / kCvW, (H + kCvH - 1) / kCvH);
-  const bool wide = (int64_t)grid.x * grid.y >= kCvWideFrom;
-  grid.z = wide ? 1 : 2;
+  const int tiles = ((W + kCvW - 1) / kCvW) * ((H + kCvH - 1) / kCvH);
+  const bool wide = tiles >= kCvWideFrom;
+  const dim3 grid(tiles, 1, wide ? 1 : 2);
   const size_t sm = (size_t)(2 * kCvStage * kCvPlane + cin * 36 * (wide ? 8 : 4)) * sizeof(float);
   if (wide) k_conv3x3<8><<<grid, 256, sm, s->st>>>(z, cin, H, W, w, bias, relu, omask, out);
   else k_conv3x3<4><<<grid, 256, sm, s->st>>>(z, cin, H, W, w, bias, relu, omask, out);
