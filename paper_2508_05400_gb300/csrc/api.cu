@@ -56,7 +56,7 @@ struct rks_ctx {
   double* Qd = nullptr;
   double* u1 = nullptr;
   double* X = nullptr;
-  double* AX = nullptr;
+  double* Uk = nullptr;
   double* rsum = nullptr;
   int* pcol = nullptr;
   double* plam = nullptr;
@@ -824,16 +824,16 @@ void ritz(rks_ctx* c) {
   c->nw = nw;
 }
 
-// Ritz vectors X = U Y (real packing), A X and FP64 residuals.
+// Ritz vectors X = U Y (real packing) and FP64 residuals.
 int finalize(rks_ctx* c) {
   const int kk = c->kk, nw = c->nw;
   if (!c->X) {
-    // X holds the nw <= k + 1 Ritz vectors; AX also serves as FP64 scratch
-    // for the kk <= min(m, 2k + 1) kept basis columns
+    // X holds the nw <= k + 1 Ritz vectors; Uk the kk <= min(m, 2k + 1) kept
+    // columns of a basis that is not FP64, converted
     const int ncx = std::min(c->m + 1, 2 * c->k + 2);
     int rc = dalloc(&c->X, (size_t)c->ldu * ncx);
     if (rc) return rc;
-    rc = dalloc(&c->AX, (size_t)c->ldu * ncx);
+    if (c->prec != RKS_PREC_FP64) rc = dalloc(&c->Uk, (size_t)c->ldu * ncx);
     if (rc) return rc;
     rc = dalloc(&c->rsum, (size_t)4 * (c->k + 1) * rks::kResidCtas);
     if (rc) return rc;
@@ -861,8 +861,8 @@ int finalize(rks_ctx* c) {
   CK(cudaMemcpyAsync(c->Qd, Yr.data(), Yr.size() * sizeof(double), cudaMemcpyHostToDevice, c->stream));
   int ps = prof_begin(c, RKS_K_OTHER);
   if (c->prec != RKS_PREC_FP64) {
-    rks::launch_df2d_cols(c->n, c->Ub, c->ldu, c->AX, c->ldu, kk, c->f32, c->stream);
-    rks::launch_rows_gemm(c->n, c->AX, c->ldu, 0, kk, c->Qd, nw, c->X, c->ldu, 0, -1, c->stream);
+    rks::launch_df2d_cols(c->n, c->Ub, c->ldu, c->Uk, c->ldu, kk, c->f32, c->stream);
+    rks::launch_rows_gemm(c->n, c->Uk, c->ldu, 0, kk, c->Qd, nw, c->X, c->ldu, 0, -1, c->stream);
   } else {
     rks::launch_rows_gemm(c->n, c->U, c->ldu, 0, kk, c->Qd, nw, c->X, c->ldu, 0, -1, c->stream);
   }
@@ -914,7 +914,7 @@ void free_ctx(rks_ctx* c) {
   cudaFree(c->U); cudaFree(c->S); cudaFree(c->colscale);
   cudaFree(c->z_raw); cudaFree(c->s_raw); cudaFree(c->z1); cudaFree(c->r1); cudaFree(c->r); cudaFree(c->rs);
   cudaFree(c->coef); cudaFree(c->flag); cudaFree(c->Qd); cudaFree(c->u1);
-  cudaFree(c->X); cudaFree(c->AX); cudaFree(c->rsum); cudaFree(c->pcol); cudaFree(c->plam);
+  cudaFree(c->X); cudaFree(c->Uk); cudaFree(c->rsum); cudaFree(c->pcol); cudaFree(c->plam);
   cudaFree(c->ell_col); cudaFree(c->ell_val2); cudaFree(c->ell_valf); cudaFree(c->dia_val2); cudaFree(c->dia_valf);
   cudaFree(c->A2.mp_row); cudaFree(c->A2.mp_val); cudaFree(c->A2.mp_w); cudaFree(c->A2.mp_part);
   cudaFree(c->vals2); cudaFree(c->U2); cudaFree(c->S2); cudaFree(c->nrs); cudaFree(c->sj); cudaFree(c->Q2);
@@ -1706,8 +1706,8 @@ int rks_get_schur(rks_ctx* c, double* T, double* U, double* b) {
   if (U) {
     const double* src = c->U;
     if (c->prec != RKS_PREC_FP64) {
-      rks::launch_df2d_cols(c->n, c->Ub, c->ldu, c->AX, c->ldu, kk, c->f32, c->stream);
-      src = c->AX;
+      rks::launch_df2d_cols(c->n, c->Ub, c->ldu, c->Uk, c->ldu, kk, c->f32, c->stream);
+      src = c->Uk;
     }
     CK(cudaMemcpy2DAsync(U, c->n * sizeof(double), src, c->ldu * sizeof(double), c->n * sizeof(double), kk,
                          c->opts.mem_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, c->stream));
