@@ -222,7 +222,7 @@ cudaError_t configure_kernels();
 // from several host threads: slot names the configuration; a failure is
 // returned and f() retried at the next call.  The record is per process and
 // is not reset by cudaDeviceReset.
-enum { kCfgBase = 0, kCfgDf = 1, kCfgTc = 2, kCfgWs = 3, kCfgSlots = 4 };
+enum { kCfgBase = 0, kCfgDf = 1, kCfgTc = 2, kCfgWs = 3, kCfgQr = 4, kCfgSlots = 5 };
 cudaError_t once_per_device(int slot, cudaError_t (*f)());
 int rows_gemm_smem(int nin, int nout, int threads);
 void launch_rows_gemm(int64_t n, const double* A, int64_t lda, int a0, int nin, const double* B, int nout,

@@ -62,6 +62,7 @@ __global__ void __launch_bounds__(256) k_df2d_scaled(int64_t n, const float2* __
 }
 
 constexpr int kRgsThreads = 256;
+constexpr int kMaxD = 8192;      // largest sketch size
 
 // Device state of the randomized Gram-Schmidt (column-major arrays).
 struct RgsState {
@@ -264,6 +265,16 @@ int setup(QrWork& w, int64_t n, int s, int d, int zeta, uint64_t seed, cudaStrea
   return RKS_OK;
 }
 
+// The largest shared memory of the small steps, once per device: a limit set
+// call by call could be lowered by another thread's smaller problem between
+// this one's setting and its launch.
+cudaError_t configure_qr_kernels_once() {
+  const int sm = (int)((kMaxD + RKS_SKETCH_QR_MAX_S) * sizeof(double));
+  cudaError_t e = cudaFuncSetAttribute(k_rgs_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_rgs_col, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+  return e;
+}
+
 float2* col(QrWork& w, int j) { return w.U + (size_t)j * w.ldu; }
 
 // U[:, c0 + o] = sum_l U[:, a0 + l] F[l, o] for o < s (F s x s, host FP64),
@@ -355,13 +366,8 @@ int rgs(QrWork& w, const double* K, int64_t ldk, std::vector<double>& R, std::ve
   g.s = s; g.d = d; g.zscale = w.zscale;
   g.Z = w.sums; g.cs = w.scale; g.nrs = w.nrs; g.flag = w.flag;
   g.sum = w.dense; g.P = g.sum + d; g.S = g.P + (size_t)d * B; g.R = g.S + (size_t)d * s;
+  if (rks::once_per_device(rks::kCfgQr, configure_qr_kernels_once) != cudaSuccess) return RKS_ECUDA;
   const size_t sm = (size_t)(d + s) * sizeof(double);
-  if (sm > 48 * 1024 &&
-      cudaFuncSetAttribute(k_rgs_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess)
-    return RKS_ECUDA;
-  if (sm > 48 * 1024 &&
-      cudaFuncSetAttribute(k_rgs_col, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess)
-    return RKS_ECUDA;
   const float2 one = make_float2(1.f, 0.f);
   QK(cudaMemcpyAsync(w.sj, &one, sizeof(float2), cudaMemcpyHostToDevice, w.st));
   QK(cudaMemsetAsync(g.R, 0, (size_t)s * s * sizeof(double), w.st));
@@ -507,7 +513,7 @@ int rhqr(QrWork& w, std::vector<double>& R, std::vector<double>& scale) {
 
 extern "C" int rks_sketch_qr(int64_t n, int s, const double* K, int64_t ldk, int d, int zeta, uint64_t seed,
                              int method, double* Q, int64_t ldq, double* R, double* S, void* stream) {
-  if (n < 2 || s < 1 || s > RKS_SKETCH_QR_MAX_S || zeta < 1 || zeta > 16 || d < 2 * zeta || d > 8192 || s > d ||
+  if (n < 2 || s < 1 || s > RKS_SKETCH_QR_MAX_S || zeta < 1 || zeta > 16 || d < 2 * zeta || d > kMaxD || s > d ||
       s > n || !K || !Q || !R || ldk < n || ldq < n)
     return RKS_EINVAL;
   if (method != RKS_QR_RGS && method != RKS_QR_WHITEN && method != RKS_QR_RCHOLQR && method != RKS_QR_RHQR)
