@@ -455,14 +455,20 @@ int rks_sketch_pairs(int64_t n, int d, int zeta, uint64_t seed, int32_t* rows, i
                      void* stream);
 
 /* z = Omega x for a device vector x (n doubles) into device z (d doubles),
- * entries sign/sqrt(zeta), FP64 accumulation.  Same requirements. */
+ * entries sign/sqrt(zeta).  Every x_i enters its sums whole: as an integer,
+ * added exactly, or (when it is far below the largest of its 2048 rows, is no
+ * number, or d > 3072) in FP64; the sums of up to 304 CTAs are scaled and
+ * added in FP64, in no fixed order.  Same requirements.  Allocates nothing per
+ * call but, once per host thread, a page-locked status word, freed when the
+ * thread ends (not valid after cudaDeviceReset).  Synchronises `stream`. */
 int rks_sketch_apply(int64_t n, int d, int zeta, uint64_t seed, const double* x, double* z,
                      void* stream);
 
 /* Largest sketch size d accepted by rks_sketch_apply_noalloc. */
 #define RKS_NOALLOC_MAX_D 8192
 
-/* z = Omega x exactly as rks_sketch_apply, but without allocating anything:
+/* z = Omega x by the kernels of rks_sketch_apply (the scale is applied to the
+ * finished sums, so the last bits may differ), but without allocating anything:
  * no cudaMalloc, cudaFree or allocating library call.  This has no
  * counterpart in the paper; it is for callers that cannot allocate device
  * memory, such as code running inside another framework's memory pool (which
@@ -493,7 +499,8 @@ int rks_sketch_apply_noalloc(int64_t n, int d, int zeta, uint64_t seed, const do
  * Q[l + o*nin] for i < n, o < nout.  U, out: device FP32 arrays with leading
  * dimension ldu >= n; out may equal U (each 128-row tile is read before it is
  * written).  Q: host FP64, nin x nout column-major, 1 <= nin <= 256,
- * 1 <= nout <= 64.  Runs on `stream` (NULL: default stream) and synchronises
+ * 1 <= nout <= 64.  Scratch as for rks_basis_product_df.  Runs on `stream`
+ * (NULL: default stream) and synchronises
  * it.  Returns RKS_OK, RKS_EINVAL (sizes, NULL pointers), RKS_ENOMEM,
  * RKS_ECUDA, or RKS_ETIMEOUT if a bounded device wait gave up. */
 int rks_basis_product_f32(int64_t n, const float* U, int64_t ldu, int nin, const double* Q, int nout, float* out,
@@ -502,15 +509,18 @@ int rks_basis_product_f32(int64_t n, const float* U, int64_t ldu, int nin, const
 /* out = U Q as the double-float restart forms it on the tensor cores: every
  * row of U is a 47-bit fixed-point integer at the row's own power-of-two
  * scale, every column of Q one at the column's scale; both are cut into seven
- * digits (a signed top digit and six of 7 bits), whose 34 leading digit-pair
- * products are accumulated in FP32 (exactly where it matters) and recombined
- * in double-float, then FP64.  Accuracy: about 2^-46 of the row's largest
- * |U[i, l]| times sum_l |Q[l, o]|.  U, out: device FP64 arrays with leading
- * dimension ldu >= n (U is read as ldu x nin values and rounded to
- * double-float pairs); Q: host FP64, nin x nout column-major,
- * 1 <= nin <= 192, 1 <= nout <= 64, and the digit
- * image of Q must fit in shared memory (else RKS_EINVAL).  Allocates its
- * scratch, runs on `stream` and synchronises it.  Returns RKS_OK,
+ * balanced 7-bit digits, whose 34 leading digit-pair products are accumulated
+ * in FP32 (exactly where it matters) and added up as 64-bit integers.
+ * Accuracy: about 2^-46 of the row's largest |U[i, l]| times sum_l |Q[l, o]|;
+ * zero rows give zeros, subnormal values of U count as zeros, and a row with
+ * an infinity or a NaN gives NaN.  U, out: device FP64 arrays with leading
+ * dimension ldu >= n; out may share memory with U: in the same rows (in place)
+ * at no cost, in other rows by way of a block of ldu nout doubles allocated
+ * for the call.  Q: host FP64, nin x nout column-major, 1 <= nin <= 192,
+ * 1 <= nout <= 64, and the digit image of Q must fit in shared memory (else
+ * RKS_EINVAL).  Scratch (the digit image, at most 0.3 MB) is kept per host
+ * thread and device until the thread ends; it is not valid after
+ * cudaDeviceReset.  Runs on `stream` and synchronises it.  Returns RKS_OK,
  * RKS_EINVAL, RKS_ENOMEM, RKS_ECUDA or RKS_ETIMEOUT. */
 int rks_basis_product_df(int64_t n, const double* U, int64_t ldu, int nin, const double* Q, int nout, double* out,
                          void* stream);
@@ -538,8 +548,8 @@ int rks_basis_product_df(int64_t n, const double* U, int64_t ldu, int nin, const
  * arithmetic, RHQR the same with Theta in place of Omega, RCHOLQR the
  * Euclidean QR of K.  Omega is the solver's
  * sparse-sign embedding for (n, d, zeta, seed).  The n-dimensional work runs
- * in double-float arithmetic on the device, the d x s and s x s work in FP64
- * on the host. */
+ * in double-float arithmetic on the device, the d x s and s x s work in FP64,
+ * on the host (RGS: on the device). */
 enum { RKS_QR_RGS = 0, RKS_QR_WHITEN = 1, RKS_QR_RCHOLQR = 2, RKS_QR_RHQR = 3 };
 #define RKS_SKETCH_QR_MAX_S 192
 
@@ -549,7 +559,8 @@ enum { RKS_QR_RGS = 0, RKS_QR_WHITEN = 1, RKS_QR_RCHOLQR = 2, RKS_QR_RHQR = 3 };
  * (measured by sketching the computed Q; for RGS the sketches the process
  * computed; for RHQR Omega' Q[s:, :], the sketched rows of Theta Q, whose
  * other rows are Q's first s rows).  RHQR needs n - s >= 2.  1 <= s <= min(RKS_SKETCH_QR_MAX_S, d, n), 1 <= zeta <= 16,
- * 2 zeta <= d <= 8192.  Work buffers (about 16 n s bytes) are allocated and
+ * 2 zeta <= d <= 8192.  Work buffers (about 16 n s bytes, 8 n s
+ * for RGS, and partial sums of up to 256 MB) are allocated and
  * freed by the call; it runs on `stream` and synchronises it.  Returns
  * RKS_OK, RKS_EINVAL, RKS_ENOMEM, RKS_ECUDA, RKS_EBREAKDOWN (a zero or
  * non-finite diagonal of R: K is rank deficient) or RKS_EDENSE (RCHOLQR: the

@@ -832,7 +832,7 @@ void tc_restart_df_blob(int nin, int nout, const double* Q, const int* pexp, std
 // FP64 in and out
 // 1.44 ms (with its conversion passes) -> 0.36 ms, bound by the digit split
 // (issue 60%, tensor pipe 20%); the whole rks_basis_product_df call 2.52 ->
-// 0.41 ms (no allocations, no double-float copies).  A 512-thread form with
+// 0.42 ms (no allocations, no double-float copies).  A 512-thread form with
 // four columns per thread and one store of 8 bytes per digit took 0.56 ms.
 template <class T>
 static void launch_df_t(int64_t n, const T* in, T* out, int64_t ldu, int nin, int nout, const void* blob,

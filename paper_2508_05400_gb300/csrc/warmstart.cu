@@ -7,15 +7,15 @@
 // invariant subspace).  The paper takes u_1 at random (Sec. 2.1); the random
 // start stays the fallback and the residual of the solve is the judge.
 //
-// Arithmetic: FP32 master weights (Adam), FP16 copies for the convolutions,
-// FP32 activations and accumulation, FP64 for the loss sums.  Activations
+// Arithmetic: FP32 master weights (Adam), copies rounded to FP16 (held as FP32)
+// for the convolutions, FP32 activations and accumulation, FP64 for the loss sums.  Activations
 // are channel-major (c x H x W) per level; every reduction is a fixed-order
 // fold of per-CTA partial sums, so a training step gives the same bits on
 // every run.
 //
 // Kernels:
-//   k_conv3x3       32 x 8 output pixels per CTA, 4 pixels x 8 outputs per
-//                   thread, optional ReLU on the output and an optional mask
+//   k_conv3x3       32 x 8 output pixels per CTA, 4 pixels x 8 (or 4)
+//                   outputs per thread, optional ReLU on the output and an optional mask
 //                   on it (the ReLU derivative of the backward pass); the
 //                   backward-data product is this kernel with the flipped,
 //                   transposed weights.  k_conv3x3_one: the one-channel layer.
