@@ -570,8 +570,10 @@ __device__ __forceinline__ void tile_write_part(const float2* acc, int d, double
 // loads of both rows are in flight at once (the products of a row are still
 // accumulated in entry order).
 // SK = false: the plain SpMV (Krylov-Schur with Euclidean CGS2), no sketch.
+// Two CTAs per SM as in k_df_spmv_ell (99 registers otherwise; rows of 1 to 13
+// entries, n = 7e5, d = 320, pairs: 43.2 us a launch, 35.4 us with two).
 template <class TA, class TU, bool SK>
-__global__ void __launch_bounds__(512) k_df_spmv_sketch(
+__global__ void __launch_bounds__(512, 2) k_df_spmv_sketch(
     const int32_t* __restrict__ rowptr, const int32_t* __restrict__ colind, const TA* __restrict__ vals,
     const TU* __restrict__ x, TU* __restrict__ w, const SketchTiles tv, double* __restrict__ part) {
   static_assert(kTileRows == 1024, "two rows per thread of a 512-thread CTA");
@@ -632,8 +634,11 @@ __global__ void __launch_bounds__(512) k_df_spmv_sketch(
 // products and sums are those of the CSR kernel, bit for bit.
 // WC > 0: rows of at most WC entries, all of a row's loads in one round
 // (5-point stencils: W = 5 fits WC = 6 without spilling at two CTAs per SM).
+// Two CTAs per SM (the grid is two per SM) must be asked for: with the gather's
+// four forms inlined the kernel takes 102 registers otherwise, one CTA per SM
+// (W = 12, n = 5e5, d = 320, pairs: 44.1 us a launch, 36.8 us with two).
 template <class TA, class TU, bool SK, int WC>
-__global__ void __launch_bounds__(512) k_df_spmv_ell(
+__global__ void __launch_bounds__(512, 2) k_df_spmv_ell(
     const int32_t* __restrict__ ecol, const TA* __restrict__ evals, int W,
     const TU* __restrict__ x, TU* __restrict__ w, const SketchTiles tv, double* __restrict__ part) {
   static_assert(kTileRows == 1024, "two rows per thread of a 512-thread CTA");
@@ -710,12 +715,17 @@ __global__ void __launch_bounds__(512) k_df_spmv_ell(
 
 // w = A x (+ partial sketches) with one warp per row inside each sketch tile
 // (rows of many entries): lanes take the row's entries with a stride of 32,
-// then a fixed xor tree adds the lanes' double-float sums.
+// then a fixed xor tree adds the lanes' double-float sums.  The bound of two
+// CTAs per SM leaves registers for the row loop's loads (40 otherwise, a third
+// CTA's room): rows of 27, n = 1e6: 156 us a launch, 123 us with the bound;
+// rows of 41 at random columns, n = 5e5, 80 columns: the first restart
+// 21.2 -> 16.5 ms.
 template <class TA, class TU, bool SK, int LPR>
-__global__ void __launch_bounds__(512) k_df_spmv_warp(const int32_t* __restrict__ rowptr,
-                                                      const int32_t* __restrict__ colind, const TA* __restrict__ vals,
-                                                      const TU* __restrict__ x, TU* __restrict__ w,
-                                                      const SketchTiles tv, double* __restrict__ part) {
+__global__ void __launch_bounds__(512, 2) k_df_spmv_warp(const int32_t* __restrict__ rowptr,
+                                                         const int32_t* __restrict__ colind,
+                                                         const TA* __restrict__ vals, const TU* __restrict__ x,
+                                                         TU* __restrict__ w, const SketchTiles tv,
+                                                         double* __restrict__ part) {
   extern __shared__ __align__(16) uint8_t smraw[];
   const int d = tv.d;
   const TileSmem lay = tile_smem_layout(d, tv.L, 0, tv.zeta);
