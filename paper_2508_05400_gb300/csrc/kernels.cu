@@ -792,10 +792,17 @@ void launch_rows_gemm(int64_t n, const double* A, int64_t lda, int a0, int nin, 
 int launch_resid(const Csr& A, const double* X, int64_t ld, int nreal, int npair, const int* slots, const int* col,
                  const int* colim, const double* lre, const double* lim, double* out, cudaStream_t st) {
   const int g = grid_for(A.n, 256, kResidCtas);
-  if (nreal > 0) {
-    dim3 grid((unsigned)g, (unsigned)((nreal + 3) / 4));
-    k_resid<false, 4><<<grid, 256, 0, st>>>(A.n, A.rowptr, A.colind, A.vals, X, ld, slots, nreal, col, colim, lre, lim,
+  // real columns four at a time, the last one to three by a kernel of that many
+  // (rows of 27, n = 5e5, one column: 257 us with the group of four, 190 us)
+  const int full = nreal & ~3;
+  if (full > 0) {
+    dim3 grid((unsigned)g, (unsigned)(full / 4));
+    k_resid<false, 4><<<grid, 256, 0, st>>>(A.n, A.rowptr, A.colind, A.vals, X, ld, slots, full, col, colim, lre, lim,
                                             out);
+  }
+  if (nreal > full) {
+    auto k = nreal - full == 1 ? k_resid<false, 1> : nreal - full == 2 ? k_resid<false, 2> : k_resid<false, 3>;
+    k<<<g, 256, 0, st>>>(A.n, A.rowptr, A.colind, A.vals, X, ld, slots + full, nreal - full, col, colim, lre, lim, out);
   }
   if (npair > 0) {
     dim3 grid((unsigned)g, (unsigned)npair);
