@@ -536,9 +536,13 @@ __global__ void k_rows_gemm(int64_t n, const double* A, int64_t lda, int a0, int
 // FMAs (the two-pass form spent 16 on the sums alone and stored A X); C = 4
 // real columns share the reads of A.  Rows of more than kLongRow entries are
 // taken by the whole warp (one thread on a row of 10^4 entries held the pass
-// up for 1.6 ms).  Measured, n = 1e6, 20 columns, 5 entries per row:
-// 0.79 -> 0.35 ms; 100 003 rows with one of 10^4 entries, 8 columns: 1.65 ->
-// 0.3 ms.
+// up for 1.6 ms), unless so many of the warp's 32 rows are long that a thread
+// each takes fewer FP64 operations: a row by the warp is its entries / 32
+// products and 5 additions, a thread each as many products as the longest row
+// has entries.  Measured, n = 1e6, 20 columns, 5 entries per row: 0.79 -> 0.35
+// ms; 100 003 rows with one of 10^4 entries, 8 columns: 1.65 -> 0.24 ms; all
+// rows of 101, n = 1e5, 8 columns: 0.55 ms in two passes, 0.72 with every row
+// by the warp, 0.24.
 constexpr int kLongRow = 64;
 template <bool CPLX, int C>
 __global__ void __launch_bounds__(256) k_resid(int64_t n, const int32_t* __restrict__ rowptr,
@@ -568,7 +572,12 @@ __global__ void __launch_bounds__(256) k_resid(int64_t n, const int32_t* __restr
   for (int64_t i0 = ((int64_t)blockIdx.x * 8 + warp) * 32; i0 < n; i0 += (int64_t)gridDim.x * 256) {
     const int64_t i = i0 + lane;
     const int p0 = i < n ? rowptr[i] : 0, p1 = i < n ? rowptr[i + 1] : 0;
-    const bool big = p1 - p0 > kLongRow;
+    bool big = p1 - p0 > kLongRow;
+    unsigned m = __ballot_sync(0xffffffffu, big);
+    if (m) {
+      const int longest = __reduce_max_sync(0xffffffffu, p1 - p0);
+      if (__popc(m) * (longest / 32 + 6) >= longest) { m = 0u; big = false; }
+    }
     double ax[V];
 #pragma unroll
     for (int v = 0; v < V; ++v) ax[v] = 0.0;
@@ -581,7 +590,7 @@ __global__ void __launch_bounds__(256) k_resid(int64_t n, const int32_t* __restr
         for (int v = 0; v < V; ++v) ax[v] = fma(a, xv[v][j], ax[v]);
       }
     }
-    for (unsigned m = __ballot_sync(0xffffffffu, big); m; m &= m - 1) {
+    for (; m; m &= m - 1) {
       const int src = __ffs(m) - 1;
       const int b0 = __shfl_sync(0xffffffffu, p0, src), b1 = __shfl_sync(0xffffffffu, p1, src);
       double part[V];
